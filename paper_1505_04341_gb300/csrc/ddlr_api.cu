@@ -171,7 +171,7 @@ struct ddlr_ctx {
     int L = 0;
     double *Yb = nullptr, *Qb = nullptr, *V = nullptr, *Z = nullptr, *Z2 = nullptr, *part = nullptr, *G = nullptr,
            *Linv = nullptr, *d = nullptr, *e = nullptr, *Hv = nullptr, *vals = nullptr, *eY = nullptr, *work = nullptr;
-    double *Vk = nullptr, *EV = nullptr, *vc = nullptr, *ev = nullptr, *uc = nullptr, *kp = nullptr, *hw = nullptr;
+    double *Vk = nullptr, *EV = nullptr, *ev = nullptr, *uc = nullptr, *kp = nullptr, *hw = nullptr;
     int *rank = nullptr;
   } rw;
   // Lanczos bidiagonalisation (lowrank_method 2), allocated at first use
@@ -181,7 +181,7 @@ struct ddlr_ctx {
     double *Vq = nullptr, *Uq = nullptr, *al = nullptr, *be = nullptr, *td = nullptr, *te = nullptr, *t = nullptr,
            *u = nullptr, *v = nullptr, *cpart = nullptr, *cvec = nullptr, *evals = nullptr, *eY = nullptr,
            *work = nullptr, *esum = nullptr, *etop = nullptr, *G = nullptr, *Vk = nullptr, *EV = nullptr,
-           *vc = nullptr, *ev = nullptr, *kp = nullptr, *hw = nullptr, *q0 = nullptr;
+           *kp = nullptr, *hw = nullptr, *q0 = nullptr;
   } lb;
   // restarted GMRES: Arnoldi basis V (n x (m+1)), Z = M^-1 V (n x m), H
   // ((m+1) x m), rotations, g, y, CGS partials, device scalars
@@ -232,7 +232,7 @@ struct ddlr_ctx {
            *qprev = nullptr, *nrm = nullptr, *ework = nullptr, *etop = nullptr, *evals = nullptr,
            *esum = nullptr, *eY = nullptr, *q0 = nullptr;
     float *Q32 = nullptr;             // FP32 copy of Q (persistent Lanczos)
-    double *V = nullptr, *EV = nullptr, *vc = nullptr, *ev = nullptr, *uc = nullptr, *kp = nullptr, *hw = nullptr;
+    double *V = nullptr, *EV = nullptr, *ev = nullptr, *uc = nullptr, *kp = nullptr, *hw = nullptr;
     int *rank = nullptr;
     LzState *st = nullptr;
     LzState *h_st = nullptr;          // pinned
@@ -943,7 +943,8 @@ void lanczos_step(ddlr_ctx *c, const LzBufs &L) {
   KL(c, "lanczos", c->stream, k_lz_advance, 1, 32, 0, L.st);
 }
 
-void hk_finalize(ddlr_ctx *c, int k, const double *kp, double *hw);
+void hk_build(ddlr_ctx *c, int k, const double *EV, double *kp, double *hw);
+void ddlr2_columns(ddlr_ctx *c, int k, const double *V, double *EV, double *ev, double *uc);
 ddlr_status lowrank_status(ddlr_ctx *c, const int *fl);
 
 // Lanczos with full reorthogonalisation and the convergence test of
@@ -955,7 +956,7 @@ ddlr_status lowrank_status(ddlr_ctx *c, const int *fl);
 // larger k, Sec. 3.4) instead of starting from q_1
 ddlr_status run_lanczos(ddlr_ctx *c, bool resume = false) {
   const Plan &P = c->P;
-  const int s = P.s, n = P.n, m0 = P.m, k = c->opt.rank_k;
+  const int s = P.s, n = P.n, k = c->opt.rank_k;
   int mmax = c->opt.lanczos_max > 0 ? c->opt.lanczos_max : 5 * k;
   mmax = std::min(mmax, s);
   mmax = std::max(mmax, k);
@@ -988,7 +989,6 @@ ddlr_status run_lanczos(ddlr_ctx *c, bool resume = false) {
       if (c->opt.variant == 2) {
         W.V = c->alloc<double>(size_t(s) * k);
         W.EV = c->alloc<double>(size_t(n) * k);
-        W.vc = c->alloc<double>(s);
         W.ev = c->alloc<double>(n);
         W.uc = c->alloc<double>(n);
         W.kp = c->alloc<double>(size_t(kRedGrid) * k * k);
@@ -1162,19 +1162,10 @@ ddlr_status run_lanczos(ddlr_ctx *c, bool resume = false) {
         read_dev(c, &c->theta, c->theta_d, sizeof(double));
       } else {
         // V_k = Q_m Y_k; U_k = A0^-1 E V_k; H_k = (I - U_k^T E V_k)^-1
-        double *V = W.V, *EV = W.EV, *vc = W.vc, *ev = W.ev, *uc = W.uc, *kp = W.kp, *hw = W.hw;
+        double *V = W.V, *EV = W.EV, *ev = W.ev, *uc = W.uc, *kp = W.kp, *hw = W.hw;
         KL(c, "ritz", c->stream, k_ritz_gemm<16>, nblk(s), kThreads, 0, s, mm, k, Q, (long long)s, eY, V);
-        const double a = c->opt.alpha;
-        for (int cc = 0; cc < k; cc++) {
-          KL(c, "ritz", c->stream, k_get_col, nblk(s), kThreads, 0, (long long)s, k, cc, V, vc);
-          KL(c, "e_vec", c->stream, k_e_vec<double>, nblk(n), kThreads, 0, m0, s, c->eh_rp, c->eh_ci,
-             c->eh64, 1.0 / a, a, vc, (const double *)nullptr, ev, (const int *)nullptr);
-          KL(c, "ritz", c->stream, k_set_col, nblk(n), kThreads, 0, (long long)n, k, cc, ev, EV);
-          a0_solve<double>(c, ev, uc, nullptr);
-          KL(c, "ritz", c->stream, k_set_col, nblk(n), kThreads, 0, (long long)n, k, cc, uc, c->U64);
-        }
-        KL(c, "ritz", c->stream, k_utv_partial, kRedGrid, 256, 0, (long long)n, k, c->U64, EV, kp);
-        hk_finalize(c, k, kp, hw);
+        ddlr2_columns(c, k, V, EV, ev, uc);
+        hk_build(c, k, EV, kp, hw);
         c->theta = 0.0;
       }
       int fl[4];
@@ -1237,15 +1228,51 @@ void batch_alloc(ddlr_ctx *c, int R);
 template <typename T>
 void a0_solve_mr(ddlr_ctx *c, const T *X, T *Z, int R, const int *gate);
 
-// H_k = (I - U_k^T E V_k)^-1 for DDLR-2 from the k_utv_partial partials:
+// H_k = (I - U_k^T E V_k)^-1 for DDLR-2 from the partial sums of its products:
 // Cholesky (an I - K that is not positive definite sets the NOT_SPD flag,
 // prop. spd-2) or, in the indefinite mode, Gauss-Jordan with partial pivoting
 // (a singular I - K sets the same flag, read as BREAKDOWN)
 void hk_finalize(ddlr_ctx *c, int k, const double *kp, double *hw) {
+  KL(c, "ritz", c->stream, k_hk_reduce, nblk((long long)k * k * 32), kThreads, 0, kRedGrid, k * k, kp, hw);
   if (c->opt.indefinite)
-    KL(c, "ritz", c->stream, k_hk_finalize_gj, 1, 32, 0, kRedGrid, k, kp, hw, c->Hk64, c->dflag + 1);
+    KL(c, "ritz", c->stream, k_hk_finalize_gj, 1, kGjThreads, 0, k, hw, c->Hk64, c->dflag + 1);
   else
-    KL(c, "ritz", c->stream, k_hk_finalize, 1, 32, 0, kRedGrid, k, kp, hw, c->Hk64, c->dflag + 1);
+    KL(c, "ritz", c->stream, k_hk_finalize, 1, kHkThreads, 0, k, hw, c->Hk64, c->dflag + 1);
+}
+
+// H_k from U_k and E V_k (both n x k row-major)
+void hk_build(ddlr_ctx *c, int k, const double *EV, double *kp, double *hw) {
+  const long long n = c->P.n;
+  if (k <= kRandMaxL)
+    KL(c, "ritz", c->stream, k_gram_partial, kRedGrid, kGramNT, 0, n, k, c->U64, EV, kp);
+  else
+    KL(c, "ritz", c->stream, k_utv_partial, kRedGrid, 256, 0, n, k, c->U64, EV, kp);
+  hk_finalize(c, k, kp, hw);
+}
+
+// E V_k and U_k = A0^-1 E V_k (V s x k, the others n x k, all row-major), all
+// columns in one batched solve: U_k's layout is that of a block of k
+// right-hand sides.  L D L^T factors and the Chebyshev solve with C_a (its work
+// blocks belong to a batch), and ranks beyond a batch, go column by column.
+// 64^3, k = 32, FP64: 2.9 ms column by column (160 launches), 0.4 ms batched.
+void ddlr2_columns(ddlr_ctx *c, int k, const double *V, double *EV, double *ev, double *uc) {
+  const Plan &P = c->P;
+  const int n = P.n, m = P.m, s = P.s;
+  const double a = c->opt.alpha;
+  KL(c, "e_vec", c->stream, k_e_block, nblk((long long)n * k), kThreads, 0, m, s, k, c->eh_rp, c->eh_ci, c->eh64,
+     1.0 / a, a, V, EV);
+  if (k >= 2 && k <= kMaxR && c->opt.factor < 2 && c->opt.c_solver != 1) {
+    const int per = c->bt.chunk_per;
+    if (per == 0) c->bt.chunk_per = std::max(1, 256 / k);
+    a0_solve_mr<double>(c, EV, c->U64, k, nullptr);
+    c->bt.chunk_per = per;
+    return;
+  }
+  for (int cc = 0; cc < k; cc++) {
+    KL(c, "ritz", c->stream, k_get_col, nblk(n), kThreads, 0, (long long)n, k, cc, EV, ev);
+    a0_solve<double>(c, ev, uc, nullptr);
+    KL(c, "ritz", c->stream, k_set_col, nblk(n), kThreads, 0, (long long)n, k, cc, uc, c->U64);
+  }
 }
 
 // status of a finished low-rank build from the device flags (timeout, NaN,
@@ -1306,7 +1333,6 @@ ddlr_status run_lbd(ddlr_ctx *c) {
     B.G = c->alloc<double>(size_t(mmax) * k);
     B.Vk = c->alloc<double>(size_t(s) * k);
     B.EV = c->alloc<double>(size_t(n) * k);
-    B.vc = c->alloc<double>(s); B.ev = c->alloc<double>(n);
     B.kp = c->alloc<double>(size_t(kRedGrid) * k * k);
     B.hw = c->alloc<double>(size_t(k) * k + k);
     // start vector: the Lanczos one (SplitMix64 stream seed over the
@@ -1398,14 +1424,9 @@ ddlr_status run_lbd(ddlr_ctx *c) {
   KL(c, "ritz", c->stream, k_ritz_gemm<16>, nblk(n), kThreads, 0, n, mm, k, B.Uq, (long long)n, B.G, c->U64);
   // H_k = (I - U_k^T E V_k)^-1
   ck(cudaMemsetAsync(c->dflag, 0, 4 * sizeof(int), c->stream), "memset");
-  for (int cc = 0; cc < k; cc++) {
-    KL(c, "ritz", c->stream, k_get_col, nblk(s), kThreads, 0, (long long)s, k, cc, B.Vk, B.vc);
-    KL(c, "e_vec", c->stream, k_e_vec<double>, nblk(n), kThreads, 0, m0, s, c->eh_rp, c->eh_ci, c->eh64, 1.0 / a, a,
-       B.vc, (const double *)nullptr, B.ev, (const int *)nullptr);
-    KL(c, "ritz", c->stream, k_set_col, nblk(n), kThreads, 0, (long long)n, k, cc, B.ev, B.EV);
-  }
-  KL(c, "ritz", c->stream, k_utv_partial, kRedGrid, 256, 0, (long long)n, k, c->U64, B.EV, B.kp);
-  hk_finalize(c, k, B.kp, B.hw);
+  KL(c, "e_vec", c->stream, k_e_block, nblk((long long)n * k), kThreads, 0, m0, s, k, c->eh_rp, c->eh_ci, c->eh64,
+     1.0 / a, a, B.Vk, B.EV);
+  hk_build(c, k, B.EV, B.kp, B.hw);
   c->theta = 0.0;
   int fl[4];
   read_dev(c, fl, c->dflag, sizeof(fl));
@@ -1444,7 +1465,6 @@ ddlr_status run_randomized(ddlr_ctx *c) {
     if (c->opt.variant == 2) {
       R.Vk = c->alloc<double>(size_t(s) * k);
       R.EV = c->alloc<double>(size_t(n) * k);
-      R.vc = c->alloc<double>(s);
       R.ev = c->alloc<double>(n);
       R.uc = c->alloc<double>(n);
       R.kp = c->alloc<double>(size_t(kRedGrid) * k * k);
@@ -1514,16 +1534,8 @@ ddlr_status run_randomized(ddlr_ctx *c) {
   } else {
     // V_k = Q Y_k; U_k = A0^-1 E V_k; H_k = (I - U_k^T E V_k)^-1
     KL(c, "ritz", c->stream, k_rm_gemm, nblk(s), kThreads, 0, (long long)s, L, k, R.Yb, R.eY, R.Vk);
-    for (int cc = 0; cc < k; cc++) {
-      KL(c, "ritz", c->stream, k_get_col, nblk(s), kThreads, 0, (long long)s, k, cc, R.Vk, R.vc);
-      KL(c, "e_vec", c->stream, k_e_vec<double>, nblk(n), kThreads, 0, m, s, c->eh_rp, c->eh_ci, c->eh64, 1.0 / a,
-         a, R.vc, (const double *)nullptr, R.ev, (const int *)nullptr);
-      KL(c, "ritz", c->stream, k_set_col, nblk(n), kThreads, 0, (long long)n, k, cc, R.ev, R.EV);
-      a0_solve<double>(c, R.ev, R.uc, nullptr);
-      KL(c, "ritz", c->stream, k_set_col, nblk(n), kThreads, 0, (long long)n, k, cc, R.uc, c->U64);
-    }
-    KL(c, "ritz", c->stream, k_utv_partial, kRedGrid, 256, 0, (long long)n, k, c->U64, R.EV, R.kp);
-    hk_finalize(c, k, R.kp, R.hw);
+    ddlr2_columns(c, k, R.Vk, R.EV, R.ev, R.uc);
+    hk_build(c, k, R.EV, R.kp, R.hw);
     c->theta = 0.0;
   }
   read_dev(c, fl, c->dflag, sizeof(fl));

@@ -91,43 +91,79 @@ __global__ void k_gm_resid(long long n, const double *b, const double *q, double
   if (i < n) r[i] = b[i] - q[i];
 }
 
-// Indefinite mode, DDLR-2: H_k = (I - K)^-1 with K from the k_utv_partial
-// partials, symmetrised as for the Cholesky path, inverted by Gauss-Jordan
-// elimination with partial pivoting (one thread; work = k x k).  A pivot of
-// magnitude <= 1e-14 times the largest entry sets *singular.  Hk row-major.
-__global__ void k_hk_finalize_gj(int G, int k, const double *partials, double *work, double *Hk, int *singular) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double *M = work;
-  double amax = 0.0;
-  for (int a = 0; a < k; a++)
-    for (int b = 0; b < k; b++) {
-      double s1 = 0, s2 = 0;
-      for (int g = 0; g < G; g++) {
-        s1 += partials[(long long)g * k * k + a * k + b];
-        s2 += partials[(long long)g * k * k + b * k + a];
-      }
-      M[a * k + b] = (a == b ? 1.0 : 0.0) - 0.5 * (s1 + s2);
-      amax = fmax(amax, fabs(M[a * k + b]));
-      Hk[a * k + b] = a == b ? 1.0 : 0.0;
-    }
+// Indefinite mode, DDLR-2: H_k = (I - K)^-1 with K the summed products
+// (k_hk_reduce), symmetrised as for the Cholesky path, inverted by Gauss-Jordan
+// elimination with partial pivoting (the first of equal magnitudes).  A pivot
+// of magnitude <= 1e-14 times the largest entry sets *singular.  Hk row-major.
+// One CTA: the row operations of a step run over all threads (one thread's
+// serial elimination took about as long as the Cholesky form, 20 ms at
+// k = 32); every entry sees the operations of the serial elimination.
+constexpr int kGjThreads = 512;
+__global__ void __launch_bounds__(kGjThreads) k_hk_finalize_gj(int k, double *M, double *Hk, int *singular) {
+  __shared__ double fs[256], s_amax[kGjThreads / 32];
+  __shared__ int s_piv;
+  __shared__ double s_pmax;
+  const int tid = threadIdx.x, wi = tid >> 5, l = tid & 31;
+  double am = 0.0;
+  for (int o = tid; o < k * k; o += kGjThreads) {
+    const int a = o / k, b = o - a * k;
+    Hk[o] = a == b ? 1.0 : 0.0;
+    if (b > a) continue;
+    const double v = (a == b ? 1.0 : 0.0) - 0.5 * (M[a * k + b] + M[b * k + a]);
+    M[a * k + b] = v;
+    M[b * k + a] = v;
+    am = fmax(am, fabs(v));
+  }
+  for (int d = 16; d > 0; d >>= 1) am = fmax(am, __shfl_xor_sync(0xffffffffu, am, d));
+  if (l == 0) s_amax[wi] = am;
+  __syncthreads();
+  am = 0.0;
+  for (int w = 0; w < kGjThreads / 32; w++) am = fmax(am, s_amax[w]);
   for (int j = 0; j < k; j++) {
-    int piv = j;
-    for (int r = j + 1; r < k; r++)
-      if (fabs(M[r * k + j]) > fabs(M[piv * k + j])) piv = r;
-    if (!(fabs(M[piv * k + j]) > 1e-14 * amax)) { *singular = 1; return; }
-    if (piv != j)
-      for (int c = 0; c < k; c++) {
-        double t = M[j * k + c]; M[j * k + c] = M[piv * k + c]; M[piv * k + c] = t;
-        t = Hk[j * k + c]; Hk[j * k + c] = Hk[piv * k + c]; Hk[piv * k + c] = t;
+    if (wi == 0) {
+      double best = -1.0;
+      int at = k;
+      for (int r = j + l; r < k; r += 32) {
+        const double v = fabs(M[r * k + j]);
+        if (v > best) { best = v; at = r; }
       }
-    const double d = M[j * k + j];
-    for (int c = 0; c < k; c++) { M[j * k + c] /= d; Hk[j * k + c] /= d; }
-    for (int r = 0; r < k; r++) {
-      if (r == j) continue;
-      const double f = M[r * k + j];
-      if (f == 0.0) continue;
-      for (int c = 0; c < k; c++) { M[r * k + c] -= f * M[j * k + c]; Hk[r * k + c] -= f * Hk[j * k + c]; }
+      for (int d = 16; d > 0; d >>= 1) {
+        const double ob = __shfl_xor_sync(0xffffffffu, best, d);
+        const int oa = __shfl_xor_sync(0xffffffffu, at, d);
+        if (ob > best || (ob == best && oa < at)) { best = ob; at = oa; }
+      }
+      if (l == 0) { s_piv = at; s_pmax = best; }
     }
+    __syncthreads();
+    const int piv = s_piv;
+    if (!(s_pmax > 1e-14 * am)) {
+      if (tid == 0) *singular = 1;
+      return;
+    }
+    const double d = M[piv * k + j];
+    __syncthreads();
+    // rows j and piv change places, row j divided by the pivot
+    for (int c = tid; c < k; c += kGjThreads) {
+      const double mp = M[piv * k + c], hp = Hk[piv * k + c];
+      if (piv != j) {
+        M[piv * k + c] = M[j * k + c];
+        Hk[piv * k + c] = Hk[j * k + c];
+      }
+      M[j * k + c] = mp / d;
+      Hk[j * k + c] = hp / d;
+    }
+    __syncthreads();
+    for (int r = tid; r < k; r += kGjThreads) fs[r] = M[r * k + j];
+    __syncthreads();
+    for (int r = wi; r < k; r += kGjThreads / 32) {
+      const double f = fs[r];
+      if (r == j || f == 0.0) continue;
+      for (int c = l; c < k; c += 32) {
+        M[r * k + c] -= f * M[j * k + c];
+        Hk[r * k + c] -= f * Hk[j * k + c];
+      }
+    }
+    __syncthreads();
   }
 }
 

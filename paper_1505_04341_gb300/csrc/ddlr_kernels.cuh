@@ -1893,7 +1893,8 @@ __global__ void k_set_col(long long n, int k, int c, const double *v, double *M)
   if (r < n) M[r * k + c] = v[r];
 }
 
-// partials of K = U^T EV over row chunks (U, EV row-major n x k)
+// partials of K = U^T EV over row chunks (U, EV row-major n x k): any k; up to
+// kRandMaxL columns take the tiled k_gram_partial instead
 __global__ void k_utv_partial(long long n, int k, const double *U,
                               const double *EV, double *partials) {
   const long long chunk = (n + gridDim.x - 1) / gridDim.x;
@@ -1906,47 +1907,87 @@ __global__ void k_utv_partial(long long n, int k, const double *U,
   }
 }
 
-// H_k = (I - (K + K^T)/2)^-1 by Cholesky (lemma 1 / prop. spd-2); failure of
-// the Cholesky flags NOT_SPD.  One thread; k is small.
-__global__ void k_hk_finalize(int G, int k, const double *partials, double *work,
-                              double *Hk, int *notspd) {
-  if (threadIdx.x != 0) return;
-  double *M = work;            // k x k
-  double *e = work + k * k;    // k
-  for (int a = 0; a < k; a++)
-    for (int b = 0; b < k; b++) {
-      double s1 = 0, s2 = 0;
-      for (int g = 0; g < G; g++) {
-        s1 += partials[(long long)g * k * k + a * k + b];
-        s2 += partials[(long long)g * k * k + b * k + a];
-      }
-      M[a * k + b] = (a == b ? 1.0 : 0.0) - 0.5 * (s1 + s2);
-    }
-  for (int j = 0; j < k; j++) {
-    double dj = M[j * k + j];
-    for (int t = 0; t < j; t++) dj -= M[j * k + t] * M[j * k + t];
-    if (!(dj > 0.0)) { *notspd = 1; return; }
-    dj = sqrt(dj);
-    M[j * k + j] = dj;
-    for (int i = j + 1; i < k; i++) {
-      double sm = M[i * k + j];
-      for (int t = 0; t < j; t++) sm -= M[i * k + t] * M[j * k + t];
-      M[i * k + j] = sm / dj;
-    }
+// K[o] = sum_g partials[g][o], o < np (warp per entry: lanes take every 32nd
+// partial, then a tree).  The k x k sums of DDLR-2 are k^2 G adds of ~67 cycles
+// latency each: one thread took 10 ms for them at k = 32, the grid takes 5 us.
+__global__ void k_hk_reduce(int G, int np, const double *partials, double *K) {
+  const int o = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, l = threadIdx.x & 31;
+  if (o >= np) return;
+  double v = 0;
+  for (int g = l; g < G; g += 32) v += partials[(long long)g * np + o];
+  for (int d = 16; d > 0; d >>= 1) v += __shfl_down_sync(0xffffffffu, v, d);
+  if (l == 0) K[o] = v;
+}
+
+// H_k = (I - (K + K^T)/2)^-1 by Cholesky (lemma 1 / prop. spd-2); a pivot that
+// is not positive flags NOT_SPD.  One CTA of kHkThreads threads: right-looking
+// factorisation (the trailing update over all warps, so the chain is k steps
+// of one FMA and one reciprocal square root), then a warp per column of the
+// inverse, its entries in the lanes' registers (rank_k is at most 256).  The
+// matrix sits in shared memory up to k = kHkSmem, beyond that in K itself.
+// 64^3, k = 32: 28 ms with one thread, 0.04 ms now (with the sums above).
+constexpr int kHkThreads = 512, kHkSmem = 64, kHkMaxK = 256;
+__global__ void __launch_bounds__(kHkThreads) k_hk_finalize(int k, double *K, double *Hk, int *notspd) {
+  __shared__ double sm[kHkSmem * (kHkSmem + 1)];
+  __shared__ double rd[kHkMaxK];         // 1 / L_jj
+  const int tid = threadIdx.x, wi = tid >> 5, l = tid & 31;
+  constexpr int NW = kHkThreads / 32;
+  const bool in_sm = k <= kHkSmem;
+  double *M = in_sm ? sm : K;
+  const int ld = in_sm ? k + 1 : k;
+  for (int o = tid; o < k * k; o += kHkThreads) {   // pairs (a, b), b <= a, are disjoint: K may be M
+    const int a = o / k, b = o - a * k;
+    if (b > a) continue;
+    const double v = (a == b ? 1.0 : 0.0) - 0.5 * (K[a * k + b] + K[b * k + a]);
+    M[a * ld + b] = v;
   }
-  for (int c = 0; c < k; c++) {
-    for (int r = 0; r < k; r++) e[r] = (r == c) ? 1.0 : 0.0;
-    for (int i = 0; i < k; i++) {
-      double sm = e[i];
-      for (int t = 0; t < i; t++) sm -= M[i * k + t] * e[t];
-      e[i] = sm / M[i * k + i];
+  __syncthreads();
+  for (int j = 0; j < k; j++) {
+    const double dj = M[j * ld + j];
+    if (!(dj > 0.0)) {                   // the same value in every thread
+      if (tid == 0) *notspd = 1;
+      return;
     }
-    for (int i = k - 1; i >= 0; i--) {
-      double sm = e[i];
-      for (int t = i + 1; t < k; t++) sm -= M[t * k + i] * e[t];
-      e[i] = sm / M[i * k + i];
+    const double r = 1.0 / sqrt(dj);
+    if (tid == 0) rd[j] = r;
+    for (int i = j + 1 + tid; i < k; i += kHkThreads) M[i * ld + j] *= r;
+    __syncthreads();
+    for (int i = j + 1 + wi; i < k; i += NW) {
+      const double f = M[i * ld + j];
+      for (int c = j + 1 + l; c <= i; c += 32) M[i * ld + c] -= f * M[c * ld + j];
     }
-    for (int r = 0; r < k; r++) Hk[r * k + c] = e[r];
+    __syncthreads();
+  }
+  constexpr int Q = kHkMaxK / 32;
+  for (int c = wi; c < k; c += NW) {
+    double e[Q];
+#pragma unroll
+    for (int q = 0; q < Q; q++) e[q] = (l + 32 * q == c) ? 1.0 : 0.0;
+#pragma unroll
+    for (int q = 0; q < Q; q++)
+      for (int i = 32 * q; i < min(k, 32 * q + 32); i++) {          // L y = e_c
+        const double y = __shfl_sync(0xffffffffu, e[q], i & 31) * rd[i];
+#pragma unroll
+        for (int p = q; p < Q; p++) {
+          const int r = l + 32 * p;
+          if (r == i) e[p] = y;
+          else if (r > i && r < k) e[p] -= M[r * ld + i] * y;
+        }
+      }
+#pragma unroll
+    for (int q = Q - 1; q >= 0; q--)
+      for (int i = min(k, 32 * q + 32) - 1; i >= 32 * q; i--) {     // L^T x = y
+        const double x = __shfl_sync(0xffffffffu, e[q], i & 31) * rd[i];
+#pragma unroll
+        for (int p = 0; p <= q; p++) {
+          const int r = l + 32 * p;
+          if (r == i) e[p] = x;
+          else if (r < i) e[p] -= M[i * ld + r] * x;
+        }
+      }
+#pragma unroll
+    for (int q = 0; q < Q; q++)
+      if (l + 32 * q < k) Hk[(l + 32 * q) * k + c] = e[q];
   }
 }
 

@@ -34,7 +34,7 @@ __global__ void k_e_block(int m, int s, int L, const int *eh_rp, const int *eh_c
                           double a, const double *W, double *V) {
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (long long)(m + s) * L) return;
-  const int r = int(unsigned(e) / unsigned(L)), c = int(e - (long long)r * L);
+  const int r = e < 0xffffffffLL ? int(unsigned(e) / unsigned(L)) : int(e / L), c = int(e - (long long)r * L);
   double v;
   if (r < m) {
     double acc = 0;
