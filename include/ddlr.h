@@ -133,7 +133,7 @@ typedef struct {
                               vector always takes two.                        */
   double wait_limit_s;     /* limit of every bounded device wait, seconds (grid
                               barriers of the persistent kernels, ready flags of
-                              the synchronisation-free solve; the TMA solve waits
+                              the synchronisation-free solve; the deep solve waits
                               at least 1 s for its copies): when it runs out the
                               kernel records it and returns, and the call gives
                               DDLR_ERR_TIMEOUT.  Default 2; (0, 3600].          */

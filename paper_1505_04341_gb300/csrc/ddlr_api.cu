@@ -26,6 +26,7 @@
 #include "ddlr_gmres.cuh"
 #include "ddlr_ldl.cuh"
 #include "ddlr_internal.h"
+#include "ddlr_deep.cuh"
 #include "ddlr_kernels.cuh"
 #include "ddlr_plan.h"
 #include "ddlr_persist.cuh"
@@ -141,12 +142,8 @@ struct ddlr_ctx {
   // the unscaled form
   double *lx64 = nullptr;
   float *lx32 = nullptr;
-  double *dinvs64 = nullptr;  // inverse diagonal in slice layout (TMA solve)
-  float *dinvs32 = nullptr;
-  int *row_slot = nullptr;
-  TmaCfg tma64{}, tma32{};
-  bool use_tma64 = false, use_tma32 = false;
   bool use_sf64 = false, use_sf32 = false;   // synchronisation-free interior solve
+  bool deep_int = true;       // interior blocks may take the pipeline of ddlr_deep.cuh
   bool uvec = true;           // vector-load U_k products (DDLR_UVEC=0: scalar kernels)
   unsigned *udone = nullptr;  // arrival counter of the fused U^T x reduction (0 between launches)
   unsigned *pdone = nullptr;  // arrival counter of the fused per-phase PCG reductions
@@ -156,6 +153,23 @@ struct ddlr_ctx {
   int *blk_row0 = nullptr;
   int *chunks = nullptr;
   int4 *lv_desc = nullptr;    // level-order row descriptors (shallow factors)
+  // deep factors (ddlr_deep.cuh): the interior blocks, a CTA each, and C_a
+  // (D_a) by one cluster; ctas == 0: not served (the interior blocks then take
+  // k_sptrsv_blocks, C_a a launch per level)
+  struct Deep {
+    DeepGeo g{};
+    int nslices = 0;
+    unsigned char *pl = nullptr, *pu = nullptr;
+  } deep64[2], deep32[2];     // [0] interior blocks, [1] C_a
+  // the same for factors with few rows per level (exact ones): panels
+  struct Panel {
+    PanelGeo g{};              // nblk == 0: not served
+    int npan = 0;
+    long long nent = 0;
+    const int *src = nullptr;  // entry -> slot in the L (below lsplit: L^T) values, -1 padding
+    const unsigned char *dir = nullptr;   // per row of kPanelNT entries: 1 = L^T
+    void *ent = nullptr, *inv = nullptr;
+  } pan64[2], pan32[2];
   // Chebyshev solve with C_a (c_solver 1): C_a as CSR over the interface
   // rows, the coefficient table (see ddlr_cheb.cuh), single-RHS workspaces
   int *cc_rp = nullptr, *cc_ci = nullptr, *cc_src = nullptr, *cc_diag = nullptr, *cz_rank = nullptr;
@@ -386,43 +400,14 @@ size_t sf_smem_bytes(const Plan &P) {
   return ((size_t(P.tma_zs) * sizeof(T) + 15) & ~size_t(15)) + size_t(P.tma_zs) * 4;
 }
 
-// geometry of the TMA-pipelined interior solve for element type T: the ring
-// takes what the shared memory of one SM leaves for each co-resident CTA
-// (enough CTAs per SM to hold every interior block in one wave, up to 4),
-// capped at one block's total staged bytes; false if a stage does not fit
-template <typename T>
-bool tma_config(const Plan &P, TmaCfg &cfg) {
-  int dev = 0, sms = 0, per_sm = 0, optin = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (P.tma_zs <= 0 || sms <= 0) return false;
-  const int cps = std::max(1, std::min(4, (P.p + sms - 1) / sms));
-  // the kernel's static shared memory (its abort word) comes out of the same
-  // per-block limit as the dynamic part
-  constexpr long long kStatic = 128;
-  const long long budget = std::min<long long>(optin, per_sm / cps - 1024) - kStatic;
-  cfg = TmaCfg{P.tma_zs, P.tma_nl, P.tma_ns, 0};
-  const long long fixed = (long long)tma_smem_bytes<T>(cfg);
-  const long long stage_max = (long long)P.tma_e * (long long)(sizeof(T) + 4) +
-                              (long long)P.tma_s * 32 * (long long)sizeof(T);
-  const long long block_total = P.tma_blk_e * (long long)(sizeof(T) + 4) +
-                                P.tma_blk_s * 32 * (long long)sizeof(T);
-  long long ring = std::min(budget - fixed, block_total + stage_max);
-  ring &= ~127LL;
-  if (ring < stage_max || ring <= 0) return false;
-  cfg.ring_bytes = int(ring);
-  return true;
-}
-
 template <typename T> struct Prec;
 template <> struct Prec<double> {
+  static ddlr_ctx::Deep *deep(ddlr_ctx *c) { return c->deep64; }
+  static ddlr_ctx::Panel *pan(ddlr_ctx *c) { return c->pan64; }
   static const double *l(ddlr_ctx *c) { return c->l64; }
   static const double *lx(ddlr_ctx *c) { return c->lx64; }
   static const double *u(ddlr_ctx *c) { return c->u64; }
   static const double *dinv(ddlr_ctx *c) { return c->dinv64; }
-  static const double *dinvs(ddlr_ctx *c) { return c->dinvs64; }
   static const double *eh(ddlr_ctx *c) { return c->eh64; }
   static const double *eht(ddlr_ctx *c) { return c->eht64; }
   static double *w(ddlr_ctx *c, int i) { return c->w64[i]; }
@@ -432,11 +417,12 @@ template <> struct Prec<double> {
   static const double *Hk(ddlr_ctx *c) { return c->Hk64; }
 };
 template <> struct Prec<float> {
+  static ddlr_ctx::Deep *deep(ddlr_ctx *c) { return c->deep32; }
+  static ddlr_ctx::Panel *pan(ddlr_ctx *c) { return c->pan32; }
   static const float *l(ddlr_ctx *c) { return c->l32; }
   static const float *lx(ddlr_ctx *c) { return c->lx32; }
   static const float *u(ddlr_ctx *c) { return c->u32; }
   static const float *dinv(ddlr_ctx *c) { return c->dinv32; }
-  static const float *dinvs(ddlr_ctx *c) { return c->dinvs32; }
   static const float *eh(ddlr_ctx *c) { return c->eh32; }
   static const float *eht(ddlr_ctx *c) { return c->eht32; }
   static float *w(ddlr_ctx *c, int i) { return c->w32[i]; }
@@ -481,6 +467,51 @@ void chunk_sweeps(ddlr_ctx *c, cudaStream_t st, const std::vector<int> &ptr, con
   for (int L = 0; L + 1 < nL; L++) launch(L, 0);
   if (nL > 0) launch(nL - 1, 2);
   for (int L = nL - 2; L >= 0; L--) launch(L, 1);
+}
+
+// launch configuration of the deep solve: one cluster of g.ctas CTAs, or (1)
+// one CTA per block
+struct DeepLaunch {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at{};
+  DeepLaunch(const DeepGeo &g, size_t smem, cudaStream_t st) {
+    cfg.gridDim = dim3(g.nparts);
+    cfg.blockDim = dim3(kDeepThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = g.ctas;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = g.ctas > 1 ? 1 : 0;
+  }
+};
+template <typename T>
+void deep_solve(ddlr_ctx *c, cudaStream_t st, const char *fam, const ddlr_ctx::Deep &D, const T *x, T *z,
+                const int *gate) {
+  ddlr_ctx::Scope sc(c, fam, st);
+  DeepLaunch L(D.g, deep_smem_bytes<T>(D.g), st);
+  ck(cudaLaunchKernelEx(&L.cfg, k_deep_solve<T>, D.g, (const unsigned char *)D.pl, (const unsigned char *)D.pu, x, z,
+                        gate, c->dflag + 3, std::max(c->wait_ns, kDeepMinWaitNs)), "cudaLaunchKernelEx");
+}
+
+template <typename T>
+void panel_solve(ddlr_ctx *c, cudaStream_t st, const char *fam, const ddlr_ctx::Panel &D, const T *x, T *z,
+                 const int *gate) {
+  KL(c, fam, st, k_panel_solve<T>, D.g.nblk, kPanelNT, panel_smem_bytes<T>(D.g.rcap), D.g, (const T *)D.ent,
+     (const T *)D.inv, x, z, gate);
+}
+
+// z_C = C_a^-1 x_C (or D_a^-1) alone: in panels when its levels are narrow, by
+// one cluster when the block is deep and its solution fits the cluster's shared
+// memory, else level by level
+template <typename T>
+void c_block_solve(ddlr_ctx *c, cudaStream_t st, const char *fam, const T *lv, const T *uv, const T *di, const T *x,
+                   T *z, const int *gate) {
+  const ddlr_ctx::Deep &D = Prec<T>::deep(c)[1];
+  if (Prec<T>::pan(c)[1].g.nblk > 0) panel_solve<T>(c, st, fam, Prec<T>::pan(c)[1], x, z, gate);
+  else if (D.g.ctas > 0) deep_solve<T>(c, st, fam, D, x, z, gate);
+  else chunk_sweeps<T>(c, st, c->P.ch_c_ptr, fam, lv, uv, di, x, z, gate);
 }
 
 // the same sweeps over the level-order descriptor list (all blocks); x may be
@@ -607,21 +638,20 @@ void a0_solve(ddlr_ctx *c, const T *x, T *z, const int *gate) {
   ck(cudaEventRecord(c->ev_fork, c->stream), "event");
   ck(cudaStreamWaitEvent(c->stream2, c->ev_fork, 0), "wait");
   if (P.p > 0) {
-    const bool use = sizeof(T) == 8 ? c->use_tma64 : c->use_tma32;
-    const TmaCfg &cfg = sizeof(T) == 8 ? c->tma64 : c->tma32;
     if (sizeof(T) == 8 ? c->use_sf64 : c->use_sf32) {
       KL(c, "sptrsv_blocks", c->stream, (k_sptrsv_blocks_sf<T, 256, 4>), P.p, 256, sf_smem_bytes<T>(P),
          c->blk_row0, RowSpan{c->l_span, c->u_span}, c->S.l_col, lv, c->S.u_col, uv, di, x, z, gate,
          c->dflag + 3, c->wait_ns);
-    } else if (use) {
-      KL(c, "sptrsv_blocks", c->stream, (k_sptrsv_blocks_tma<T, 256>), P.p, 256, tma_smem_bytes<T>(cfg),
-         c->S, lv, uv, Prec<T>::dinvs(c), x, z, gate, cfg, c->dflag + 3, std::max(c->wait_ns, kTmaMinWaitNs));
+    } else if (Prec<T>::pan(c)[0].g.nblk > 0) {
+      panel_solve<T>(c, c->stream, "sptrsv_blocks", Prec<T>::pan(c)[0], x, z, gate);
+    } else if (Prec<T>::deep(c)[0].g.ctas > 0) {
+      deep_solve<T>(c, c->stream, "sptrsv_blocks", Prec<T>::deep(c)[0], x, z, gate);
     } else {
       KL(c, "sptrsv_blocks", c->stream, (k_sptrsv_blocks<T, 256>), P.p, 256, 0,
          c->S, lv, uv, di, x, z, gate);
     }
   }
-  chunk_sweeps<T>(c, c->stream2, P.ch_c_ptr, "sptrsv_c", lv, uv, di, x, z, gate);
+  c_block_solve<T>(c, c->stream2, "sptrsv_c", lv, uv, di, x, z, gate);
   if (cheb) cheb_tail<T>(c, c->stream2, x, z, 1, gate);
   else if (c->opt.c_solver == 2) mr_apply_c<T>(c, c->stream2, x, z, 1, gate);
   ck(cudaEventRecord(c->ev_join, c->stream2), "event");
@@ -1196,6 +1226,318 @@ void lowrank_to_low_precision(ddlr_ctx *c) {
   KL(c, "setup", c->stream, (k_cast<float, double>), nblk((long long)k * k), kThreads, 0, (long long)k * k, c->Hk64, c->Hk32, (const int *)nullptr);
 }
 
+// Whether the blocks (which = 0 interior, 1 C_a) have deep factors, and whether
+// their levels are narrow: below kNarrowRows rows on average a panel of 32 rows
+// spans several levels, and the panel's two dot products take less than its
+// levels' steps one by one (0.35 us each in k_deep_solve, 0.75 us a panel).
+constexpr int kNarrowRows = 8;
+bool deep_blocks(const ddlr_ctx *c, int which, bool &narrow) {
+  const Plan &P = c->P;
+  const char *env = getenv("DDLR_DEEP");
+  if ((env && env[0] == '0') || c->opt.factor >= 2) return false;
+  if (std::max(P.levels_interior, P.levels_c) <= kShallowLevels) return false;
+  const int NLc = P.blk_lvl0[P.p + 1] - P.blk_lvl0[P.p], NLi = P.blk_lvl0[P.p];
+  if (which == 1 ? NLc <= kShallowLevels : (P.m == 0 || !c->deep_int)) return false;
+  narrow = which == 1 ? P.s < (long long)kNarrowRows * NLc : P.m < (long long)kNarrowRows * NLi;
+  return true;
+}
+
+// Tables of the panel solve in precision T, for narrow blocks whose solution
+// fits the shared memory of a CTA
+template <typename T>
+void panel_plan(ddlr_ctx *c, int which) {
+  const Plan &P = c->P;
+  ddlr_ctx::Panel &D = Prec<T>::pan(c)[which];
+  bool narrow = false;
+  if (!deep_blocks(c, which, narrow) || !narrow) return;
+  int dev = 0, optin = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  const int b0 = which == 0 ? 0 : P.p, b1 = which == 0 ? P.p : P.p + 1;
+  PanelGeo g{};
+  std::vector<int2> blk, prow;
+  std::vector<int4> pan;
+  std::vector<int> src, col;
+  std::vector<unsigned char> dirs;
+  for (int b = b0; b < b1; b++) {
+    const int r0 = P.blk_row0[b], r1 = P.blk_row0[b + 1];
+    g.rcap = std::max(g.rcap, r1 - r0);
+    blk.push_back(make_int2(int(prow.size()), (r1 - r0 + kPanelRows - 1) / kPanelRows));
+    for (int p0 = r0; p0 < r1; p0 += kPanelRows) {
+      const int pe = std::min(r1, p0 + kPanelRows);
+      int4 pn{};
+      for (int dir = 0; dir < 2; dir++) {
+        const auto &span = dir ? P.u_span : P.l_span;
+        const auto &cc = dir ? P.u_col : P.l_col;
+        const size_t base = src.size();
+        int w = 0;
+        for (int r = p0; r < pe; r++) {
+          int cnt = 0;
+          for (int kk = 0; kk < span[2 * r + 1]; kk++) {
+            const int slot = span[2 * r] + 32 * kk, ci = cc[slot];
+            if (dir ? ci < pe : ci >= p0) continue;          // inside the panel
+            const int u = cnt / kPanelLanes;
+            if (u >= w) {
+              w = u + 1;
+              src.resize(base + size_t(w) * kPanelNT, -1);
+              col.resize(src.size(), 0);
+            }
+            const size_t e = base + size_t(u) * kPanelNT + (r - p0) * kPanelLanes + cnt % kPanelLanes;
+            src[e] = slot;
+            col[e] = ci - r0;
+            cnt++;
+          }
+        }
+        if (src.size() / kPanelNT > 0x3fffffff) return;
+        (dir ? pn.z : pn.x) = int(base / kPanelNT);
+        (dir ? pn.w : pn.y) = w;
+        dirs.resize(src.size() / kPanelNT, (unsigned char)dir);
+      }
+      pan.push_back(pn);
+      prow.push_back(make_int2(p0, pe - p0));
+    }
+  }
+  const size_t smem = panel_smem_bytes<T>(g.rcap);
+  if ((long long)smem > optin - 128) return;
+  raise_smem_limit((const void *)k_panel_solve<T>, smem);
+  g.nblk = b1 - b0;
+  g.blk = c->upload(blk);
+  g.pan = c->upload(pan);
+  g.prow = c->upload(prow);
+  g.col = c->upload(col);
+  D.src = c->upload(src);
+  D.dir = c->upload(dirs);
+  D.npan = int(prow.size());
+  D.nent = (long long)src.size();
+  D.ent = c->alloc<T>(src.size());
+  D.inv = c->alloc<T>(size_t(2) * kPanelRows * kPanelRows * prow.size());
+  sync(c);                                    // the tables above are locals
+  D.g = g;
+}
+
+// Tables of the deep solve in precision T (ddlr_deep.cuh): which = 0 the
+// interior blocks (a part each), 1 C_a cut into the parts of one cluster.
+// C_a takes the smallest cluster that holds its solution and gives a level of
+// average width at most one pass of a set of warps per CTA (64^3, natural order,
+// 420 rows a level: see k_deep_solve).  Served where every part's solution,
+// tables and a ring of eight of its largest stages (or of all its stages) fit
+// the shared memory of a CTA.
+// DDLR_DEEP=0 switches it off, DDLR_DEEP_CTAS sets the smallest cluster (tests).
+template <typename T>
+void deep_plan(ddlr_ctx *c, int which) {
+  const Plan &P = c->P;
+  ddlr_ctx::Deep &D = Prec<T>::deep(c)[which];
+  const char *force = getenv("DDLR_DEEP_CTAS");
+  bool narrow = false;
+  if (!deep_blocks(c, which, narrow) || narrow) return;
+  const int NLc = P.blk_lvl0[P.p + 1] - P.blk_lvl0[P.p];
+  int dev = 0, optin = 0, per_sm = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (sms <= 0) return;
+  // blocks beyond one per SM share an SM's memory, up to four of them
+  const int cps = which == 1 ? 1 : std::max(1, std::min(4, (P.p + sms - 1) / sms));
+  const long long budget0 = std::min<long long>(optin, per_sm / cps - 1024) - 128;
+  const int cmin = which == 0 ? 1 : std::max(force ? atoi(force) : 1, int((long long)P.s / (128LL * NLc)));
+  for (int C = 1; C <= (which == 0 ? 1 : kDeepMaxCtas); C *= 2) {
+    if (which == 1 && C < cmin && C < kDeepMaxCtas) continue;
+    // multicolour orders (deep ones come from fill) scatter a level over the
+    // original order: nearly every row would be exchanged (64^3, IC(2): more
+    // received values than fit), so they are cut no further than one part
+    if (which == 1 && C > 1 && c->opt.c_order != 0) return;
+    if (which == 1 && ((long long)P.s / C) * (long long)sizeof(T) > budget0) continue;
+    const int np = which == 0 ? P.p : C;
+    std::vector<DeepPart> part;
+    std::vector<DeepStage> stage;
+    std::vector<int4> sl, push, fix;
+    std::vector<int2> srow;
+    std::vector<int> rpos(P.n, 0);
+    std::vector<int> lvl_of_stage, owner;      // owner: part of an interface row
+    std::vector<std::vector<int>> stage_of(np);// stage of (part, level) forward, counted in the part, or -1
+    if (which == 1) {
+      owner.resize(P.s);
+      for (int j = 0; j < P.s; j++) owner[j] = int((long long)P.iface_rank[j] * C / P.s);
+    }
+    long long ol = 0, ou = 0, total_max = 0, stage_max = 0;
+    int zcap = 0, scap = 0, tcap = 0;
+    bool bad = false;
+    for (int q = 0; q < np; q++) {
+      DeepPart pt{int(sl.size()), 0, int(stage.size()), 0, 0, 0};
+      const int b = which == 0 ? q : P.p, l0 = P.blk_lvl0[b], NL = P.blk_lvl0[b + 1] - l0;
+      stage_of[q].assign(NL, -1);
+      for (int l = 0; l < NL; l++) {
+        const int r0 = P.lvl_row0[l0 + l], r1 = r0 + P.lvl_nrows[l0 + l], s0 = int(sl.size());
+        for (int r = r0; r < r1;) {
+          if (which == 1 && owner[r - P.m] != q) { r++; continue; }
+          int e = r;
+          while (e < r1 && e - r < kSlice && (which == 0 || owner[e - P.m] == q)) e++;
+          int wl = 0, wu = 0;
+          for (int t = r; t < e; t++) {
+            wl = std::max(wl, P.l_span[2 * t + 1]);
+            wu = std::max(wu, P.u_span[2 * t + 1]);
+            rpos[t] = (int(sl.size()) - pt.slice0) * 32 + (t - r);
+          }
+          wl = deep_width(wl);
+          wu = deep_width(wu);
+          sl.push_back(make_int4(int(ol / 128), wl, int(ou / 128), wu));
+          srow.push_back(make_int2(r, e - r));
+          ol += (long long)deep_slice_bytes<T>(wl);
+          ou += (long long)deep_slice_bytes<T>(wu);
+          r = e;
+        }
+        if (int(sl.size()) == s0) continue;
+        stage_of[q][l] = int(stage.size()) - pt.stage0;
+        DeepStage st{};
+        st.a = s0 - pt.slice0;
+        st.b = int(sl.size()) - pt.slice0;
+        stage.push_back(st);
+        lvl_of_stage.push_back(l);
+      }
+      pt.nslice = int(sl.size()) - pt.slice0;
+      pt.nfwd = int(stage.size()) - pt.stage0;
+      for (int j = pt.nfwd - 1; j >= 0; j--) {
+        stage.push_back(stage[pt.stage0 + j]);
+        lvl_of_stage.push_back(lvl_of_stage[pt.stage0 + j]);
+      }
+      pt.nstage = 2 * pt.nfwd;
+      part.push_back(pt);
+      scap = std::max(scap, pt.nslice);
+      tcap = std::max(tcap, pt.nstage);
+      if (ol / 128 > 0x7fffffffLL || ou / 128 > 0x7fffffffLL) { bad = true; break; }
+    }
+    if (bad) return;
+    // received values: every row of another part that a part's rows read, once
+    // per sweep, counted for the stage that reads it first
+    std::vector<std::vector<std::vector<int4>>> out(np);
+    if (np > 1 && which == 1) {
+      for (int q = 0; q < np; q++) out[q].resize(part[q].nstage);
+      std::vector<int> seen(P.s), at(P.s);
+      for (int dir = 0; dir < 2; dir++) {
+        std::fill(seen.begin(), seen.end(), -1);
+        for (int q = 0; q < np; q++) {
+          DeepPart &pt = part[q];
+          for (int j = 0; j < pt.nfwd; j++) {
+            const int js = dir ? pt.nfwd + j : j;
+            DeepStage &sg = stage[pt.stage0 + js];
+            for (int i = sg.a; i < sg.b; i++)
+              for (int t = 0; t < srow[pt.slice0 + i].y; t++) {
+                const int r = srow[pt.slice0 + i].x + t;
+                const int *sp = (dir ? P.u_span.data() : P.l_span.data()) + 2 * size_t(r);
+                for (int kk = 0; kk < sp[1]; kk++) {
+                  const int cc = (dir ? P.u_col : P.l_col)[sp[0] + 32 * kk], h = cc - P.m, o = owner[h];
+                  if (o == q) continue;
+                  if (seen[h] != q) {
+                    seen[h] = q;
+                    at[h] = pt.nslice * 32 + pt.nhalo++;
+                    sg.halo++;
+                    // the level of row cc is that of its stage in its part
+                    const int lv = int(std::upper_bound(P.lvl_row0.begin() + P.blk_lvl0[P.p], P.lvl_row0.end(), cc) -
+                                       P.lvl_row0.begin()) - 1 - P.blk_lvl0[P.p];
+                    const int so = stage_of[o][lv];
+                    out[o][dir ? part[o].nstage - 1 - so : so].push_back(make_int4(rpos[cc], q, at[h], js));
+                  }
+                  fix.push_back(make_int4(pt.slice0 + i, dir, kk * 32 + t, at[h]));
+                }
+              }
+          }
+        }
+      }
+    }
+    for (int q = 0; q < np; q++) zcap = std::max(zcap, part[q].nslice * 32 + part[q].nhalo);
+    for (int q = 0; q < np; q++) {
+      const DeepPart &pt = part[q];
+      long long lin = 0;
+      for (int j = 0; j < pt.nstage; j++) {
+        DeepStage &sg = stage[pt.stage0 + j];
+        const int4 ea = sl[pt.slice0 + sg.a], eb = sl[pt.slice0 + sg.b - 1];
+        const bool f = j < pt.nfwd;
+        sg.src = f ? ea.x : ea.z;
+        sg.bytes = (f ? eb.x : eb.z) - sg.src + int(deep_slice_bytes<T>(f ? eb.y : eb.w) / 128);
+        sg.push = int(push.size());
+        if (!out[q].empty()) push.insert(push.end(), out[q][j].begin(), out[q][j].end());
+        stage_max = std::max(stage_max, (long long)sg.bytes * 128);
+        lin += sg.bytes;
+      }
+      total_max = std::max(total_max, lin * 128);
+    }
+    DeepStage end{};
+    end.push = int(push.size());
+    stage.push_back(end);
+    DeepGeo g{};
+    g.ctas = C; g.nparts = np; g.zcap = zcap; g.scap = scap; g.tcap = tcap;
+    const long long budget = budget0 - (long long)deep_smem_bytes<T>(g);
+    const long long want = std::min(total_max + stage_max, std::max(8 * stage_max, 16LL << 10));
+    const long long ring = std::min(std::min(budget, total_max + stage_max), 64LL << 10) & ~127LL;
+    if (std::min(budget, std::max(want, ring)) < want) continue;
+    g.ring_bytes = int(std::max(ring, (want + 127) & ~127LL));
+    // places in the ring: one stage after the other, from the start again
+    // where one does not fit before the end
+    for (const DeepPart &pt : part) {
+      int pos = 0, lin = 0;
+      const int R = g.ring_bytes / 128;
+      for (int j = 0; j < pt.nstage; j++) {
+        DeepStage &sg = stage[pt.stage0 + j];
+        if (pos + sg.bytes > R) { lin += R - pos; pos = 0; }
+        sg.pos = pos;
+        sg.lin = lin;
+        pos += sg.bytes;
+        lin += sg.bytes;
+      }
+    }
+    const size_t smem = deep_smem_bytes<T>(g);
+    if ((long long)smem > budget0) continue;
+    raise_smem_limit((const void *)k_deep_solve<T>, smem);
+    if (C > 8) ck(cudaFuncSetAttribute(k_deep_solve<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1), "attr");
+    if (C > 1) {
+      int fit = 0;
+      DeepLaunch L(g, smem, nullptr);
+      if (cudaOccupancyMaxActiveClusters(&fit, k_deep_solve<T>, &L.cfg) != cudaSuccess || fit < 1) {
+        cudaGetLastError();
+        continue;
+      }
+    }
+    if (push.empty()) push.push_back(make_int4(0, 0, 0, 0));
+    g.part = c->upload(part);
+    g.stage = c->upload(stage);
+    g.push = c->upload(push);
+    g.sl = c->upload(sl);
+    g.srow = c->upload(srow);
+    const int *rp = c->upload(rpos);
+    const int4 *fx = c->upload(fix);
+    D.nslices = int(sl.size());
+    D.pl = c->alloc<unsigned char>(size_t(ol));
+    D.pu = c->alloc<unsigned char>(size_t(ou));
+    KL(c, "setup", c->stream, k_deep_cols<T>, D.nslices, 128, 0, g, c->l_span, c->u_span, c->S.l_col, c->S.u_col, rp,
+       D.pl, D.pu);
+    if (!fix.empty())
+      KL(c, "setup", c->stream, k_deep_fix<T>, nblk((long long)fix.size()), kThreads, 0, int(fix.size()), g, fx, D.pl,
+         D.pu);
+    sync(c);                                  // the tables above are locals
+    D.g = g;
+    return;
+  }
+}
+
+// the factor's values packed for the deep solve (after the numeric setup)
+template <typename T>
+void deep_pack(ddlr_ctx *c) {
+  for (int i = 0; i < 2; i++) {
+    const ddlr_ctx::Panel &N = Prec<T>::pan(c)[i];
+    if (N.g.nblk > 0) {
+      if (N.nent > 0)                           // none when every block is one panel
+        KL(c, "setup", c->stream, k_panel_vals<T>, nblk(N.nent), kThreads, 0, N.nent, N.src, N.dir,
+           Prec<T>::l(c), Prec<T>::u(c), (T *)N.ent);
+      KL(c, "setup", c->stream, k_panel_inv<T>, N.npan, 32, 0, N.g.prow, c->f_rp, c->f_ci, c->fval, (T *)N.inv);
+    }
+    const ddlr_ctx::Deep &D = Prec<T>::deep(c)[i];
+    if (D.g.ctas > 0)
+      KL(c, "setup", c->stream, k_deep_pack<T>, D.nslices, 128, 0, D.g, c->l_span, c->u_span, Prec<T>::l(c),
+         Prec<T>::u(c), Prec<T>::dinv(c), D.pl, D.pu);
+  }
+}
+
 // FP32 / BF16 copies used by the mixed-precision preconditioner
 void make_low_precision(ddlr_ctx *c) {
   const Plan &P = c->P;
@@ -1207,8 +1549,7 @@ void make_low_precision(ddlr_ctx *c) {
        (const int *)nullptr);
   KL(c, "setup", c->stream, (k_cast<float, double>), nblk(lu), kThreads, 0, lu, c->u64, c->u32, (const int *)nullptr);
   KL(c, "setup", c->stream, (k_cast<float, double>), nblk(P.n), kThreads, 0, (long long)P.n, c->dinv64, c->dinv32, (const int *)nullptr);
-  const long long nds = (long long)P.nslice * kSlice;
-  KL(c, "setup", c->stream, (k_cast<float, double>), nblk(nds), kThreads, 0, nds, c->dinvs64, c->dinvs32, (const int *)nullptr);
+  deep_pack<float>(c);
   const long long ne = (long long)P.eh_ci.size();
   KL(c, "setup", c->stream, (k_cast<float, double>), nblk(ne), kThreads, 0, ne, c->eh64, c->eh32, (const int *)nullptr);
   KL(c, "setup", c->stream, (k_cast<float, double>), nblk(ne), kThreads, 0, ne, c->eht64, c->eht32, (const int *)nullptr);
@@ -1610,7 +1951,7 @@ ddlr_status cheb_setup(ddlr_ctx *c) {
   double *r = c->w64[0], *z = c->w64[1], *q = c->w64[2], *pv = c->w64[3], *pp = c->w64[4], *w = c->w64[5];
   const double *lv = c->l64, *uv = c->u64, *di = c->dinv64;
   KL(c, "setup", c->stream, k_cheb_start, nblk(s), kThreads, 0, s, m, c->cz_rank, c->opt.seed, r);
-  chunk_sweeps<double>(c, c->stream, P.ch_c_ptr, "cheb_dsolve", lv, uv, di, r, z, nullptr);
+  c_block_solve<double>(c, c->stream, "cheb_dsolve", lv, uv, di, r, z, nullptr);
   KL(c, "setup", c->stream, (k_dot_partial<double, 256>), kRedGrid, 256, 0, (long long)s, r + m, z + m, c->part64,
      (const int *)nullptr);
   KL(c, "setup", c->stream, k_cheb_reduce_norm, 1, 32, 0, kRedGrid, c->part64, c->cz_b0);
@@ -1626,7 +1967,7 @@ ddlr_status cheb_setup(ddlr_ctx *c) {
     KL(c, "setup", c->stream, k_reduce_scalar, 1, 32, 0, kRedGrid, c->part64, c->cz_al + j, 0,
        (const int *)nullptr);
     KL(c, "setup", c->stream, k_cheb_lz_sub, nblk(s), kThreads, 0, s, m, c->cz_al + j, pv, w);
-    chunk_sweeps<double>(c, c->stream, P.ch_c_ptr, "cheb_dsolve", lv, uv, di, w, z, nullptr);
+    c_block_solve<double>(c, c->stream, "cheb_dsolve", lv, uv, di, w, z, nullptr);
     KL(c, "setup", c->stream, (k_dot_partial<double, 256>), kRedGrid, 256, 0, (long long)s, w + m, z + m,
        c->part64, (const int *)nullptr);
     KL(c, "setup", c->stream, k_cheb_reduce_norm, 1, 32, 0, kRedGrid, c->part64, c->cz_be + j);
@@ -1692,12 +2033,13 @@ ddlr_status numeric_setup(ddlr_ctx *c) {
   ck(cudaMemsetAsync(c->l64, 0, sizeof(double) * P.l_col.size(), c->stream), "memset");
   ck(cudaMemsetAsync(c->u64, 0, sizeof(double) * P.u_col.size(), c->stream), "memset");
   KL(c, "setup", c->stream, k_solve_layout<double>, nblk(nf), kThreads, 0, (int)nf, c->f_row, c->f_rp,
-     c->map_l, c->map_u, c->row_slot, c->fval, c->l64, c->u64, c->dinv64, c->dinvs64);
+     c->map_l, c->map_u, c->fval, c->l64, c->u64, c->dinv64);
   if (c->lx64) {
     const long long nsl = (long long)P.l_col.size();
     KL(c, "setup", c->stream, k_prescale_cols<double>, nblk(nsl), kThreads, 0, nsl, c->S.l_col, c->l64,
        c->dinv64, c->lx64);
   }
+  deep_pack<double>(c);
   int fl[4];
   read_dev(c, fl, c->dflag, sizeof(fl));
   if (fl[3]) { clear_timeout(c); c->err = "a bounded device wait timed out"; return DDLR_ERR_TIMEOUT; }
@@ -1908,17 +2250,14 @@ void allocate(ddlr_ctx *c) {
     }
   }
   c->dinv64 = c->alloc<double>(n);
-  c->dinvs64 = c->alloc<double>(size_t(P.nslice) * kSlice);
-  ck(cudaMemsetAsync(c->dinvs64, 0, sizeof(double) * size_t(P.nslice) * kSlice, c->stream), "memset");
-  c->row_slot = c->upload(P.row_slot);
   c->l_span = reinterpret_cast<int2 *>(c->upload(P.l_span));
   c->u_span = reinterpret_cast<int2 *>(c->upload(P.u_span));
   c->blk_row0 = c->upload(P.blk_row0);
   c->chunks = c->upload(P.chunks);
   if (!P.lv_desc.empty()) c->lv_desc = reinterpret_cast<int4 *>(c->upload(P.lv_desc));
   {
-    // interior-solve kernel for deep factors: TMA-pipelined level schedule
-    // (default), synchronisation-free, or plain level schedule
+    // interior-solve kernel for deep factors: the level pipeline of
+    // ddlr_deep.cuh (default), synchronisation-free, or plain level schedule
     // (DDLR_SOLVE=tma|sf|plain)
     const char *env = getenv("DDLR_SOLVE");
     const std::string kind = env ? env : "tma";
@@ -1932,9 +2271,7 @@ void allocate(ddlr_ctx *c) {
     const bool sf_ok = P.tma_zs > 0 && kind == "sf";
     c->use_sf64 = sf_ok && sf_smem_bytes<double>(P) <= size_t(optin);
     c->use_sf32 = sf_ok && sf_smem_bytes<float>(P) <= size_t(optin);
-    const bool off = kind == "plain";
-    c->use_tma64 = !off && !c->use_sf64 && tma_config<double>(P, c->tma64);
-    c->use_tma32 = !off && !c->use_sf32 && tma_config<float>(P, c->tma32);
+    c->deep_int = kind != "plain" && !c->use_sf64 && !c->use_sf32;
     if (c->use_sf64)
       raise_smem_limit((const void *)k_sptrsv_blocks_sf<double, 256, 4>, sf_smem_bytes<double>(P));
     if (c->use_sf32)
@@ -1946,10 +2283,6 @@ void allocate(ddlr_ctx *c) {
     ck(cudaFuncSetAttribute(k_u_add_smem, cudaFuncAttributePreferredSharedMemoryCarveout, 100), "attr");
     ck(cudaFuncSetAttribute(k_u_add_smem, cudaFuncAttributeMaxDynamicSharedMemorySize, int(urows_smem_bytes(64))),
        "attr");
-    if (c->use_tma64)
-      raise_smem_limit((const void *)k_sptrsv_blocks_tma<double, 256>, tma_smem_bytes<double>(c->tma64));
-    if (c->use_tma32)
-      raise_smem_limit((const void *)k_sptrsv_blocks_tma<float, 256>, tma_smem_bytes<float>(c->tma32));
   }
   c->eh64 = c->alloc<double>(P.eh_ci.size());
   c->eht64 = c->alloc<double>(P.eht_ci.size());
@@ -1972,11 +2305,18 @@ void allocate(ddlr_ctx *c) {
   mmax = std::max(std::min(mmax, P.s), k);
   c->part64 = c->alloc<double>(size_t(kRedGrid) * std::max(k + 2, mmax + 2) + 2 * kRedGrid);
   pz_setup(c, mmax);
+  panel_plan<double>(c, 0);
+  deep_plan<double>(c, 0);
+  panel_plan<double>(c, 1);
+  deep_plan<double>(c, 1);
   if (c->opt.precision == 1) {
+    panel_plan<float>(c, 0);
+  deep_plan<float>(c, 0);
+    panel_plan<float>(c, 1);
+  deep_plan<float>(c, 1);
     c->l32 = c->alloc<float>(P.l_col.size());
     c->u32 = c->alloc<float>(P.u_col.size());
     c->dinv32 = c->alloc<float>(n);
-    c->dinvs32 = c->alloc<float>(size_t(P.nslice) * kSlice);
     c->eh32 = c->alloc<float>(P.eh_ci.size());
     c->eht32 = c->alloc<float>(P.eht_ci.size());
     if (c->opt.uk_bf16) c->Ub16 = c->alloc<__nv_bfloat16>(size_t(c->urows) * k);
@@ -2461,7 +2801,7 @@ void cheb_dsolve(ddlr_ctx *c, cudaStream_t st, const T *x, T *z, int R, const in
   const T *lv0 = Prec<T>::l(c), *lx = Prec<T>::lx(c), *uv = Prec<T>::u(c), *di = Prec<T>::dinv(c);
   const std::vector<int> &ptr = c->P.ch_c_ptr;
   if (R == 1) {
-    chunk_sweeps<T>(c, st, ptr, "cheb_dsolve", lv0, uv, di, x, z, gate);
+    c_block_solve<T>(c, st, "cheb_dsolve", lv0, uv, di, x, z, gate);
     return;
   }
   const int nL = int(ptr.size()) - 1;

@@ -135,14 +135,12 @@ __global__ void k_ic_level(int cnt, const int *rows, const int *f_rp,
 template <typename T>
 __global__ void k_solve_layout(int nf, const int *f_row, const int *f_rp,
                                const int *map_l, const int *map_u,
-                               const int *row_slot, const double *fval, T *lval,
-                               T *uval, T *dinv, T *dinv_s) {
+                               const double *fval, T *lval, T *uval, T *dinv) {
   int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= nf) return;
   const int g = f_row[q];
   if (q == f_rp[g + 1] - 1) {
     dinv[g] = T(1.0 / fval[q]);
-    dinv_s[row_slot[g]] = T(1.0 / fval[q]);
   } else {
     lval[map_l[q]] = T(fval[q]);
     uval[map_u[q]] = T(fval[q]);
@@ -198,14 +196,6 @@ k_sptrsv_blocks(SolveLayout S, const T *lval, const T *uval, const T *dinv,
   }
 }
 
-// ----------------------------------------- TMA-pipelined interior solves
-// Shared-memory geometry of k_sptrsv_blocks_tma, chosen on the host.
-struct TmaCfg {
-  int zs_cap;      // rows of the largest interior block
-  int nl_cap;      // levels of the deepest block
-  int ns_cap;      // slices of the largest block + 1
-  int ring_bytes;  // staging ring (multiple of 128, >= the largest stage)
-};
 // nanoseconds of the global timer (bounded waits)
 __device__ __forceinline__ unsigned long long gtimer_ns() {
   unsigned long long t;
@@ -213,10 +203,9 @@ __device__ __forceinline__ unsigned long long gtimer_ns() {
   return t;
 }
 
-constexpr int kNBar = 64;       // mbarriers = stages in flight at most
-// the TMA solve waits at least this long for its copies (a CTA must not exit
+// the deep solve waits at least this long for its copies (a CTA must not exit
 // with copies still in flight into its shared memory)
-constexpr unsigned long long kTmaMinWaitNs = 1000000000ull;
+constexpr unsigned long long kDeepMinWaitNs = 1000000000ull;
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
   return (uint32_t)__cvta_generic_to_shared(p);
@@ -249,156 +238,6 @@ __device__ __forceinline__ void tma_load_1d(void *dst, const void *src, unsigned
       : "memory");
 }
 __host__ __device__ inline size_t al128(size_t b) { return (b + 127) & ~size_t(127); }
-
-template <typename T>
-__host__ __device__ inline size_t tma_smem_bytes(const TmaCfg &c) {
-  // barriers | ring | block solution | stage table (2 int4 + 1 int64 per stage) | slice table
-  return 8 * kNBar + size_t(c.ring_bytes) + al128(size_t(c.zs_cap) * sizeof(T)) +
-         al128(size_t(2 * c.nl_cap) * 40) + size_t(4 * c.ns_cap) * 4;
-}
-
-// All interior blocks of A0 in one launch, one CTA per block (Sec. 4.2: the p
-// local solves are independent).  The block's solution lives in shared
-// memory.  The sliced-ELL data of each level (values, column indices and the
-// inverse diagonal in slice layout; every piece a multiple of 128 bytes) is a
-// "stage"; stages are brought in by 1-D TMA bulk copies into a byte ring,
-// placed one after the other (wrapping to the ring start when a stage does
-// not fit before the end), as far ahead as the ring and the 64 mbarriers
-// allow.  Placement is a pure function of the stage sizes and is tabulated in
-// the prologue.  The last thread of the CTA issues the copies after the
-// barrier that ends a level (it has no row in levels narrower than NT-32, so
-// this stays off the level chain).  Forward sweep with L, backward sweep with
-// L^T.  Waits are bounded: on timeout *err is set and the CTA returns.
-template <typename T, int NT>
-__global__ void __launch_bounds__(NT)
-k_sptrsv_blocks_tma(SolveLayout S, const T *lval, const T *uval, const T *dinv_s,
-                    const T *x, T *z, const int *gate, TmaCfg cfg, int *err, unsigned long long limit_ns) {
-  if (gate && *gate) return;
-  __shared__ int s_abort;
-  extern __shared__ __align__(128) unsigned char smraw[];
-  uint64_t *bar = reinterpret_cast<uint64_t *>(smraw);
-  unsigned char *ring = smraw + 8 * kNBar;
-  const int R = cfg.ring_bytes;
-  T *zs = reinterpret_cast<T *>(ring + R);
-  unsigned char *tab = reinterpret_cast<unsigned char *>(zs) + al128(size_t(cfg.zs_cap) * sizeof(T));
-  int4 *sg0 = reinterpret_cast<int4 *>(tab);                  // {r0, nr, sa, oa}
-  int4 *sg1 = sg0 + 2 * cfg.nl_cap;                           // {ne, nsl, pos, bytes}
-  long long *slin = reinterpret_cast<long long *>(sg1 + 2 * cfg.nl_cap);  // linear start
-  int *st = reinterpret_cast<int *>(tab + al128(size_t(2 * cfg.nl_cap) * 40));
-  const int b = blockIdx.x, tid = threadIdx.x;
-  const int l0 = S.blk_lvl0[b], l1 = S.blk_lvl0[b + 1], NL = l1 - l0;
-  if (NL == 0) return;
-  const int rb0 = S.lvl_row0[l0], sb0 = S.lvl_slice0[l0];
-  const int NS = S.lvl_slice0[l1] - sb0;
-  const int nb = S.lvl_row0[l1 - 1] + S.lvl_nrows[l1 - 1] - rb0;
-  const int nstage = 2 * NL;
-  constexpr int PROD = NT - 1;
-  // stage j: forward level j (j < NL) or backward level 2NL-1-j
-  for (int j = tid; j < nstage; j += NT) {
-    const bool fwd = j < NL;
-    const int li = fwd ? j : nstage - 1 - j;
-    const int sa = S.lvl_slice0[l0 + li] - sb0, sbn = S.lvl_slice0[l0 + li + 1] - sb0;
-    const int *soff = fwd ? S.l_soff : S.u_soff;
-    const int oa = soff[sb0 + sa], ne = soff[sb0 + sbn] - oa;
-    sg0[j] = make_int4(S.lvl_row0[l0 + li] - rb0, S.lvl_nrows[l0 + li], sa, oa);
-    sg1[j] = make_int4(ne, sbn - sa, 0, ne * int(sizeof(T) + 4) + (sbn - sa) * 32 * int(sizeof(T)));
-  }
-  for (int i = tid; i <= NS; i += NT) {
-    st[4 * i] = S.l_soff[sb0 + i];
-    st[4 * i + 1] = i < NS ? S.l_sw[sb0 + i] : 0;
-    st[4 * i + 2] = S.u_soff[sb0 + i];
-    st[4 * i + 3] = i < NS ? S.u_sw[sb0 + i] : 0;
-  }
-  for (int i = tid; i < nb; i += NT) zs[i] = x[rb0 + i];
-  __syncthreads();
-  if (tid == PROD) {
-    // ring placement: consecutive, wrapping to 0 when a stage does not fit
-    long long lin = 0;
-    int pos = 0;
-    for (int j = 0; j < nstage; j++) {
-      const int by = sg1[j].w;
-      if (pos + by > R) { lin += R - pos; pos = 0; }
-      sg1[j].z = pos;
-      slin[j] = lin;
-      lin += by;
-      pos += by;
-    }
-    for (int q = 0; q < kNBar; q++) mbar_init(bar + q, 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    s_abort = 0;
-  }
-  int jn = 0;   // producer: next stage to issue
-  auto produce = [&](int jc) {
-    const long long lim = slin[jc] + R;
-    while (jn < nstage && jn - jc < kNBar) {
-      const int4 g0 = sg0[jn], g1 = sg1[jn];
-      if (slin[jn] + g1.w > lim) break;          // would reach the oldest live stage
-      const bool fwd = jn < NL;
-      unsigned char *dst = ring + g1.z;
-      uint64_t *bj = bar + (jn % kNBar);
-      mbar_expect_tx(bj, unsigned(g1.w));
-      if (g1.x > 0) {
-        tma_load_1d(dst, (fwd ? lval : uval) + g0.w, unsigned(g1.x) * (unsigned)sizeof(T), bj);
-        tma_load_1d(dst + size_t(g1.x) * sizeof(T), (fwd ? S.l_col : S.u_col) + g0.w, unsigned(g1.x) * 4u, bj);
-      }
-      tma_load_1d(dst + size_t(g1.x) * (sizeof(T) + 4), dinv_s + size_t(sb0 + g0.z) * 32,
-                  unsigned(g1.y) * 32u * (unsigned)sizeof(T), bj);
-      jn++;
-    }
-  };
-  if (tid == PROD) produce(0);
-  __syncthreads();
-  for (int j = 0; j < nstage; j++) {
-    const unsigned par = unsigned(j / kNBar) & 1u;
-    if (!mbar_try_wait(bar + (j % kNBar), par)) {
-      // bounded wait; a thread that gives up tells the others (the decision
-      // to stop is the CTA's, taken at the barrier below)
-      const unsigned long long t0 = gtimer_ns();
-      while (!mbar_try_wait(bar + (j % kNBar), par)) {
-        if (*(volatile int *)&s_abort) break;
-        if (gtimer_ns() - t0 > limit_ns) { atomicExch(&s_abort, 1); break; }
-      }
-    }
-    __syncthreads();
-    if (s_abort) {
-      // the copies issued for stages j .. jn-1 may still be in flight into
-      // this CTA's shared memory: the producer waits for them (bounded)
-      // before the CTA exits
-      if (tid == PROD) {
-        *err = 1;
-        for (int q = j; q < jn; q++) {
-          const unsigned pq = unsigned(q / kNBar) & 1u;
-          const unsigned long long t0 = gtimer_ns();
-          while (!mbar_try_wait(bar + (q % kNBar), pq) && gtimer_ns() - t0 < limit_ns) {
-          }
-        }
-      }
-      return;
-    }
-    const int4 g0 = sg0[j], g1 = sg1[j];
-    const bool fwd = j < NL;
-    const unsigned char *slot = ring + g1.z;
-    const T *sv = reinterpret_cast<const T *>(slot);
-    const int *sc = reinterpret_cast<const int *>(slot + size_t(g1.x) * sizeof(T));
-    const T *sd = reinterpret_cast<const T *>(slot + size_t(g1.x) * (sizeof(T) + 4));
-    const int r0 = g0.x, nr = g0.y, sa = g0.z, oa = g0.w;
-    for (int i = tid; i < nr; i += NT) {
-      const int sl = sa + (i >> 5), ln = i & 31;
-      const int2 so = *reinterpret_cast<const int2 *>(st + 4 * sl + (fwd ? 0 : 2));
-      const int o = so.x - oa + ln, w = so.y;
-      T acc = zs[r0 + i];
-      for (int kk = 0; kk < w; kk++) acc -= sv[o + 32 * kk] * zs[sc[o + 32 * kk] - rb0];
-      zs[r0 + i] = acc * sd[i];
-    }
-    __syncthreads();
-    if (tid == PROD && jn < nstage) {
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      produce(j + 1);
-    }
-  }
-  for (int i = tid; i < nb; i += NT) z[rb0 + i] = zs[i];
-}
 
 // --------------------------------------- synchronisation-free interior solve
 // Row r of the factor (device order) keeps {first slot, number of entries} of
