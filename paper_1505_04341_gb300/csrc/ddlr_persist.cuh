@@ -141,49 +141,131 @@ __device__ __forceinline__ double *pz_buf(const PzOp<T, TU> &O, int slot) {
   return O.part + (size_t)(slot % 3) * gridDim.x * O.pstride;
 }
 
-// CTA sum of v written to pt[blockIdx.x * pstride] (sm: NT/32 doubles)
+// Reductions.  On this part an FP64 warp instruction takes 64 cycles of its
+// sub-partition whatever its active lanes, so a shuffle tree in each of 32
+// warps costs 32 x 5 / 4 x 64 = 2,560 cycles, and a scalar division by every
+// thread about twice that.  Values are therefore summed by 4 warps (one per
+// sub-partition) from shared memory, each lane several of them before its
+// shuffles, and scalars are formed by one thread and broadcast.
+
+// CTA sum of v over the first `active` threads (the others hold none; the same
+// number in every thread), written to pt[blockIdx.x * pstride].  sm: NT + 32
+// doubles.
 template <int NT>
-__device__ __forceinline__ void pz_put(double v, double *pt, int pstride, double *sm) {
-  v = block_sum<double, NT>(v, sm);
-  if (threadIdx.x == 0) pt[(size_t)blockIdx.x * pstride] = v;
+__device__ __forceinline__ void pz_put(double v, int active, double *pt, int pstride, double *sm) {
+  const int cnt = min(NT, active);
+  if (threadIdx.x < cnt) sm[threadIdx.x] = v;
+  __syncthreads();
+  if (threadIdx.x < 128) {
+    double a = 0, b = 0;
+    int i = threadIdx.x;
+    for (; i + 128 < cnt; i += 256) { a += sm[i]; b += sm[i + 128]; }
+    if (i < cnt) a += sm[i];
+    a += b;
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+    if ((threadIdx.x & 31) == 0) sm[NT + 16 + (threadIdx.x >> 5)] = a;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const double *t = sm + NT + 16;
+    pt[(size_t)blockIdx.x * pstride] = (t[0] + t[1]) + (t[2] + t[3]);
+  }
 }
 
-// sum over CTAs of pt[g * pstride] in a fixed order, returned to every thread
-__device__ __forceinline__ double pz_get(const double *pt, int pstride, double *bc) {
+// whether v is infinite or a NaN, and a <= b for values that are neither and not
+// negative, on the bit patterns (a double comparison is an FP64 instruction)
+__device__ __forceinline__ bool pz_bad(double v) {
+  return (__double_as_longlong(v) & 0x7ff0000000000000LL) == 0x7ff0000000000000LL;
+}
+__device__ __forceinline__ bool pz_le(double a, double b) { return __double_as_longlong(a) <= __double_as_longlong(b); }
+
+// sum over CTAs of pt[g * pstride] in a fixed order; then f(sum), evaluated by
+// one thread, returned to every thread beside it (divisions, roots)
+struct PzScalar { double sum; double2 f; };
+template <typename F>
+__device__ __forceinline__ PzScalar pz_get(const double *pt, int pstride, double *bc, F f) {
   if (threadIdx.x < 32) {
     const int l = threadIdx.x;
     double s = 0;
     for (int g = l; g < (int)gridDim.x; g += 32) s += pt[(size_t)g * pstride];
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (l == 0) bc[0] = s;
+    if (l == 0) {
+      const double2 d = f(s);
+      bc[0] = s; bc[1] = d.x; bc[2] = d.y;
+    }
   }
   __syncthreads();
-  const double r = bc[0];
+  const PzScalar r{bc[0], make_double2(bc[1], bc[2])};
   __syncthreads();
   return r;
+}
+__device__ __forceinline__ double pz_get(const double *pt, int pstride, double *bc) {
+  return pz_get(pt, pstride, bc, [](double) { return make_double2(0.0, 0.0); }).sum;
+}
+
+// sums over groups: out[c] = f(c, sum_{q < ng} in[q * ld + c]), c < nc, with up
+// to 128 threads (TPC of them per column, a power of two); in: shared memory
+template <typename T, typename F>
+__device__ __forceinline__ void pz_fold(const T *in, int ng, int ld, int nc, F f) {
+  int lt = 0;                                        // log2(TPC)
+  while (lt < 5 && (nc << (lt + 1)) <= 128) lt++;
+  const int tpc = 1 << lt;
+  for (int c0 = 0; c0 < nc; c0 += 128 >> lt) {
+    const int c = c0 + (threadIdx.x >> lt), part = threadIdx.x & (tpc - 1);
+    if (threadIdx.x < 128) {
+      T a = 0, b = 0;
+      if (c < nc) {
+        int q = part;
+        for (; q + tpc < ng; q += 2 * tpc) { a += in[q * ld + c]; b += in[(q + tpc) * ld + c]; }
+        if (q < ng) a += in[q * ld + c];
+      }
+      a += b;
+      for (int o = tpc >> 1; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o, tpc);
+      if (c < nc && part == 0) f(c, a);
+    }
+  }
 }
 
 // out[c] = (coef ? coef[c] : 1) * sum_g pt[g * pstride + c], c < ncol, in
 // precision T in shared memory; with H (ncol x ncol row-major): out = H *
-// (those sums)
+// (those sums).  Lanes run over columns (the partials are read coalesced);
+// tmp: NT values of T.
 template <int NT, typename T>
 __device__ __forceinline__ void pz_get_cols(const double *pt, int pstride, int ncol, const T *coef, const T *H,
                                             T *out, T *tmp) {
-  const int wi = threadIdx.x >> 5, l = threadIdx.x & 31;
-  T *dst = H ? tmp : out;
-  for (int c = wi; c < ncol; c += NT / 32) {
-    T s = 0;
-    for (int g = l; g < (int)gridDim.x; g += 32) s += T(pt[(size_t)g * pstride + c]);
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (l == 0) dst[c] = coef ? ro(coef + c) * s : s;
+  const int G = (int)gridDim.x, P = min(G, max(1, NT / ncol));
+  for (int e = threadIdx.x; e < P * ncol; e += NT) {
+    const int q = e / ncol, c = e - q * ncol;
+    T a = 0, b = 0;
+    int g = q;
+    for (; g + P < G; g += 2 * P) {
+      a += T(pt[(size_t)g * pstride + c]);
+      b += T(pt[(size_t)(g + P) * pstride + c]);
+    }
+    if (g < G) a += T(pt[(size_t)g * pstride + c]);
+    if (P == 1) out[c] = H ? a + b : (coef ? ro(coef + c) * (a + b) : a + b);
+    else tmp[e] = a + b;
   }
   __syncthreads();
+  if (P > 1) {
+    pz_fold<T>(tmp, P, ncol, ncol, [&](int c, T v) { out[c] = coef && !H ? ro(coef + c) * v : v; });
+    __syncthreads();
+  }
   if (H) {
-    for (int c = threadIdx.x; c < ncol; c += NT) {
-      T s = 0;
-      for (int b = 0; b < ncol; b++) s += ro(H + c * ncol + b) * tmp[b];
-      out[c] = s;
+    // the product by rows: four lanes per row
+    for (int c0 = 0; c0 < ncol; c0 += NT / 4) {
+      const int c = c0 + (threadIdx.x >> 2), part = threadIdx.x & 3;
+      T v = 0;
+      if (c < ncol)
+        for (int b = part; b < ncol; b += 4) v += ro(H + c * ncol + b) * out[b];
+      if (c0 + ((threadIdx.x & ~31) >> 2) < ncol) {
+        v += __shfl_down_sync(0xffffffffu, v, 2, 4);
+        v += __shfl_down_sync(0xffffffffu, v, 1, 4);
+      }
+      if (c < ncol && part == 0) tmp[c] = v;
     }
+    __syncthreads();
+    for (int c = threadIdx.x; c < ncol; c += NT) out[c] = tmp[c];
     __syncthreads();
   }
 }
@@ -193,20 +275,51 @@ __device__ __forceinline__ void pz_get_cols(const double *pt, int pstride, int n
 template <int NT, typename T, typename TU, typename TX>
 __device__ __forceinline__ void pz_utx(int k, const TU *U, const TX *x, const double *xsc, int r0, int r1,
                                        double *pt, int pstride, double *red) {
-  const int G = NT / k;
+  const int G = min(NT / k, max(1, r1 - r0));
   const int c = threadIdx.x % k, g = threadIdx.x / k;
-  T acc = 0;
-  if (g < G)
-    for (int r = r0 + g; r < r1; r += G) acc += T(to_acc(ro(U + (size_t)r * k + c))) * pz_in<T>(x, xsc, r);
   T *rt = reinterpret_cast<T *>(red);
-  rt[threadIdx.x] = (g < G) ? acc : T(0);
-  __syncthreads();
-  if (threadIdx.x < k) {
-    T s = 0;
-    for (int gg = 0; gg < G; gg++) s += rt[gg * k + threadIdx.x];
-    pt[(size_t)blockIdx.x * pstride + threadIdx.x] = double(s);
+  if (g < G) {
+    T a = 0, b = 0;
+    int r = r0 + g;
+    for (; r + G < r1; r += 2 * G) {
+      a += T(to_acc(ro(U + (size_t)r * k + c))) * pz_in<T>(x, xsc, r);
+      b += T(to_acc(ro(U + (size_t)(r + G) * k + c))) * pz_in<T>(x, xsc, r + G);
+    }
+    if (r < r1) a += T(to_acc(ro(U + (size_t)r * k + c))) * pz_in<T>(x, xsc, r);
+    rt[threadIdx.x] = a + b;
   }
   __syncthreads();
+  pz_fold<T>(rt, G, k, k, [&](int cc, T v) { pt[(size_t)blockIdx.x * pstride + cc] = double(v); });
+  __syncthreads();
+}
+
+// sum_c row[c] vec[c], the row by 16-byte loads where its length allows (then
+// every row of U is aligned), in two chains
+template <typename T, typename TU>
+__device__ __forceinline__ T pz_row_dot(const TU *row, const T *vec, int k) {
+  constexpr int E = Unpack16<TU>::E;
+  T a = 0, b = 0;
+  if (k % E == 0) {
+    const uint4 *row4 = reinterpret_cast<const uint4 *>(row);
+#pragma unroll 4
+    for (int q = 0; q < k / E; q++) {
+      T e[E];
+      Unpack16<TU>::run(__ldg(row4 + q), e);
+#pragma unroll
+      for (int i = 0; i < E; i += 2) {
+        a += e[i] * vec[q * E + i];
+        b += e[i + 1] * vec[q * E + i + 1];
+      }
+    }
+  } else {
+    int c = 0;
+    for (; c + 1 < k; c += 2) {
+      a += T(to_acc(ro(row + c))) * vec[c];
+      b += T(to_acc(ro(row + c + 1))) * vec[c + 1];
+    }
+    if (c < k) a += T(to_acc(ro(row + c))) * vec[c];
+  }
+  return a + b;
 }
 
 // One level L of every block: mode 0 forward, 1 backward, 2 forward then
@@ -216,8 +329,10 @@ __device__ __forceinline__ void pz_utx(int k, const TU *U, const TX *x, const do
 template <int NT, typename T, typename TU, typename TX>
 __device__ __forceinline__ void pz_level(const PzOp<T, TU> &O, int L, int mode, const TX *x, const double *xsc,
                                          T *z, const double *racc, const double *zsc, double &acc, T *z2) {
-  const int c0 = O.lvl_ptr[L], cnt = O.lvl_ptr[L + 1] - c0;
-  for (int v = blockIdx.x * NT + threadIdx.x; v < cnt; v += gridDim.x * NT) {
+  const int c0 = O.lvl_ptr[L];
+  int v0, v1;
+  pz_range(O.lvl_ptr[L + 1] - c0, v0, v1);        // a level's rows over all CTAs
+  for (int v = v0 + threadIdx.x; v < v1; v += NT) {
     const int4 d = ro(O.desc + c0 + v);
     const int r = d.x;
     T zr;
@@ -282,10 +397,7 @@ __device__ __forceinline__ bool pz_apply(const PzOp<T, TU> &O, const double *x, 
     if (!pz_sync(O.gs, ep)) return false;
     pz_get_cols<NT, T>(pt, O.pstride, k, nullptr, O.Hk, vec, reinterpret_cast<T *>(red));   // H_k t
     for (int r = i0 + threadIdx.x; r < i1; r += NT) {
-      T t = 0;
-      const TU *row = O.U + (size_t)r * k;
-      for (int c = 0; c < k; c++) t += T(to_acc(ro(row + c))) * vec[c];
-      const T ur = u[r] + t;
+      const T ur = u[r] + pz_row_dot<T, TU>(O.U + (size_t)r * k, vec, k);
       u[r] = ur;
       if (racc) acc += racc[r] * (O.dsc ? ro(O.dsc + r) * double(ur) : double(ur));
     }
@@ -310,10 +422,7 @@ __device__ __forceinline__ bool pz_apply(const PzOp<T, TU> &O, const double *x, 
   pz_get_cols<NT, T>(pt, O.pstride, k, O.coef, (const T *)nullptr, vec, reinterpret_cast<T *>(red));
   const T i1mt = ro(O.inv1mt);
   for (int j = j0 + threadIdx.x; j < j1; j += NT) {                // w = G^-1 y; x_C - a w
-    T t = 0;
-    const TU *row = O.U + (size_t)j * k;
-    for (int c = 0; c < k; c++) t += T(to_acc(ro(row + c))) * vec[c];
-    const T wj = i1mt * y[j] + t;
+    const T wj = i1mt * y[j] + pz_row_dot<T, TU>(O.U + (size_t)j * k, vec, k);
     w[j] = wj;
     const T rv = pz_in<T>(x, xsc, m + j) - a * wj;
     rhs[m + j] = rv;
@@ -367,6 +476,17 @@ __global__ void __launch_bounds__(NT, 1) k_pcg_persist(PzOp<T, TU> O, PzPcg<T> P
   const int n = O.n;
   int i0, i1;
   pz_range(n, i0, i1);
+  // threads that hold a share of r.z after the preconditioner: its last rows
+  // are those of the levels (DDLR-1) or this CTA's range (DDLR-2)
+  int zact = i1 - i0;
+  if (O.variant != 2) {
+    zact = 0;
+    for (int L = 0; L < O.nL; L++) {
+      int v0, v1;
+      pz_range(O.lvl_ptr[L + 1] - O.lvl_ptr[L], v0, v1);
+      zact = max(zact, v1 - v0);
+    }
+  }
   // the first A0 solve of the preconditioner writes here (its first level
   // is done by whoever produces r)
   T *a0out = O.variant == 2 ? P.u : P.z;
@@ -380,7 +500,7 @@ __global__ void __launch_bounds__(NT, 1) k_pcg_persist(PzOp<T, TU> O, PzPcg<T> P
     pz_l0(O, i, pz_in<T>(P.b, O.dsc, i), a0out);
   }
   double *pt = pz_buf(O, slot++);
-  pz_put<NT>(acc, pt, O.pstride, red);
+  pz_put<NT>(acc, i1 - i0, pt, O.pstride, red);
   if (!pz_sync(O.gs, ep)) return;
   const double bb = pz_get(pt, O.pstride, bc);
   const double tol2 = P.tol * P.tol * bb;
@@ -391,10 +511,10 @@ __global__ void __launch_bounds__(NT, 1) k_pcg_persist(PzOp<T, TU> O, PzPcg<T> P
     acc = 0;
     if (!pz_apply<NT>(O, P.r, P.u, P.z, P.y, P.w, P.rhs, P.r, acc, ep, slot, red, vec, O.fuse0 != 0)) return;
     pt = pz_buf(O, slot++);
-    pz_put<NT>(acc, pt, O.pstride, red);
+    pz_put<NT>(acc, zact, pt, O.pstride, red);
     if (!pz_sync(O.gs, ep)) return;
     rz = pz_get(pt, O.pstride, bc);
-    if (!(rz == rz) || isinf(rz)) { status = 7; done = true; }
+    if (pz_bad(rz)) { status = 7; done = true; }
   }
   double *pold = P.p0, *pnew = P.p1;
   bool restart = false;
@@ -418,11 +538,12 @@ __global__ void __launch_bounds__(NT, 1) k_pcg_persist(PzOp<T, TU> O, PzPcg<T> P
       acc += pnew[i] * qi;
     }
     pt = pz_buf(O, slot++);
-    pz_put<NT>(acc, pt, O.pstride, red);
+    pz_put<NT>(acc, i1 - i0, pt, O.pstride, red);
     if (!pz_sync(O.gs, ep)) return;
-    pq = pz_get(pt, O.pstride, bc);
-    alpha = rz / pq;
-    if (!(alpha == alpha) || isinf(alpha)) { status = 7; break; }
+    const PzScalar sp = pz_get(pt, O.pstride, bc, [&](double v) { return make_double2(rz / v, 0.0); });
+    pq = sp.sum;
+    alpha = sp.f.x;
+    if (pz_bad(alpha)) { status = 7; break; }
     // x += alpha p; r -= alpha q; r.r (and r.z_old for flexible CG)
     acc = 0;
     double acc2 = 0;
@@ -435,14 +556,17 @@ __global__ void __launch_bounds__(NT, 1) k_pcg_persist(PzOp<T, TU> O, PzPcg<T> P
       pz_l0(O, i, pz_in<T>(P.r, O.dsc, i), a0out);
     }
     pt = pz_buf(O, slot++);
-    pz_put<NT>(acc, pt, O.pstride, red);
-    if (kFlex) pz_put<NT>(acc2, pt + 1, O.pstride, red);
+    pz_put<NT>(acc, i1 - i0, pt, O.pstride, red);
+    if (kFlex) {
+      __syncthreads();
+      pz_put<NT>(acc2, i1 - i0, pt + 1, O.pstride, red);
+    }
     if (!pz_sync(O.gs, ep)) return;
     rr = pz_get(pt, O.pstride, bc);
     if (kFlex) rzo = pz_get(pt + 1, O.pstride, bc);
     its += 1;
-    if (!(rr == rr) || isinf(rr)) { status = 7; break; }
-    if (rr <= tol2) {
+    if (pz_bad(rr)) { status = 7; break; }
+    if (pz_le(rr, tol2)) {
       // confirm with the true residual t = b - A x
       acc = 0;
       for (int i = i0 + threadIdx.x; i < i1; i += NT) {
@@ -455,10 +579,10 @@ __global__ void __launch_bounds__(NT, 1) k_pcg_persist(PzOp<T, TU> O, PzPcg<T> P
         acc += tr * tr;
       }
       pt = pz_buf(O, slot++);
-      pz_put<NT>(acc, pt, O.pstride, red);
+      pz_put<NT>(acc, i1 - i0, pt, O.pstride, red);
       if (!pz_sync(O.gs, ep)) return;
       rt2 = pz_get(pt, O.pstride, bc);
-      if (rt2 <= tol2) { status = 0; done = true; break; }
+      if (!pz_bad(rt2) && pz_le(rt2, tol2)) { status = 0; done = true; break; }
       restart = true;                       // continue from the true residual
       if (its >= P.maxit) { status = 5; break; }
       for (int i = i0 + threadIdx.x; i < i1; i += NT) {
@@ -473,13 +597,15 @@ __global__ void __launch_bounds__(NT, 1) k_pcg_persist(PzOp<T, TU> O, PzPcg<T> P
     acc = 0;
     if (!pz_apply<NT>(O, P.r, P.u, P.z, P.y, P.w, P.rhs, P.r, acc, ep, slot, red, vec, O.fuse0 != 0)) return;
     pt = pz_buf(O, slot++);
-    pz_put<NT>(acc, pt, O.pstride, red);
+    pz_put<NT>(acc, zact, pt, O.pstride, red);
     if (!pz_sync(O.gs, ep)) return;
-    const double rzn = pz_get(pt, O.pstride, bc);
-    beta = restart ? 0.0 : (kFlex ? (rzn - rzo) / rz : rzn / rz);
-    rz = rzn;
+    const PzScalar sz = pz_get(pt, O.pstride, bc, [&](double v) {
+      return make_double2(restart ? 0.0 : (kFlex ? (v - rzo) / rz : v / rz), 0.0);
+    });
+    beta = sz.f.x;
+    rz = sz.sum;
     restart = false;
-    if (!(rzn == rzn) || isinf(rzn)) { status = 7; break; }
+    if (pz_bad(rz)) { status = 7; break; }
     double *tp = pold;
     pold = pnew;
     pnew = tp;
@@ -511,41 +637,50 @@ struct LzCount {
   double q64, q32;
 };
 
-// partials of Q_{ncol}^T w over this CTA's rows [r0, r1), warp per column
-// (red: NT/32 doubles of shared memory).  With fewer columns than warps the
-// rows are split into nseg segments per column so every warp works; the
-// segment sums are added in a fixed order.
+// partials of Q_{ncol}^T w over this CTA's rows [r0, r1), a warp per four
+// columns: w is read once for the four, and their lane sums share one tree (6
+// FP64 adds for four columns instead of 20; at 64^3 a CTA has 14 products per
+// lane and column).  The rows are split into as many segments per group (nseg)
+// as spread the groups' segments best over the warps -- 20 groups on 32 warps
+// would leave 12 idle, and the basis streams at the rate of the loads in flight
+// -- and the segment sums are added in a fixed order.  red: NT doubles.
 template <int NT>
 __device__ __forceinline__ void pz_gemvT(const double *Q, long long ld, int ncol, const double *w, int r0,
                                          int r1, double *pt, int pstride, double *red) {
   constexpr int NW = NT / 32;
   const int wi = threadIdx.x >> 5, l = threadIdx.x & 31;
-  if (ncol >= NW) {
-    for (int j = wi; j < ncol; j += NW) {
-      const double *q = Q + (long long)j * ld;
-      double acc = 0;
-      for (int r = r0 + l; r < r1; r += 32) acc += ld_stream(q + r) * w[r];
-      for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-      if (l == 0) pt[(size_t)blockIdx.x * pstride + j] = acc;
-    }
-    return;
+  const int ng = (ncol + 3) / 4;
+  int nseg = 1, best = 0;
+  for (int q = 1; q <= 8 && q * ncol <= NT && 32 * (q - 1) < r1 - r0; q++) {
+    const int use = ng * q * 64 / ((ng * q + NW - 1) / NW);     // warps at work, in units of 1/64
+    if (use > best + 64) { best = use; nseg = q; }
   }
-  const int nseg = NW / ncol, len = (r1 - r0 + nseg - 1) / nseg;
-  if (wi < ncol * nseg) {
-    const int j = wi / nseg, sg = wi % nseg;
+  const int len = (((r1 - r0 + nseg - 1) / nseg) + 31) & ~31;
+  double *dst = nseg == 1 ? pt + (size_t)blockIdx.x * pstride : red;
+  for (int un = wi; un < ng * nseg; un += NW) {
+    const int sg = un / ng, gq = un - sg * ng, j = 4 * gq, nc = min(4, ncol - j);
     const int a = r0 + sg * len, b = min(r1, a + len);
     const double *q = Q + (long long)j * ld;
-    double acc = 0;
-    for (int r = a + l; r < b; r += 32) acc += ld_stream(q + r) * w[r];
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    if (l == 0) red[wi] = acc;
+    double acc[4] = {0, 0, 0, 0};
+#pragma unroll 2
+    for (int r = a + l; r < b; r += 32) {
+      const double wr = w[r];
+#pragma unroll
+      for (int i = 0; i < 4; i++)
+        if (i < nc) acc[i] += ld_stream(q + i * ld + r) * wr;
+    }
+    // lanes with bit 4 keep columns 1 and 3, with bit 3 columns 2 and 3
+    const bool h4 = l & 16, h3 = l & 8;
+    double s0 = (h4 ? acc[1] : acc[0]) + __shfl_xor_sync(0xffffffffu, h4 ? acc[0] : acc[1], 16);
+    double s1 = (h4 ? acc[3] : acc[2]) + __shfl_xor_sync(0xffffffffu, h4 ? acc[2] : acc[3], 16);
+    double t = (h3 ? s1 : s0) + __shfl_xor_sync(0xffffffffu, h3 ? s0 : s1, 8);
+    for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    const int ci = (h4 ? 1 : 0) + (h3 ? 2 : 0);
+    if ((l & 7) == 0 && ci < nc) dst[sg * ncol + j + ci] = t;
   }
+  if (nseg == 1) return;
   __syncthreads();
-  if (threadIdx.x < ncol) {
-    double sum = 0;
-    for (int sg = 0; sg < nseg; sg++) sum += red[threadIdx.x * nseg + sg];
-    pt[(size_t)blockIdx.x * pstride + threadIdx.x] = sum;
-  }
+  pz_fold<double>(red, nseg, ncol, ncol, [&](int c, double v) { pt[(size_t)blockIdx.x * pstride + c] = v; });
   __syncthreads();
 }
 
@@ -611,17 +746,22 @@ __device__ __forceinline__ bool pz_use32(const double *cs, int ncol, double ww0,
 // one classical Gram-Schmidt pass, and a second one when always2 or when the
 // first left less than half of ||w||^2 (the DGKS criterion; every CTA reads
 // the same partials in the same order, so all take the same branch).  ww0 is
-// this thread's share of ||w||^2 before the first pass.  Returns ||w||^2
-// after the last pass to every thread.
+// this thread's share of ||w||^2 before the first pass.  ww_out: ||w||^2 after
+// the last pass with its root and the root's inverse, in every thread.
 // The correction of each pass is formed in FP32 when pz_use32 allows it.
 template <int NT>
 __device__ __forceinline__ bool pz_cgs(const PzOp<double, double> &O, const PzLz &L, int ncol, int j0, int j1,
                                        unsigned &ep, int &slot, double *red, double *bc, double *cs, float *cs32,
-                                       bool always2, double ww0, double &ww_out, LzCount &cnt) {
+                                       bool always2, double ww0, PzScalar &ww_out, LzCount &cnt) {
+  const auto roots = [](double v) {                 // ||w|| and 1 / ||w||
+    const double b = sqrt(v);
+    return make_double2(b, 1.0 / b);
+  };
+  const int act = j1 - j0;
   double *pt = pz_buf(O, slot++);
   pz_gemvT<NT>(L.Q, L.ld, ncol, L.w, j0, j1, pt, O.pstride, red);
   __syncthreads();
-  pz_put<NT>(ww0, pt + ncol, O.pstride, red);       // column ncol: ||w||^2 before
+  pz_put<NT>(ww0, act, pt + ncol, O.pstride, red);  // column ncol: ||w||^2 before
   if (!pz_sync(O.gs, ep)) return false;
   pz_get_cols<NT, double>(pt, O.pstride, ncol + 1, nullptr, nullptr, cs, red);
   const double w0 = cs[ncol];
@@ -637,24 +777,21 @@ __device__ __forceinline__ bool pz_cgs(const PzOp<double, double> &O, const PzLz
   };
   double ww = update(w0);
   pt = pz_buf(O, slot++);
-  pz_put<NT>(ww, pt, O.pstride, red);
+  pz_put<NT>(ww, act, pt, O.pstride, red);
   if (!pz_sync(O.gs, ep)) return false;
-  ww = pz_get(pt, O.pstride, bc);
-  if (!always2 && !(ww < 0.5 * w0)) {
-    ww_out = ww;
-    return true;
-  }
+  ww_out = pz_get(pt, O.pstride, bc, roots);
+  if (!always2 && !(ww_out.sum < 0.5 * w0)) return true;
   cnt.npass2 += 1;
-  const double w1 = ww;
+  const double w1 = ww_out.sum;
   pt = pz_buf(O, slot++);
   pz_gemvT<NT>(L.Q, L.ld, ncol, L.w, j0, j1, pt, O.pstride, red);
   if (!pz_sync(O.gs, ep)) return false;
   pz_get_cols<NT, double>(pt, O.pstride, ncol, nullptr, nullptr, cs, red);
   ww = update(w1);
   pt = pz_buf(O, slot++);
-  pz_put<NT>(ww, pt, O.pstride, red);
+  pz_put<NT>(ww, act, pt, O.pstride, red);
   if (!pz_sync(O.gs, ep)) return false;
-  ww_out = pz_get(pt, O.pstride, bc);
+  ww_out = pz_get(pt, O.pstride, bc, roots);
   return true;
 }
 
@@ -737,7 +874,7 @@ __global__ void __launch_bounds__(NT, 1) k_lz_persist(PzOp<double, double> O, Pz
       acc += L.qcur[r] * wr;
     }
     double *pt = pz_buf(O, slot++);
-    pz_put<NT>(acc, pt, O.pstride, red);
+    pz_put<NT>(acc, j1 - j0, pt, O.pstride, red);
     if (!pz_sync(O.gs, ep)) return;
     const double alpha = pz_get(pt, O.pstride, bc);
     if (blockIdx.x == 0 && threadIdx.x == 0) L.al[j] = alpha;
@@ -750,11 +887,11 @@ __global__ void __launch_bounds__(NT, 1) k_lz_persist(PzOp<double, double> O, Pz
       ww0 += t * t;
     }
     __syncthreads();
-    double ww = 0;
+    PzScalar ww;
     if (!pz_cgs<NT>(O, L, j + 1, j0, j1, ep, slot, red, bc, cs, cs32, L.reorth2 != 0, ww0, ww, cnt)) return;
-    const double beta = sqrt(ww);
+    const double beta = ww.f.x;
     if (blockIdx.x == 0 && threadIdx.x == 0) L.be[j] = beta;
-    if (!(alpha == alpha) || isinf(alpha) || !(beta == beta) || isinf(beta)) {
+    if (pz_bad(alpha) || pz_bad(beta)) {
       if (nan_step < 0) nan_step = j;
       stop = true;
       break;
@@ -763,7 +900,7 @@ __global__ void __launch_bounds__(NT, 1) k_lz_persist(PzOp<double, double> O, Pz
     const bool brk = beta <= 1e-12 * (scale > 0 ? scale : 1.0);
     // q_{j+1} = w * (1 / beta): one division, then products (an FP64
     // division is about ten FP64 issue slots on this part)
-    double rdiv = 1.0 / beta;
+    double rdiv = ww.f.y;
     if (!brk) {
       scale = fmax(scale, beta);
       for (int r = j0 + threadIdx.x; r < j1; r += NT) {
@@ -781,15 +918,14 @@ __global__ void __launch_bounds__(NT, 1) k_lz_persist(PzOp<double, double> O, Pz
       for (int r = j0 + threadIdx.x; r < j1; r += NT)
         L.w[r] = d_sm64_pm1(S0.seed + (unsigned long long)restarts, (unsigned long long)ro(L.rank + r));
       __syncthreads();
-      double nn = 0;
+      PzScalar nn;
       // a restart vector's passes are counted in bytes, not as second passes
       LzCount rc{0, 0, 0.0, 0.0};
       if (!pz_cgs<NT>(O, L, j + 1, j0, j1, ep, slot, red, bc, cs, cs32, true, 0.0, nn, rc)) return;
       cnt.nfp32 += rc.nfp32;
       cnt.q64 += rc.q64;
       cnt.q32 += rc.q32;
-      const double nrm = sqrt(nn);
-      rdiv = 1.0 / nrm;
+      rdiv = nn.f.y;
       for (int r = j0 + threadIdx.x; r < j1; r += NT) {
         const double q1 = L.w[r] * rdiv;
         L.Q[(long long)(j + 1) * L.ld + r] = q1;
