@@ -148,27 +148,47 @@ __device__ __forceinline__ double *pz_buf(const PzOp<T, TU> &O, int slot) {
 // sub-partition) from shared memory, each lane several of them before its
 // shuffles, and scalars are formed by one thread and broadcast.
 
+// Four threads sum 32 values get(0..31) in the tree of a shuffle-down reduction
+// (strides 16, 8, 4, 2, 1): thread `part` holds values part + 4 t, so the first
+// three strides are its own and the last two cross the four threads.  The four
+// are consecutive lanes; the sum is valid in part 0.
+template <typename T, typename G>
+__device__ __forceinline__ T pz_tree32(int part, G get) {
+  T v[8];
+#pragma unroll
+  for (int t = 0; t < 8; t++) v[t] = get(part + 4 * t);
+#pragma unroll
+  for (int h = 4; h > 0; h >>= 1)
+#pragma unroll
+    for (int t = 0; t < h; t++) v[t] += v[t + h];
+  v[0] += __shfl_down_sync(0xffffffffu, v[0], 2, 4);
+  v[0] += __shfl_down_sync(0xffffffffu, v[0], 1, 4);
+  return v[0];
+}
+
 // CTA sum of v over the first `active` threads (the others hold none; the same
-// number in every thread), written to pt[blockIdx.x * pstride].  sm: NT + 32
-// doubles.
+// number in every thread), in the order of block_sum, written to
+// pt[blockIdx.x * pstride].  Warp k of four sums the values of warps k, k + 4,
+// ..., k + 28.  sm: NT + 32 doubles.
 template <int NT>
 __device__ __forceinline__ void pz_put(double v, int active, double *pt, int pstride, double *sm) {
+  static_assert(NT == 1024, "32 warps");
   const int cnt = min(NT, active);
   if (threadIdx.x < cnt) sm[threadIdx.x] = v;
   __syncthreads();
   if (threadIdx.x < 128) {
-    double a = 0, b = 0;
-    int i = threadIdx.x;
-    for (; i + 128 < cnt; i += 256) { a += sm[i]; b += sm[i + 128]; }
-    if (i < cnt) a += sm[i];
-    a += b;
-    for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
-    if ((threadIdx.x & 31) == 0) sm[NT + 16 + (threadIdx.x >> 5)] = a;
+    const int k = threadIdx.x >> 5, l = threadIdx.x & 31;
+    const int w = (k + 4 * (l >> 2)) * 32;
+    double a = pz_tree32<double>(l & 3, [&](int i) { return w + i < cnt ? sm[w + i] : 0.0; });
+    a += __shfl_down_sync(0xffffffffu, a, 16);
+    a += __shfl_down_sync(0xffffffffu, a, 8);
+    a += __shfl_down_sync(0xffffffffu, a, 4);
+    if (l == 0) sm[NT + 16 + k] = a;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
     const double *t = sm + NT + 16;
-    pt[(size_t)blockIdx.x * pstride] = (t[0] + t[1]) + (t[2] + t[3]);
+    pt[(size_t)blockIdx.x * pstride] = (t[0] + t[2]) + (t[1] + t[3]);
   }
 }
 
@@ -228,27 +248,33 @@ __device__ __forceinline__ void pz_fold(const T *in, int ng, int ld, int nc, F f
 
 // out[c] = (coef ? coef[c] : 1) * sum_g pt[g * pstride + c], c < ncol, in
 // precision T in shared memory; with H (ncol x ncol row-major): out = H *
-// (those sums).  Lanes run over columns (the partials are read coalesced);
-// tmp: NT values of T.
+// (those sums).  A column's sum is that of a warp whose lane j takes every 32nd
+// partial from j on before a shuffle tree, but lanes run over columns, so that
+// no FP64 instruction is spent on part of a warp and the partials are read
+// coalesced: NT / 32 columns at a time.  tmp: NT values of T.
 template <int NT, typename T>
 __device__ __forceinline__ void pz_get_cols(const double *pt, int pstride, int ncol, const T *coef, const T *H,
                                             T *out, T *tmp) {
-  const int G = (int)gridDim.x, P = min(G, max(1, NT / ncol));
-  for (int e = threadIdx.x; e < P * ncol; e += NT) {
-    const int q = e / ncol, c = e - q * ncol;
-    T a = 0, b = 0;
-    int g = q;
-    for (; g + P < G; g += 2 * P) {
-      a += T(pt[(size_t)g * pstride + c]);
-      b += T(pt[(size_t)(g + P) * pstride + c]);
+  constexpr int CW = NT / 32;                       // columns of a pass
+  const int G = (int)gridDim.x;
+  for (int c0 = 0; c0 < ncol; c0 += CW) {
+    const int w = min(CW, ncol - c0);
+    for (int e = threadIdx.x; e < 32 * w; e += NT) {
+      const int j = e / w, c = c0 + e - j * w;
+      T a = 0;
+#pragma unroll 5
+      for (int g = j; g < G; g += 32) a += T(pt[(size_t)g * pstride + c]);
+      tmp[e] = a;
     }
-    if (g < G) a += T(pt[(size_t)g * pstride + c]);
-    if (P == 1) out[c] = H ? a + b : (coef ? ro(coef + c) * (a + b) : a + b);
-    else tmp[e] = a + b;
-  }
-  __syncthreads();
-  if (P > 1) {
-    pz_fold<T>(tmp, P, ncol, ncol, [&](int c, T v) { out[c] = coef && !H ? ro(coef + c) * v : v; });
+    __syncthreads();
+    for (int c1 = 0; c1 < w; c1 += 32) {            // four threads per column
+      const int c = c1 + (threadIdx.x >> 2);
+      if (threadIdx.x < 128) {
+        const int cc = min(c, w - 1);
+        const T v = pz_tree32<T>(threadIdx.x & 3, [&](int j) { return tmp[j * w + cc]; });
+        if (c < w && (threadIdx.x & 3) == 0) out[c0 + c] = coef && !H ? ro(coef + c0 + c) * v : v;
+      }
+    }
     __syncthreads();
   }
   if (H) {
@@ -637,50 +663,70 @@ struct LzCount {
   double q64, q32;
 };
 
-// partials of Q_{ncol}^T w over this CTA's rows [r0, r1), a warp per four
-// columns: w is read once for the four, and their lane sums share one tree (6
-// FP64 adds for four columns instead of 20; at 64^3 a CTA has 14 products per
-// lane and column).  The rows are split into as many segments per group (nseg)
-// as spread the groups' segments best over the warps -- 20 groups on 32 warps
-// would leave 12 idle, and the basis streams at the rate of the loads in flight
-// -- and the segment sums are added in a fixed order.  red: NT doubles.
+// partials of Q_{ncol}^T w over this CTA's rows [r0, r1).  A column's sum is a
+// warp's: lanes stride the rows, then a shuffle-down tree.  Below kPzWideRows
+// rows a warp takes four columns at once (w is read once for the four, and their
+// trees share 6 FP64 adds instead of 20: at 64^3 a CTA has 14 products per lane
+// and column); above, one column per warp keeps all warps' loads in flight (at
+// 128^3, 4,050 rows a CTA, four columns a warp took the setup from 53 to 63 ms).
+// With fewer columns than warps the rows are split into nseg segments per column
+// so every warp works; the segment sums are added in a fixed order.  The sums
+// are the same in every form.  red: NT doubles.
+constexpr int kPzWideRows = 1024;
 template <int NT>
 __device__ __forceinline__ void pz_gemvT(const double *Q, long long ld, int ncol, const double *w, int r0,
                                          int r1, double *pt, int pstride, double *red) {
   constexpr int NW = NT / 32;
   const int wi = threadIdx.x >> 5, l = threadIdx.x & 31;
-  const int ng = (ncol + 3) / 4;
-  int nseg = 1, best = 0;
-  for (int q = 1; q <= 8 && q * ncol <= NT && 32 * (q - 1) < r1 - r0; q++) {
-    const int use = ng * q * 64 / ((ng * q + NW - 1) / NW);     // warps at work, in units of 1/64
-    if (use > best + 64) { best = use; nseg = q; }
+  if (ncol >= NW && r1 - r0 < kPzWideRows) {
+    for (int j = 4 * wi; j < ncol; j += 4 * NW) {
+      const int nc = min(4, ncol - j);
+      const double *q = Q + (long long)j * ld;
+      double acc[4] = {0, 0, 0, 0};
+#pragma unroll 2
+      for (int r = r0 + l; r < r1; r += 32) {
+        const double wr = w[r];
+#pragma unroll
+        for (int i = 0; i < 4; i++)
+          if (i < nc) acc[i] += ld_stream(q + i * ld + r) * wr;
+      }
+      // lanes with bit 4 keep columns 1 and 3, with bit 3 columns 2 and 3
+      const bool h4 = l & 16, h3 = l & 8;
+      double s0 = (h4 ? acc[1] : acc[0]) + __shfl_xor_sync(0xffffffffu, h4 ? acc[0] : acc[1], 16);
+      double s1 = (h4 ? acc[3] : acc[2]) + __shfl_xor_sync(0xffffffffu, h4 ? acc[2] : acc[3], 16);
+      double t = (h3 ? s1 : s0) + __shfl_xor_sync(0xffffffffu, h3 ? s0 : s1, 8);
+      for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      const int ci = (h4 ? 1 : 0) + (h3 ? 2 : 0);
+      if ((l & 7) == 0 && ci < nc) pt[(size_t)blockIdx.x * pstride + j + ci] = t;
+    }
+    return;
   }
-  const int len = (((r1 - r0 + nseg - 1) / nseg) + 31) & ~31;
-  double *dst = nseg == 1 ? pt + (size_t)blockIdx.x * pstride : red;
-  for (int un = wi; un < ng * nseg; un += NW) {
-    const int sg = un / ng, gq = un - sg * ng, j = 4 * gq, nc = min(4, ncol - j);
+  if (ncol >= NW) {
+    for (int j = wi; j < ncol; j += NW) {
+      const double *q = Q + (long long)j * ld;
+      double acc = 0;
+      for (int r = r0 + l; r < r1; r += 32) acc += ld_stream(q + r) * w[r];
+      for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+      if (l == 0) pt[(size_t)blockIdx.x * pstride + j] = acc;
+    }
+    return;
+  }
+  const int nseg = NW / ncol, len = (r1 - r0 + nseg - 1) / nseg;
+  if (wi < ncol * nseg) {
+    const int j = wi / nseg, sg = wi % nseg;
     const int a = r0 + sg * len, b = min(r1, a + len);
     const double *q = Q + (long long)j * ld;
-    double acc[4] = {0, 0, 0, 0};
-#pragma unroll 2
-    for (int r = a + l; r < b; r += 32) {
-      const double wr = w[r];
-#pragma unroll
-      for (int i = 0; i < 4; i++)
-        if (i < nc) acc[i] += ld_stream(q + i * ld + r) * wr;
-    }
-    // lanes with bit 4 keep columns 1 and 3, with bit 3 columns 2 and 3
-    const bool h4 = l & 16, h3 = l & 8;
-    double s0 = (h4 ? acc[1] : acc[0]) + __shfl_xor_sync(0xffffffffu, h4 ? acc[0] : acc[1], 16);
-    double s1 = (h4 ? acc[3] : acc[2]) + __shfl_xor_sync(0xffffffffu, h4 ? acc[2] : acc[3], 16);
-    double t = (h3 ? s1 : s0) + __shfl_xor_sync(0xffffffffu, h3 ? s0 : s1, 8);
-    for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    const int ci = (h4 ? 1 : 0) + (h3 ? 2 : 0);
-    if ((l & 7) == 0 && ci < nc) dst[sg * ncol + j + ci] = t;
+    double acc = 0;
+    for (int r = a + l; r < b; r += 32) acc += ld_stream(q + r) * w[r];
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+    if (l == 0) red[wi] = acc;
   }
-  if (nseg == 1) return;
   __syncthreads();
-  pz_fold<double>(red, nseg, ncol, ncol, [&](int c, double v) { pt[(size_t)blockIdx.x * pstride + c] = v; });
+  if (threadIdx.x < ncol) {
+    double sum = 0;
+    for (int sg = 0; sg < nseg; sg++) sum += red[threadIdx.x * nseg + sg];
+    pt[(size_t)blockIdx.x * pstride + threadIdx.x] = sum;
+  }
   __syncthreads();
 }
 
