@@ -93,7 +93,8 @@ struct ddlr_ctx {
     float *cb32[5] = {nullptr};
     double *part64 = nullptr;
     float *part32 = nullptr;
-    double *fpart = nullptr;   // per-64-row-block column partials of the fused step kernels
+    double *fpart = nullptr;   // column partials of the step kernels (per 64-row block, per sub-range)
+    unsigned *count = nullptr; // arrival counter of their reductions (0 between launches)
     PcgStateMR *st = nullptr;
     struct G {
       cudaGraphExec_t exec = nullptr;
@@ -2713,7 +2714,9 @@ void batch_alloc(ddlr_ctx *c, int R) {
     B.part32 = (float *)al((size_t(kTcRedGrid) + 1) * std::max<size_t>(k * R, 2 * R) * 4);
   }
   B.part64 = (double *)al(size_t(kRedGrid) * std::max<size_t>(k * R, 2 * R) * 8);
-  B.fpart = (double *)al(size_t((P.n + kFbRows - 1) / kFbRows) * R * 8);
+  B.fpart = (double *)al(std::max(size_t((P.n + kFbRows - 1) / kFbRows), size_t(2 * kRedGrid * kDotSub)) * R * 8);
+  B.count = (unsigned *)al(16);
+  ck(cudaMemsetAsync(B.count, 0, 16, c->stream), "memset");
   if (c->opt.c_solver == 1)
     for (int i = 0; i < 5; i++) {
       B.cb64[i] = (double *)al(nR * 8);
@@ -2985,42 +2988,101 @@ void batch_autotune(ddlr_ctx *c, int R) {
   B.tuned = true;
 }
 
-void pcg_mr_iteration(ddlr_ctx *c, int R, int flexible) {
+// The preconditioner inside the block PCG reads in = TI(d .* r) (formed by the
+// update of r) and leaves Z in its own precision, unscaled; the kernels that use
+// z = d .* Z scale it as they read it.
+template <typename T>
+struct MrPrec {
+  T *in, *z;                             // in == nullptr: it reads Rr
+};
+template <typename T>
+MrPrec<T> mr_prec(ddlr_ctx *c);
+template <>
+MrPrec<double> mr_prec<double>(ddlr_ctx *c) {
+  return {c->dsc_dev ? c->bt.S : nullptr, c->bt.Z};
+}
+template <>
+MrPrec<float> mr_prec<float>(ddlr_ctx *c) {
+  return {c->bt.w32[5], c->bt.w32[6]};
+}
+const int *mr_gate(ddlr_ctx *c) {
+  return reinterpret_cast<const int *>(reinterpret_cast<const char *>(c->bt.st) + offsetof(PcgStateMR, all_done));
+}
+// launch shape of the row-block kernels
+struct FbShape {
+  unsigned nb, grid, threads;
+  FbShape(const ddlr_ctx *c, int R) {
+    nb = (unsigned)((c->P.n + kFbRows - 1) / kFbRows);
+    grid = (nb + fb_groups(R) - 1) / fb_groups(R);
+    threads = unsigned(fb_groups(R) * kFbLanes * R);
+  }
+};
+template <MrStep S>
+void mr_reduce(ddlr_ctx *c, int rows, int no, const int *gate) {
+  KL(c, "pcg_mr_red", c->stream, k_reduce_step_mr<S>, kRedGrid, kMrRedNT, 0, rows, no, c->bt.fpart, c->bt.part64,
+     c->bt.st, c->bt.count, gate);
+}
+inline void mr_apply_prec(ddlr_ctx *c, const double *in, double *z, int R, const int *gate) {
+  apply_mr<double, double>(c, c->U64, in, z, R, gate);
+}
+inline void mr_apply_prec(ddlr_ctx *c, const float *in, float *z, int R, const int *gate) {
+  if (c->opt.uk_bf16) apply_mr<float, __nv_bfloat16>(c, c->Ub16, in, z, R, gate);
+  else apply_mr<float, float>(c, c->U32, in, z, R, gate);
+}
+
+// z = M^-1 r, the dot products with their scalar step, p = z + beta p; flex:
+// the flexible CG's z_old
+template <typename T, MrStep S>
+void mr_precond_p(ddlr_ctx *c, int R, bool flex, const int *gate) {
   auto &B = c->bt;
   const int n = c->P.n;
   const long long nR = (long long)n * R;
-  const int bd = B.bd_elem;
-  const int *gate = reinterpret_cast<const int *>(reinterpret_cast<const char *>(B.st) +
-                                                  offsetof(PcgStateMR, all_done));
-  double *part = B.part64;
-  // q = A p with the p.q partials, and the x, r update with the r.r partials,
-  // in one pass each (64-row blocks, then the blocks of each reduction range)
-  const unsigned nb = (unsigned)((n + kFbRows - 1) / kFbRows);
-  const int fg = fb_groups(R);
-  const unsigned fgrid = (nb + fg - 1) / fg, fthreads = unsigned(fg * kFbLanes * R);
-  KL(c, "spmv_mr", c->stream, k_spmv_pq_mr, fgrid, fthreads, 0, n, c->a_soff, c->a_sw, c->a_col, c->a_val, B.P,
+  const MrPrec<T> M = mr_prec<T>(c);
+  const FbShape F(c, R);
+  const T *in = M.in;
+  if constexpr (std::is_same<T, double>::value)
+    if (!in) in = B.Rr;
+  mr_apply_prec(c, in, M.z, R, gate);
+  double *zo = flex ? B.Zo : nullptr;
+  constexpr int units = kRedGrid * kDotSub;
+  KL(c, "pcg_mr_dot", c->stream, k_dot_rz_mr<T>, (units + fb_groups(R) - 1) / fb_groups(R), F.threads, 0,
+     (long long)n, R, B.Rr, M.z, S == kMrBeta ? zo : (const double *)nullptr, c->dsc_dev, B.fpart, gate);
+  mr_reduce<S>(c, units, S == kMrBeta && zo ? 2 * R : R, gate);
+  KL(c, "pcg_mr_p", c->stream, k_pcgmr_p<T>, eblk((nR + kMrPUnr - 1) / kMrPUnr, 256), 256, 0, (long long)n, B.st, M.z, c->dsc_dev,
+     B.P, zo);
+}
+
+template <typename T>
+void pcg_mr_iteration_t(ddlr_ctx *c, int R, int flexible) {
+  auto &B = c->bt;
+  const int n = c->P.n;
+  const long long nR = (long long)n * R;
+  const int *gate = mr_gate(c);
+  const MrPrec<T> M = mr_prec<T>(c);
+  // q = A p with the p.q partials, and the x, r update with the r.r partials
+  // and the preconditioner's input, in one pass each (64-row blocks, then the
+  // blocks of each reduction range and the scalar step)
+  const FbShape F(c, R);
+  KL(c, "spmv_mr", c->stream, k_spmv_pq_mr, F.grid, F.threads, 0, n, c->a_soff, c->a_sw, c->a_col, c->a_val, B.P,
      B.Q, R, B.fpart, gate);
-  KL(c, "pcg_mr_red", c->stream, k_fused_partials_reduce, kRedGrid, 64, 0, (int)nb, R, B.fpart, part, gate);
-  KL(c, "pcg_mr_scalar", c->stream, k_pcgmr_alpha, 1, kScalarThreads, 0, B.st, part, kRedGrid);
-  KL(c, "pcg_mr_axpy", c->stream, k_update_rr_mr, fgrid, fthreads, 0, (long long)n, B.st, B.P, B.Q, B.X, B.Rr,
-     B.fpart);
-  KL(c, "pcg_mr_red", c->stream, k_fused_partials_reduce, kRedGrid, 64, 0, (int)nb, R, B.fpart, part, gate);
-  KL(c, "pcg_mr_scalar", c->stream, k_pcgmr_rr, 1, kScalarThreads, 0, B.st, part, kRedGrid);
-  // the check kernels run on a bounded grid: most iterations they return at once
-  const unsigned gchk = (unsigned)std::min<long long>(eblk(nR, bd), 152LL * 8);
-  KL(c, "pcg_mr_check", c->stream, k_pcgmr_true_res, gchk, bd, 0, n, B.st, c->a_soff, c->a_sw, c->a_col, c->a_val,
-     B.B, B.X, B.T);
-  // T.T only when a column's true residual is checked this iteration
-  const int *gate_chk = reinterpret_cast<const int *>(reinterpret_cast<const char *>(B.st) +
-                                                      offsetof(PcgStateMR, no_check));
-  KL(c, "pcg_mr_dot", c->stream, k_dot_mr_partial, kRedGrid, 256, 0, (long long)n, R, B.T, B.T, (const double *)nullptr, part,
-     gate_chk);
-  KL(c, "pcg_mr_scalar", c->stream, k_pcgmr_true_dec, 1, kScalarThreads, 0, B.st, part, kRedGrid);
-  KL(c, "pcg_mr_check", c->stream, k_pcgmr_copy_r, gchk, bd, 0, (long long)n, B.st, B.T, B.Rr);
-  precond_mr(c, B.Rr, B.Z, R, gate);
-  KL(c, "pcg_mr_dot", c->stream, k_dot_mr_partial, kRedGrid, 256, 0, (long long)n, R, B.Rr, B.Z, flexible ? B.Zo : B.Z, part, gate);
-  KL(c, "pcg_mr_scalar", c->stream, k_pcgmr_beta, 1, kScalarThreads, 0, B.st, part, kRedGrid);
-  KL(c, "pcg_mr_p", c->stream, k_pcgmr_p, eblk(nR, bd), bd, 0, (long long)n, B.st, B.Z, B.P, flexible ? B.Zo : (double *)nullptr);
+  mr_reduce<kMrAlpha>(c, int(F.nb), R, gate);
+  KL(c, "pcg_mr_axpy", c->stream, k_update_rr_mr<T>, F.grid, F.threads, 0, (long long)n, B.st, B.P, B.Q, B.X, B.Rr,
+     c->dsc_dev, M.in, B.fpart);
+  mr_reduce<kMrRr>(c, int(F.nb), R, gate);
+  // the check kernels run on a small grid: most iterations they return at once
+  // (1,216 CTAs took 17 us to do so, 304 take 3)
+  const unsigned gchk = (unsigned)std::min<long long>(eblk(nR, 256), 2 * 152);
+  KL(c, "pcg_mr_check", c->stream, k_pcgmr_true_res, std::min(F.grid, 2 * 152u), F.threads, 0, n, B.st, c->a_soff,
+     c->a_sw, c->a_col, c->a_val, B.B, B.X, B.T, B.fpart);
+  mr_reduce<kMrDec>(c, int(F.nb), R, gate);
+  KL(c, "pcg_mr_check", c->stream, k_pcgmr_copy_r<T>, gchk, 256, 0, (long long)n, B.st, B.T, B.Rr, c->dsc_dev,
+     M.in);
+  mr_precond_p<T, kMrBeta>(c, R, flexible != 0, gate);
+}
+
+void pcg_mr_iteration(ddlr_ctx *c, int R, int flexible) {
+  if (c->opt.precision == 0) pcg_mr_iteration_t<double>(c, R, flexible);
+  else pcg_mr_iteration_t<float>(c, R, flexible);
 }
 
 // the captured graph of one batched iteration of width R on c->stream (a
@@ -3067,8 +3129,7 @@ void pcg_mr_dev(ddlr_ctx *c, int R, double tol, int maxit, ddlr_solve_info *info
   const int n = c->P.n;
   const long long nR = (long long)n * R;
   const int flexible = c->opt.precision == 1 ? 1 : 0;
-  const int *gate = reinterpret_cast<const int *>(reinterpret_cast<const char *>(B.st) +
-                                                  offsetof(PcgStateMR, all_done));
+  const int *gate = mr_gate(c);
   const char *ng = getenv("DDLR_NO_GRAPH");
   const bool use_graph = !c->timing && !(ng && ng[0] == '1');
   cudaStream_t user = c->stream;
@@ -3089,11 +3150,17 @@ void pcg_mr_dev(ddlr_ctx *c, int R, double tol, int maxit, ddlr_solve_info *info
   ck(cudaMemcpyAsync(B.Rr, B.B, sizeof(double) * nR, cudaMemcpyDeviceToDevice, c->stream), "copy");
   KL(c, "pcg_mr", c->stream, k_dot_mr_partial, kRedGrid, 256, 0, (long long)n, R, B.B, B.B, (const double *)nullptr, part, (const int *)nullptr);
   KL(c, "pcg_mr", c->stream, k_pcgmr_init, 1, kScalarThreads, 0, B.st, part, kRedGrid, R, tol, maxit, flexible);
-  precond_mr(c, B.Rr, B.Z, R, gate);
-  KL(c, "pcg_mr", c->stream, k_dot_mr_partial, kRedGrid, 256, 0, (long long)n, R, B.Rr, B.Z, (const double *)nullptr, part, gate);
-  KL(c, "pcg_mr", c->stream, k_pcgmr_rz0, 1, kScalarThreads, 0, B.st, part, kRedGrid);
-  ck(cudaMemcpyAsync(B.P, B.Z, sizeof(double) * nR, cudaMemcpyDeviceToDevice, c->stream), "copy");
-  ck(cudaMemcpyAsync(B.Zo, B.Z, sizeof(double) * nR, cudaMemcpyDeviceToDevice, c->stream), "copy");
+  // z = M^-1 b, rz = b.z, p = z (beta = 0 on a zero p)
+  ck(cudaMemsetAsync(B.P, 0, sizeof(double) * nR, c->stream), "memset");
+  if (c->opt.precision == 0) {
+    if (c->dsc_dev)
+      KL(c, "vec_mr", c->stream, k_scale_rows_mr, eblk(nR, bd), bd, 0, (long long)n, R, c->dsc_dev, B.Rr, B.S, gate);
+    mr_precond_p<double, kMrRz0>(c, R, false, gate);
+  } else {
+    KL(c, "vec_mr", c->stream, (k_scale_cast_mr<float, double>), eblk((nR + 3) / 4, 256), 256, 0, (long long)n, R,
+       c->dsc_dev, B.Rr, B.w32[5], gate);
+    mr_precond_p<float, kMrRz0>(c, R, true, gate);
+  }
   if (use_graph) mr_graph(c, R, flexible);
   const int batch = 4;
   for (int it = 0; it < maxit + batch; it += batch) {
@@ -4068,10 +4135,11 @@ ddlr_status ddlr_get_traffic(ddlr_handle c, double *apply_bytes, double *a0_byte
       else if (f == "e_int_mr") b = ne * (v + 4.0) + 4.0 * m + 2.0 * m * R * v;
       else if (f == "u_add_mr") b = n * k * ub + 2.0 * n * R * v;
       else if (f == "spmv_mr") b = nnz_a * 12.0 + 2.0 * n * R * 8.0;
-      else if (f == "pcg_mr_dot") b = 2.0 * n * R * 8.0;
+      // (z in the preconditioner's precision; z_old too for flexible CG)
+      else if (f == "pcg_mr_dot") b = n * R * (8.0 + v + (c->opt.precision == 1 ? 8.0 : 0.0));
       else if (f == "pcg_mr_red") b = (std::ceil(n / kFbRows) + kRedGrid) * R * 8.0;
-      else if (f == "pcg_mr_axpy") b = 6.0 * n * R * 8.0;
-      else if (f == "pcg_mr_p") b = (c->opt.precision == 1 ? 4.0 : 3.0) * n * R * 8.0;
+      else if (f == "pcg_mr_axpy") b = n * R * (48.0 + (c->opt.precision == 1 || c->dsc_dev ? v : 0.0));
+      else if (f == "pcg_mr_p") b = n * R * (16.0 + v + (c->opt.precision == 1 ? 8.0 : 0.0));
       else if (f == "vec_mr") b = n * R * (8.0 + v) + (c->dsc_dev ? 8.0 * n : 0.0);
       else if (f == "lanczos_persist") b = c->pz_lz_runs ? c->pz_lz_bytes / double(c->pz_lz_runs) : 0.0;
       family_bytes[i] = b;

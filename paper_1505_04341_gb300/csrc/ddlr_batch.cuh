@@ -773,11 +773,51 @@ struct PcgStateMR {
   int pad[2];
 };
 
+// Binary64 <-> binary32 conversions written out on the bit patterns (IEEE 754:
+// rounding to nearest, ties to even, for results in the normal binary32 range;
+// widening is exact), in integer instructions.  On this part the hardware
+// conversions issue to the FP64 pipe, which the scaling multiply already
+// occupies; the streaming cast kernels were bound by that pipe.  Zeros,
+// subnormal results, overflow, infinities and NaNs take the hardware
+// conversion.
+// The hardware conversions sit behind calls: inlined, the compiler turns the
+// tests into predicated or selected conversions, which still take FP64 slots.
+__device__ __noinline__ float f64_to_f32_rare(double x) { return __double2float_rn(x); }
+__device__ __noinline__ double f32_to_f64_rare(float v) { return double(v); }
+__device__ __forceinline__ float f64_to_f32_rn(double x) {
+  const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(x));
+  const unsigned hi = unsigned(b >> 32);
+  const unsigned e = (hi >> 20) & 0x7ffu;            // binary64 biased exponent
+  if (e >= 897u && e <= 1150u) {                      // binary32 biased exponent e - 896 in [1, 254]
+    const unsigned long long m = b & 0x000fffffffffffffull;
+    unsigned f = ((e - 896u) << 23) | unsigned(m >> 29);
+    const unsigned rest = unsigned(m & 0x1fffffffull);   // the 29 bits dropped
+    if (rest > 0x10000000u || (rest == 0x10000000u && (f & 1u))) f += 1u;   // a carry moves to the exponent
+    return __uint_as_float(f | (hi & 0x80000000u));
+  }
+  return f64_to_f32_rare(x);
+}
+__device__ __forceinline__ double f32_to_f64(float v) {
+  const unsigned u = __float_as_uint(v);
+  const unsigned e = (u >> 23) & 0xffu;
+  if (e != 0u && e != 255u) {
+    const unsigned long long b = (static_cast<unsigned long long>(u & 0x80000000u) << 32) |
+                                 (static_cast<unsigned long long>(e + 896u) << 52) |
+                                 (static_cast<unsigned long long>(u & 0x7fffffu) << 29);
+    return __longlong_as_double(static_cast<long long>(b));
+  }
+  return f32_to_f64_rare(v);
+}
+__device__ __forceinline__ double to_f64(float v) { return f32_to_f64(v); }
+__device__ __forceinline__ double to_f64(double v) { return v; }
+__device__ __forceinline__ void from_f64(double x, float &o) { o = f64_to_f32_rn(x); }
+__device__ __forceinline__ void from_f64(double x, double &o) { o = x; }
+
 // ---- fused step kernels of the block PCG with their column dot products.
 // Rows are taken in blocks of kFbRows = 64; in a block, row lane l (of 8)
 // takes rows l, l + 8, ... of the block in order, a thread owns one (row
 // lane, column) pair, and the 8 lane sums of a column are added in lane order
-// into partials[block][q].  k_fused_partials_reduce then adds the blocks of each
+// into partials[block][q].  k_reduce_step_mr then adds the blocks of each
 // of the G = kRedGrid reduction ranges in order into the [g][2R] layout the
 // scalar kernels read.  Nothing in this order depends on R, so a column's dot
 // products are the same in every batch.  Launch: a CTA takes fb_groups(R)
@@ -825,10 +865,13 @@ __global__ void k_spmv_pq_mr(int n, const int *__restrict__ soff, const int *__r
   }
 }
 
-// X += alpha P; Rr -= alpha Q for the running columns, and the column
-// partials of Rr.Rr (all columns)
+// X += alpha P; Rr -= alpha Q for the running columns, the column partials of
+// Rr.Rr (all columns), and the preconditioner's input in = TI(d_r r) of every
+// column (in == nullptr: it reads Rr itself): one pass instead of a second read
+// of r by a scaling kernel (96^3 x 32, FP32 input: 208 + 106 -> 246 us).
+template <typename TI>
 __global__ void k_update_rr_mr(long long n, const PcgStateMR *st, const double *P, const double *Q, double *X,
-                               double *Rr, double *bpart) {
+                               double *Rr, const double *d, TI *in, double *bpart) {
   if (st->all_done) return;
   __shared__ double red[kFbMaxRed];
   const int R = st->R;
@@ -851,6 +894,7 @@ __global__ void k_update_rr_mr(long long n, const PcgStateMR *st, const double *
         rv -= a * Q[e];
         Rr[e] = rv;
       }
+      if (in) from_f64(d ? rv * d[r] : rv, in[e]);
       acc = fma(rv, rv, acc);
     }
   }
@@ -863,20 +907,66 @@ __global__ void k_update_rr_mr(long long n, const PcgStateMR *st, const double *
   }
 }
 
-// partials[g][q] (stride 2R) = sum over the blocks of reduction range g, in
-// order, of bpart[block][q]; grid kRedGrid, R threads
-__global__ void k_fused_partials_reduce(int nblocks, int R, const double *bpart, double *partials,
-                                        const int *gate) {
+// Column partials of Rr.z and (Zo) Rr.z_old, z = d .* Z as the preconditioner
+// left it (d == nullptr: Z), in the order of k_dot_mr_partial: the rows in
+// kRedGrid ranges of 8 sub-ranges, a sub-range's rows in eight interleaved sums
+// combined in a fixed tree.  bpart[range * 8 + sub-range][no], no = R or 2 R;
+// k_reduce_step_mr adds the sub-ranges in order.  A thread per (interleaved sum,
+// column) instead of per column: eight times the threads, and no idle lanes for
+// narrow blocks.  z is scaled here and in k_pcgmr_p instead of in a pass of its
+// own that wrote it out in FP64.  96^3 x 32, mixed: casting back, products and p
+// 106 + 210 + 147 us -> products and p 178 + 132 us.
+constexpr int kDotSub = 8;
+template <typename TZ>
+__global__ void __launch_bounds__(kFbMaxRed, 2)
+k_dot_rz_mr(long long n, int R, const double *Rr, const TZ *Z, const double *Zo, const double *d, double *bpart,
+            const int *gate) {
   if (gate && *gate) return;
-  const int q = threadIdx.x;
-  if (q >= R) return;
-  long long b0, b1;
-  red_range(nblocks, blockIdx.x, gridDim.x, b0, b1);
-  double v = 0.0;
-  for (long long b = b0; b < b1; b++) v += bpart[b * R + q];
-  partials[(long long)blockIdx.x * 2 * R + q] = v;
+  __shared__ double red[2 * kFbMaxRed];
+  const int gt = kFbLanes * R, gi = threadIdx.x / gt, tt = threadIdx.x % gt;
+  const int q = tt % R, l = tt / R;
+  const int unit = blockIdx.x * fb_groups(R) + gi;
+  const bool live = unit < kRedGrid * kDotSub;
+  double a1 = 0.0, a2 = 0.0;
+  if (live) {
+    long long g0, g1;
+    red_range(n, unit / kDotSub, kRedGrid, g0, g1);
+    const long long sub = (g1 - g0 + kDotSub - 1) / kDotSub;
+    const long long r0 = min(g1, g0 + (unit % kDotSub) * sub), r1 = min(g1, r0 + sub);
+    constexpr int U = 4;
+    for (long long rb = r0 + l; rb < r1; rb += U * kFbLanes) {
+      double rv[U], ov[U], dv[U];
+      TZ zv[U];
+#pragma unroll
+      for (int u = 0; u < U; u++) {
+        const long long r = rb + u * kFbLanes, e = r * R + q;
+        if (r < r1) {
+          rv[u] = Rr[e];
+          zv[u] = Z[e];
+          if (Zo) ov[u] = Zo[e];
+          if (d) dv[u] = d[r];
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < U; u++) {
+        if (rb + u * kFbLanes >= r1) break;
+        const double z = d ? __dmul_rn(to_f64(zv[u]), dv[u]) : to_f64(zv[u]);
+        a1 = fma(rv[u], z, a1);
+        if (Zo) a2 = fma(rv[u], ov[u], a2);
+      }
+    }
+  }
+  double *mine = red + (gi * kFbLanes + l) * R + q;
+  mine[0] = a1;
+  if (Zo) mine[kFbMaxRed] = a2;
+  __syncthreads();
+  const int no = Zo ? 2 * R : R;
+  if (l < (Zo ? 2 : 1) && live) {
+    const double *t = red + l * kFbMaxRed + gi * kFbLanes * R + q;
+    bpart[(long long)unit * no + l * R + q] =
+        ((t[0] + t[R]) + (t[2 * R] + t[3 * R])) + ((t[4 * R] + t[5 * R]) + (t[6 * R] + t[7 * R]));
+  }
 }
-
 
 // sums[o] = sum over the G partial rows of column o (o < no), a warp per
 // column: lanes take every 32nd partial in order, then a shuffle tree (a
@@ -887,7 +977,8 @@ __device__ __forceinline__ void col_sums(const double *partials, int G, int R, i
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
   for (int o = w; o < no; o += nw) {
     double v = 0;
-    for (int g = l; g < G; g += 32) v += partials[(long long)g * 2 * R + o];
+#pragma unroll 10
+    for (int g = l; g < G; g += 32) v += __ldcg(partials + (long long)g * 2 * R + o);
     for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
     if (l == 0) sums[o] = v;
   }
@@ -918,141 +1009,208 @@ __global__ void k_pcgmr_init(PcgStateMR *st, const double *partials, int G, int 
   }
 }
 
-__global__ void k_pcgmr_rz0(PcgStateMR *st, const double *partials, int G) {
-  if (st->all_done) return;
-  const int q = threadIdx.x, R = st->R;
-  __shared__ double sm[kMaxR];
-  col_sums(partials, G, R, R, sm);
-  if (q < R && !st->done[q]) {
-    const double s = sm[q];
-    st->rz[q] = s;
-    if (!(s == s) || isinf(s)) { st->status[q] = 7; st->done[q] = 1; }
-  }
-}
+// ---- the scalar step that follows a column reduction, by the CTA that finishes
+// it (sums: the column sums in shared memory; every thread calls it)
+enum MrStep { kMrRz0, kMrAlpha, kMrRr, kMrDec, kMrBeta };
 
-__global__ void k_pcgmr_alpha(PcgStateMR *st, const double *partials, int G) {
-  if (st->all_done) return;
-  const int q = threadIdx.x, R = st->R;
-  __shared__ double sm[kMaxR];
-  col_sums(partials, G, R, R, sm);
-  if (q < R) {
-    double a = 0.0;
-    if (!st->done[q] && !st->fresh[q]) {
-      const double pq = sm[q];
-      st->pq[q] = pq;
-      a = st->rz[q] / pq;
-      if (!(a == a) || isinf(a)) { st->status[q] = 7; st->done[q] = 1; a = 0.0; }
-    }
-    st->alpha[q] = a;
-  }
-}
-
-
-__global__ void k_pcgmr_rr(PcgStateMR *st, const double *partials, int G) {
-  if (st->all_done) return;
-  const int q = threadIdx.x, R = st->R;
-  __shared__ int anyc;
-  __shared__ double sm[kMaxR];
-  if (q == 0) anyc = 0;
-  col_sums(partials, G, R, R, sm);
-  if (q < R && !st->done[q] && !st->fresh[q]) {
-    const double rr = sm[q];
-    st->rr[q] = rr;
-    st->its[q] += 1;
-    if (!(rr == rr) || isinf(rr)) { st->status[q] = 7; st->done[q] = 1; }
-    else {
-      st->check[q] = (rr <= st->tol2[q]) ? 1 : 0;
-      if (st->check[q]) atomicOr(&anyc, 1);
-      else if (st->its[q] >= st->maxit) { st->status[q] = 5; st->done[q] = 1; }
-    }
-  }
+__device__ __forceinline__ void mr_all_done(PcgStateMR *st) {
   __syncthreads();
-  if (q == 0) { st->any_check = anyc; st->no_check = anyc ? 0 : 1; }
-}
-
-// T = B - A X for the columns whose true residual is to be checked
-__global__ void k_pcgmr_true_res(int n, const PcgStateMR *st, const int *soff, const int *sw,
-                                 const int *col, const double *val, const double *B,
-                                 const double *X, double *Tt) {
-  if (st->all_done || !st->any_check) return;
-  const int R = st->R;
-  for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < (long long)n * R;
-       idx += (long long)gridDim.x * blockDim.x) {
-    const long long r = row_of(idx, R);
-    const int q = col_of(idx, r, R);
-    if (!st->check[q]) continue;
-    const int g = int(r >> 5), l = int(r & 31);
-    const int off = soff[g] + l, w = sw[g];
-    double ax = 0;
-    for (int kk = 0; kk < w; kk++) ax += val[off + kk * 32] * X[(long long)col[off + kk * 32] * R + q];
-    Tt[idx] = B[idx] - ax;
-  }
-}
-
-__global__ void k_pcgmr_true_dec(PcgStateMR *st, const double *partials, int G) {
-  const int q = threadIdx.x, R = st->R;
-  if (q == 0) st->no_check = 1;   // the check of this iteration is consumed here
-  if (st->all_done || !st->any_check) return;
-  __shared__ double sm[kMaxR];
-  col_sums(partials, G, R, R, sm);
-  if (q < R && st->check[q] && !st->done[q]) {
-    const double rt2 = sm[q];
-    st->rt2[q] = rt2;
-    if (rt2 <= st->tol2[q]) { st->status[q] = 0; st->done[q] = 1; }
-    else {
-      st->restart[q] = 1;
-      if (st->its[q] >= st->maxit) { st->status[q] = 5; st->done[q] = 1; }
-    }
-  }
-  if (q < R) st->check[q] = 0;
-}
-
-// (a restart is only ever set by a true-residual check of this iteration)
-__global__ void k_pcgmr_copy_r(long long n, const PcgStateMR *st, const double *Tt, double *Rr) {
-  if (st->all_done || !st->any_check) return;
-  const int R = st->R;
-  for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < n * R;
-       idx += (long long)gridDim.x * blockDim.x) {
-    const int q = col_of(idx, row_of(idx, R), R);
-    if (st->restart[q] && !st->done[q]) Rr[idx] = Tt[idx];
-  }
-}
-
-__global__ void k_pcgmr_beta(PcgStateMR *st, const double *partials, int G) {
-  if (st->all_done) return;
-  const int q = threadIdx.x, R = st->R;
-  __shared__ double sm[2 * kMaxR];
-  col_sums(partials, G, R, 2 * R, sm);
-  if (q < R && !st->done[q]) {
-    const double rzn = sm[q];
-    const double rzo = sm[R + q];
-    double beta = st->flexible ? (rzn - rzo) / st->rz[q] : rzn / st->rz[q];
-    if (st->restart[q] || st->fresh[q]) beta = 0.0;
-    st->beta[q] = beta;
-    st->rz[q] = rzn;
-    st->restart[q] = 0;
-    st->fresh[q] = 0;
-    if (!(rzn == rzn) || isinf(rzn)) { st->status[q] = 7; st->done[q] = 1; }
-  }
-  __syncthreads();
-  if (q == 0) {
+  if (threadIdx.x == 0) {
     int all = 1;
-    for (int c = 0; c < R; c++) all &= st->done[c];
+    for (int c = 0; c < st->R; c++) all &= st->done[c];
     st->all_done = all;
   }
 }
 
-// P = Z + beta P (and Zold = Z) for the columns still running
-__global__ void k_pcgmr_p(long long n, const PcgStateMR *st, const double *Z, double *P,
-                          double *Zold) {
+template <MrStep S>
+__device__ __forceinline__ void mr_step(PcgStateMR *st, const double *sm) {
+  const int q = threadIdx.x, R = st->R;
+  if (S == kMrRz0) {
+    if (q < R && !st->done[q]) {
+      const double s = sm[q];
+      st->rz[q] = s;
+      st->beta[q] = 0.0;
+      if (!(s == s) || isinf(s)) { st->status[q] = 7; st->done[q] = 1; }
+    }
+  } else if (S == kMrAlpha) {
+    if (q < R) {
+      double a = 0.0;
+      if (!st->done[q] && !st->fresh[q]) {
+        const double pq = sm[q];
+        st->pq[q] = pq;
+        a = st->rz[q] / pq;
+        if (!(a == a) || isinf(a)) { st->status[q] = 7; st->done[q] = 1; a = 0.0; }
+      }
+      st->alpha[q] = a;
+    }
+  } else if (S == kMrRr) {
+    __shared__ int anyc;
+    if (q == 0) anyc = 0;
+    __syncthreads();
+    if (q < R && !st->done[q] && !st->fresh[q]) {
+      const double rr = sm[q];
+      st->rr[q] = rr;
+      st->its[q] += 1;
+      if (!(rr == rr) || isinf(rr)) { st->status[q] = 7; st->done[q] = 1; }
+      else {
+        st->check[q] = (rr <= st->tol2[q]) ? 1 : 0;
+        if (st->check[q]) atomicOr(&anyc, 1);
+        else if (st->its[q] >= st->maxit) { st->status[q] = 5; st->done[q] = 1; }
+      }
+    }
+    __syncthreads();
+    if (q == 0) { st->any_check = anyc; st->no_check = anyc ? 0 : 1; }
+  } else if (S == kMrDec) {
+    if (q < R && st->check[q] && !st->done[q]) {
+      const double rt2 = sm[q];
+      st->rt2[q] = rt2;
+      if (rt2 <= st->tol2[q]) { st->status[q] = 0; st->done[q] = 1; }
+      else {
+        st->restart[q] = 1;
+        if (st->its[q] >= st->maxit) { st->status[q] = 5; st->done[q] = 1; }
+      }
+    }
+    if (q < R) st->check[q] = 0;
+    if (q == 0) st->no_check = 1;   // the check of this iteration is consumed here
+  } else {
+    if (q < R && !st->done[q]) {
+      const double rzn = sm[q];
+      const double rzo = st->flexible ? sm[R + q] : 0.0;
+      double beta = st->flexible ? (rzn - rzo) / st->rz[q] : rzn / st->rz[q];
+      if (st->restart[q] || st->fresh[q]) beta = 0.0;
+      st->beta[q] = beta;
+      st->rz[q] = rzn;
+      st->restart[q] = 0;
+      st->fresh[q] = 0;
+      if (!(rzn == rzn) || isinf(rzn)) { st->status[q] = 7; st->done[q] = 1; }
+    }
+    mr_all_done(st);
+  }
+}
+
+// Second stage of a column reduction and the scalar step: CTA g of kRedGrid adds
+// the rows of range g of bpart (row blocks; kDotSub per range after
+// k_dot_rz_mr) in order into partials[g][o], o < no; the CTA that arrives last
+// (counter, no waiting) adds the ranges as col_sums does and takes step S.  One
+// launch instead of two.  The rows are staged in shared memory by all threads,
+// so that one load latency precedes the serial adds instead of one per few.
+constexpr int kMrRedNT = 512, kMrStage = 2048;
+template <MrStep S>
+__global__ void __launch_bounds__(kMrRedNT)
+k_reduce_step_mr(int nrows, int no, const double *bpart, double *partials, PcgStateMR *st, unsigned *count,
+                 const int *gate) {
+  if (gate && *gate) return;
+  if (S == kMrDec && !st->any_check) return;
+  __shared__ double stage[kMrStage], sm[2 * kMaxR];
+  __shared__ bool last;
+  long long b0, b1;
+  red_range(nrows, blockIdx.x, gridDim.x, b0, b1);
+  const int R = st->R, per = kMrStage / no;           // rows staged at once
+  double v = 0.0;
+  for (long long b = b0; b < b1; b += per) {
+    const int cnt = (int)min((long long)per, b1 - b);
+    for (int i = threadIdx.x; i < cnt * no; i += kMrRedNT) stage[i] = bpart[b * no + i];
+    __syncthreads();
+    if (threadIdx.x < no)
+      for (int i = 0; i < cnt; i++) v += stage[i * no + threadIdx.x];
+    __syncthreads();
+  }
+  if (threadIdx.x < no) partials[(long long)blockIdx.x * 2 * R + threadIdx.x] = v;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(count, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  col_sums(partials, gridDim.x, R, no, sm);
+  mr_step<S>(st, sm);
+  if (threadIdx.x == 0) *count = 0u;
+}
+
+// T = B - A X for the columns whose true residual is to be checked, and the
+// column partials of T.T per row block (0 for the others)
+__global__ void k_pcgmr_true_res(int n, const PcgStateMR *st, const int *soff, const int *sw, const int *col,
+                                 const double *val, const double *B, const double *X, double *Tt, double *bpart) {
+  if (st->all_done || !st->any_check) return;
+  __shared__ double red[kFbMaxRed];
   const int R = st->R;
-  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n * R) return;
-  const int q = col_of(idx, row_of(idx, R), R);
-  if (st->done[q]) return;
-  const double z = Z[idx];
-  P[idx] = z + st->beta[q] * P[idx];
-  if (Zold) Zold[idx] = z;
+  const int gt = kFbLanes * R, gi = threadIdx.x / gt, tt = threadIdx.x % gt;
+  const int q = tt % R, l = tt / R;
+  const int nblk = (n + kFbRows - 1) / kFbRows;
+  for (int rb0 = blockIdx.x * fb_groups(R); rb0 < nblk; rb0 += gridDim.x * fb_groups(R)) {
+    const int rb = rb0 + gi;
+    double acc = 0.0;
+    if (rb < nblk && st->check[q])
+      for (int i = l; i < kFbRows; i += kFbLanes) {
+        const int r = rb * kFbRows + i;
+        if (r >= n) break;
+        const int off = soff[r >> 5] + (r & 31), w = sw[r >> 5];
+        double ax = 0;
+        for (int kk = 0; kk < w; kk++) ax += val[off + kk * 32] * X[(long long)col[off + kk * 32] * R + q];
+        const double t = B[(long long)r * R + q] - ax;
+        Tt[(long long)r * R + q] = t;
+        acc = fma(t, t, acc);
+      }
+    red[(gi * kFbLanes + l) * R + q] = acc;
+    __syncthreads();
+    if (l == 0 && rb < nblk) {
+      double v = 0.0;
+      for (int j = 0; j < kFbLanes; j++) v += red[(gi * kFbLanes + j) * R + q];
+      bpart[(long long)rb * R + q] = v;
+    }
+    __syncthreads();
+  }
+}
+
+// (a restart is only ever set by a true-residual check of this iteration)
+template <typename TI>
+__global__ void k_pcgmr_copy_r(long long n, const PcgStateMR *st, const double *Tt, double *Rr, const double *d,
+                               TI *in) {
+  if (st->all_done || !st->any_check) return;
+  const int R = st->R;
+  for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < n * R;
+       idx += (long long)gridDim.x * blockDim.x) {
+    const long long r = row_of(idx, R);
+    const int q = col_of(idx, r, R);
+    if (st->restart[q] && !st->done[q]) {
+      const double t = Tt[idx];
+      Rr[idx] = t;
+      if (in) from_f64(d ? t * d[r] : t, in[idx]);
+    }
+  }
+}
+
+// P = z + beta P for the columns still running, z = d .* Z (and Zold = z for
+// flexible CG)
+// Four elements per thread, a CTA's width apart, their loads before the rest
+// (one element per thread held too few bytes in flight for its extra read of d).
+constexpr int kMrPUnr = 4;
+template <typename TZ>
+__global__ void __launch_bounds__(256, 5) k_pcgmr_p(long long n, const PcgStateMR *st, const TZ *Z, const double *d, double *P, double *Zold) {
+  const int R = st->R;
+  const long long nR = n * R, i0 = (long long)blockIdx.x * blockDim.x * kMrPUnr + threadIdx.x;
+  TZ z[kMrPUnr];
+  double pv[kMrPUnr], dv[kMrPUnr];
+  int q[kMrPUnr];
+#pragma unroll
+  for (int u = 0; u < kMrPUnr; u++) {
+    const long long i = i0 + (long long)u * blockDim.x;
+    q[u] = -1;
+    if (i >= nR) continue;
+    const long long r = row_of(i, R);
+    q[u] = col_of(i, r, R);
+    z[u] = Z[i];
+    pv[u] = P[i];
+    dv[u] = d ? d[r] : 1.0;
+  }
+#pragma unroll
+  for (int u = 0; u < kMrPUnr; u++) {
+    if (q[u] < 0 || st->done[q[u]]) continue;
+    const long long i = i0 + (long long)u * blockDim.x;
+    const double zi = d ? __dmul_rn(to_f64(z[u]), dv[u]) : to_f64(z[u]);
+    P[i] = fma(st->beta[q[u]], pv[u], zi);
+    if (Zold) Zold[i] = zi;
+  }
 }
 
 // ------------------------------------------------ continuous batching (serving)
@@ -1149,42 +1307,6 @@ __global__ void k_batch_out(int n, int R, const int *perm, const double *in, dou
   const int q = col_of(idx, g, R);
   out[q * ld + perm[g]] = in[idx];
 }
-// Binary64 <-> binary32 conversions written out on the bit patterns (IEEE 754:
-// rounding to nearest, ties to even, for results in the normal binary32 range;
-// widening is exact), in integer instructions.  On this part the hardware
-// conversions issue to the FP64 pipe, which the scaling multiply already
-// occupies; the streaming cast kernels were bound by that pipe.  Zeros,
-// subnormal results, overflow, infinities and NaNs take the hardware
-// conversion.
-__device__ __forceinline__ float f64_to_f32_rn(double x) {
-  const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(x));
-  const unsigned hi = unsigned(b >> 32);
-  const unsigned e = (hi >> 20) & 0x7ffu;            // binary64 biased exponent
-  if (e >= 897u && e <= 1150u) {                      // binary32 biased exponent e - 896 in [1, 254]
-    const unsigned long long m = b & 0x000fffffffffffffull;
-    unsigned f = ((e - 896u) << 23) | unsigned(m >> 29);
-    const unsigned rest = unsigned(m & 0x1fffffffull);   // the 29 bits dropped
-    if (rest > 0x10000000u || (rest == 0x10000000u && (f & 1u))) f += 1u;   // a carry moves to the exponent
-    return __uint_as_float(f | (hi & 0x80000000u));
-  }
-  return __double2float_rn(x);
-}
-__device__ __forceinline__ double f32_to_f64(float v) {
-  const unsigned u = __float_as_uint(v);
-  const unsigned e = (u >> 23) & 0xffu;
-  if (e != 0u && e != 255u) {
-    const unsigned long long b = (static_cast<unsigned long long>(u & 0x80000000u) << 32) |
-                                 (static_cast<unsigned long long>(e + 896u) << 52) |
-                                 (static_cast<unsigned long long>(u & 0x7fffffu) << 29);
-    return __longlong_as_double(static_cast<long long>(b));
-  }
-  return double(v);
-}
-__device__ __forceinline__ double to_f64(float v) { return f32_to_f64(v); }
-__device__ __forceinline__ double to_f64(double v) { return v; }
-__device__ __forceinline__ void from_f64(double x, float &o) { o = f64_to_f32_rn(x); }
-__device__ __forceinline__ void from_f64(double x, double &o) { o = x; }
-
 // tests: out[i] = the bit-pattern conversions of in[i] (dir 0: binary64 ->
 // binary32 -> stored widened; dir 1: the binary32 reading of the low word
 // widened), compared with the hardware conversions by the caller
