@@ -342,7 +342,8 @@ ddlr_status ddlr_set_stream(ddlr_handle h, void *cuda_stream);
  * captured CUDA graphs are rebuilt at their next use.  A wait that runs out
  * sets a device flag, every CTA of the kernel returns, and the call that
  * launched it returns DDLR_ERR_TIMEOUT (its results are invalid); the flag is
- * cleared then, so the handle stays usable.  Errors: INVALID. */
+ * cleared then, so the handle stays usable.  A call that does not wait for the
+ * device (an apply into device memory) leaves it to the next one that does.  Errors: INVALID. */
 ddlr_status ddlr_set_wait_limit(ddlr_handle h, double seconds);
 
 /* Self-test of the library's binary64 <-> binary32 conversions written on the

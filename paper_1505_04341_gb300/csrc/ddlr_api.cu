@@ -204,6 +204,8 @@ struct ddlr_ctx {
     int m = 0;
     double *V = nullptr, *Z = nullptr, *H = nullptr, *cs = nullptr, *sn = nullptr, *g = nullptr, *y = nullptr,
            *cpart = nullptr, *cvec = nullptr, *st = nullptr;
+    double *pz_part = nullptr;        // partial sums of the persistent form, pz_stride columns
+    int pz_stride = 0;
     // Arnoldi step j of a cycle as one CUDA graph each (captured at first
     // use; they hold the arrays above and the handle's wait limit)
     std::vector<cudaGraphExec_t> step;
@@ -257,6 +259,7 @@ struct ddlr_ctx {
   // persistent cooperative kernels (shallow factors): one CTA per SM
   double *pz_part = nullptr;  // 3 x pz_grid x pz_pstride partial sums
   unsigned *pz_bar = nullptr; // grid-barrier arrival counter
+  unsigned *pz_bar2 = nullptr;// the same and the exit counter of the kernels that reset them (pz_exit)
   unsigned char *pz_lvl0 = nullptr;  // rows on the first level of their block
   int pz_grid = 0, pz_pstride = 0, pz_mmax = 0;
   bool pz_pcg = false, pz_lz = false;
@@ -2122,6 +2125,8 @@ void pz_setup(ddlr_ctx *c, int mmax) {
   if (!c->pz_pcg && !c->pz_lz) return;
   c->pz_part = c->alloc<double>(size_t(3) * c->pz_grid * c->pz_pstride);
   c->pz_bar = c->alloc<unsigned>(1);
+  c->pz_bar2 = c->alloc<unsigned>(2);
+  ck(cudaMemsetAsync(c->pz_bar2, 0, 2 * sizeof(unsigned), c->stream), "memset");
   std::vector<unsigned char> f0(P.n, 0);
   for (int b = 0; b + 1 < int(P.blk_lvl0.size()); b++) {
     const int l0 = P.blk_lvl0[b];
@@ -2202,6 +2207,64 @@ bool pz_launch(ddlr_ctx *c, const char *fam, const void *fn, size_t smem, void *
   }
   ck(e, "cudaLaunchCooperativeKernel");
   return true;
+}
+
+// a cooperative launch of a kernel that resets its counters itself, on `grid`
+// CTAs; false as for pz_launch
+bool pz_launch_own(ddlr_ctx *c, const char *fam, const void *fn, int grid, size_t smem, void **args) {
+  ddlr_ctx::Scope sc(c, fam, c->stream);
+  const char *fake = getenv("DDLR_FAKE_COOP_REFUSAL");
+  const cudaError_t e = (fake && fake[0] == '1')
+                            ? cudaErrorCooperativeLaunchTooLarge
+                            : cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kPzThreads), args, smem, c->stream);
+  if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+    cudaGetLastError();   // not sticky: clear it
+    c->pz_pcg = c->pz_lz = false;
+    return false;
+  }
+  ck(e, "cudaLaunchCooperativeKernel");
+  return true;
+}
+// CTAs of a persistent apply or GMRES solve: a CTA has at least kPzMinRows rows
+// (64 to 512 rows measured alike, 1,024 slower: 24^3 GMRES 55, 60 and 73 us a
+// step with 256, 512 and 1,024)
+constexpr int kPzMinRows = 256;
+int pz_small_grid(const ddlr_ctx *c) {
+  return std::max(1, std::min(c->pz_grid, (c->P.n + kPzMinRows - 1) / kPzMinRows));
+}
+
+template <typename T, typename TU>
+bool apply_persist_t(ddlr_ctx *c, const double *x, double *y, T *u, T *z, T *v, T *w, T *rhs) {
+  PzOp<T, TU> O = make_pzop<T, TU>(c);
+  O.gs.count = c->pz_bar2;
+  PzApply<T> A{x, y, c->pv[1], c->perm, u, z, v, w, rhs};
+  void *args[] = {&O, &A};
+  return pz_launch_own(c, "apply_persist", (const void *)k_apply_persist<kPzThreads, T, TU>, pz_small_grid(c),
+                       pz_pcg_smem(c->opt.rank_k), args);
+}
+// y = M^-1 x in the caller's order as one launch; false: not served
+bool apply_persist(ddlr_ctx *c, const double *x, double *y) {
+  if (!c->pz_pcg) return false;
+  double *const *D = c->w64;
+  float *const *F = c->w32;
+  if (c->opt.precision == 0) return apply_persist_t<double, double>(c, x, y, c->pv[7], D[0], D[1], D[2], D[3]);
+  if (c->opt.uk_bf16) return apply_persist_t<float, __nv_bfloat16>(c, x, y, F[4], F[0], F[1], F[2], F[3]);
+  return apply_persist_t<float, float>(c, x, y, F[4], F[0], F[1], F[2], F[3]);
+}
+
+template <typename T, typename TU>
+bool gmres_persist_t(ddlr_ctx *c, const double *b, double *x, double tol, int maxit, int m, T *u, T *z, T *y, T *w,
+                     T *rhs) {
+  PzOp<T, TU> O = make_pzop<T, TU>(c);
+  O.gs.count = c->pz_bar2;
+  O.pstride = c->gm.pz_stride;
+  O.part = c->gm.pz_part;
+  PzGm<T> P{b, x, c->pv[1], c->pv[3], c->gm.V, c->gm.Z, u, z, y, w, rhs, c->pcg, tol, maxit, m};
+  void *args[] = {&O, &P};
+  const size_t smem = pz_gm_smem(c->opt.rank_k, m);
+  raise_smem_limit((const void *)k_gmres_persist<kPzThreads, T, TU>, smem);
+  return pz_launch_own(c, "gmres_persist", (const void *)k_gmres_persist<kPzThreads, T, TU>, pz_small_grid(c), smem,
+                       args);
 }
 
 // grid barriers of one PCG iteration and of one Lanczos step, upper bounds
@@ -2538,6 +2601,35 @@ void gmres_dev(ddlr_ctx *c, const double *b, double *x, double tol, int maxit, i
     G.cvec = c->alloc<double>(m + 1);
     G.st = c->alloc<double>(4);
     G.m = m;
+  }
+  // shallow factors on small problems: the whole solve in one launch
+  if (c->pz_pcg && m <= kPzGmMaxRestart &&
+      (long long)(maxit + 2) * (2 * pz_barriers_per_iteration(c)) * c->pz_grid < (1LL << 31)) {
+    const int stride = std::max(c->opt.rank_k, m + 2);
+    if (G.pz_stride < stride) {
+      G.pz_part = c->alloc<double>(size_t(3) * c->pz_grid * stride);
+      G.pz_stride = stride;
+    }
+    double *const *D = c->w64;
+    float *const *F = c->w32;
+    const bool ok = c->opt.precision == 0 ? gmres_persist_t<double, double>(c, b, x, tol, maxit, m, c->pv[7], D[0],
+                                                                           D[1], D[2], D[3])
+                    : c->opt.uk_bf16
+                        ? gmres_persist_t<float, __nv_bfloat16>(c, b, x, tol, maxit, m, F[4], F[0], F[1], F[2], F[3])
+                        : gmres_persist_t<float, float>(c, b, x, tol, maxit, m, F[4], F[0], F[1], F[2], F[3]);
+    if (ok) {
+      PcgState hs;
+      int dfl[4];
+      ck(cudaMemcpyAsync(&hs, c->pcg, sizeof(PcgState), cudaMemcpyDeviceToHost, c->stream), "D2H");
+      read_dev(c, dfl, c->dflag, sizeof(dfl));
+      if (dfl[3]) timeout_fail(c);
+      if (info) {
+        info->its = hs.its;
+        info->relres = hs.bb > 0 ? hs.rr / hs.bb : 0.0;
+        info->status = hs.status == 0 ? DDLR_OK : (hs.status == 5 ? DDLR_ERR_NOCONV : DDLR_ERR_NAN);
+      }
+      return;
+    }
   }
   const int ld = m + 1;
   double *r = c->pv[1], *w = c->pv[3], *q = c->pv[4];
@@ -3232,6 +3324,7 @@ namespace {
 // and report DDLR_ERR_TIMEOUT
 void clear_timeout(ddlr_ctx *c) {
   cudaMemsetAsync(c->dflag + 3, 0, sizeof(int), c->stream);
+  if (c->pz_bar2) cudaMemsetAsync(c->pz_bar2, 0, 2 * sizeof(unsigned), c->stream);
   cudaStreamSynchronize(c->stream);
 }
 [[noreturn]] void timeout_fail(ddlr_ctx *c) {
@@ -3686,8 +3779,10 @@ static ddlr_status vec_call(ddlr_ctx *c, const double *x, double *y, int nrhs, i
       if (hy) yd = c->stg_out;
       body(xd, yd);
       if (hy) {
+        int timed_out;   // a device wait of this call or of one before it that did not wait
         ck(cudaMemcpyAsync(yj, yd, sizeof(double) * n, cudaMemcpyDeviceToHost, c->stream), "D2H");
-        sync(c);
+        read_dev(c, &timed_out, c->dflag + 3, sizeof(int));
+        if (timed_out) timeout_fail(c);
       }
     }
     return DDLR_OK;
@@ -3715,6 +3810,7 @@ ddlr_status ddlr_apply(ddlr_handle c, const double *x, double *y, int nrhs, int 
   }
   return vec_call(c, x, y, nrhs, ld, [c](const double *xd, double *yd) {
     const int n = c->P.n;
+    if (apply_persist(c, xd, yd)) return;
     double *xi = c->pv[1], *yo = c->pv[2];
     KL(c, "perm", c->stream, k_permute_in<double>, nblk(n), kThreads, 0, n, c->perm, xd, xi);
     precond(c, xi, yo, nullptr);

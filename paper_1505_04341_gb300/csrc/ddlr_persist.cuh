@@ -348,13 +348,27 @@ __device__ __forceinline__ T pz_row_dot(const TU *row, const T *vec, int k) {
   return a + b;
 }
 
+// Where a persistent apply leaves its result besides its own vector: out[perm[r]]
+// (perm == nullptr: out[r]) = sc_r z_r in FP64, written by the thread that
+// finalises row r
+struct PzOut {
+  double *out;
+  const int *perm;
+  const double *sc;
+};
+template <typename T>
+__device__ __forceinline__ void pz_out(const PzOut &o, int r, T z) {
+  o.out[o.perm ? ro(o.perm + r) : r] = o.sc ? ro(o.sc + r) * double(z) : double(z);
+}
+
 // One level L of every block: mode 0 forward, 1 backward, 2 forward then
 // backward (the top level).  x is read as pz_in.  Rows finalised here (modes
 // 1, 2) add racc_r (zsc_r z_r) to acc when racc is given; z2 (level 0,
 // backward) receives the first forward level of a solve whose input is z.
-template <int NT, typename T, typename TU, typename TX>
+template <int NT, bool OUT = false, typename T, typename TU, typename TX>
 __device__ __forceinline__ void pz_level(const PzOp<T, TU> &O, int L, int mode, const TX *x, const double *xsc,
-                                         T *z, const double *racc, const double *zsc, double &acc, T *z2) {
+                                         T *z, const double *racc, const double *zsc, double &acc, T *z2,
+                                         const PzOut &po = PzOut{}) {
   const int c0 = O.lvl_ptr[L];
   int v0, v1;
   pz_range(O.lvl_ptr[L + 1] - c0, v0, v1);        // a level's rows over all CTAs
@@ -376,6 +390,7 @@ __device__ __forceinline__ void pz_level(const PzOp<T, TU> &O, int L, int mode, 
       if (mode == 2) zr = zr * dr;
     }
     z[r] = zr;
+    if (OUT && mode != 0) pz_out(po, r, zr);
     if (racc && mode != 0) acc += racc[r] * (zsc ? ro(zsc + r) * double(zr) : double(zr));
     if (z2) z2[r] = zr * dr;          // first forward level of a solve with input z
   }
@@ -385,19 +400,19 @@ __device__ __forceinline__ void pz_level(const PzOp<T, TU> &O, int L, int mode, 
 // the last phase is left open (the caller adds its own work and barrier).
 // l0_done: the producer of x has already done the first forward level
 // (pz_l0).  z2: see pz_level (only with fuse0).
-template <int NT, typename T, typename TU, typename TX>
+template <int NT, bool OUT = false, typename T, typename TU, typename TX>
 __device__ __forceinline__ bool pz_a0(const PzOp<T, TU> &O, const TX *x, const double *xsc, T *z,
                                       const double *racc, const double *zsc, double &acc, unsigned &ep,
-                                      bool l0_done, T *z2 = nullptr) {
+                                      bool l0_done, T *z2 = nullptr, const PzOut &po = PzOut{}) {
   const int nL = O.nL;
   for (int L = l0_done ? 1 : 0; L + 1 < nL; L++) {
     pz_level<NT>(O, L, 0, x, xsc, z, nullptr, nullptr, acc, (T *)nullptr);
     if (!pz_sync(O.gs, ep)) return false;
   }
-  pz_level<NT>(O, nL - 1, 2, x, xsc, z, racc, zsc, acc, (T *)nullptr);
+  pz_level<NT, OUT>(O, nL - 1, 2, x, xsc, z, racc, zsc, acc, (T *)nullptr, po);
   for (int L = nL - 2; L >= 0; L--) {
     if (!pz_sync(O.gs, ep)) return false;
-    pz_level<NT>(O, L, 1, x, xsc, z, racc, zsc, acc, L == 0 ? z2 : (T *)nullptr);
+    pz_level<NT, OUT>(O, L, 1, x, xsc, z, racc, zsc, acc, L == 0 ? z2 : (T *)nullptr, po);
   }
   return true;
 }
@@ -407,10 +422,10 @@ __device__ __forceinline__ bool pz_a0(const PzOp<T, TU> &O, const TX *x, const d
 // as it is read.  acc collects sum_r racc_r (dsc_r u_r) over the rows this CTA
 // finalises.  Scratch: z (n), y, w (s), rhs (n).  The last phase is left
 // open.  `slot` is the next partial-sum buffer.
-template <int NT, typename T, typename TU>
+template <int NT, bool OUT = false, typename T, typename TU>
 __device__ __forceinline__ bool pz_apply(const PzOp<T, TU> &O, const double *x, T *u, T *z, T *y, T *w, T *rhs,
                                          const double *racc, double &acc, unsigned &ep, int &slot, double *red,
-                                         T *vec, bool l0_done) {
+                                         T *vec, bool l0_done, const PzOut &po = PzOut{}) {
   const double *xsc = O.dsc;
   const int n = O.n, m = O.m, s = O.s, k = O.k;
   if (O.variant == 2) {
@@ -425,6 +440,7 @@ __device__ __forceinline__ bool pz_apply(const PzOp<T, TU> &O, const double *x, 
     for (int r = i0 + threadIdx.x; r < i1; r += NT) {
       const T ur = u[r] + pz_row_dot<T, TU>(O.U + (size_t)r * k, vec, k);
       u[r] = ur;
+      if (OUT) pz_out(po, r, ur);
       if (racc) acc += racc[r] * (O.dsc ? ro(O.dsc + r) * double(ur) : double(ur));
     }
     return true;
@@ -466,7 +482,58 @@ __device__ __forceinline__ bool pz_apply(const PzOp<T, TU> &O, const double *x, 
     pz_l0(O, i, rv, u);
   }
   if (!pz_sync(O.gs, ep)) return false;
-  return pz_a0<NT>(O, rhs, (const double *)nullptr, u, racc, O.dsc, acc, ep, O.fuse0 != 0);
+  return pz_a0<NT, OUT>(O, rhs, (const double *)nullptr, u, racc, O.dsc, acc, ep, O.fuse0 != 0, (T *)nullptr, po);
+}
+
+// The last act of a kernel with a counter of its own: the CTA that leaves last
+// puts the barrier's counter and the exit counter behind it back to 0, so that
+// the next launch needs no memset (a launch of its own, as long as two phases).
+// Every CTA has passed its last barrier when the last one leaves.  A launch that
+// timed out leaves them as they are; the host clears them with the flag, and
+// until then a launch does nothing (pz_stale).
+__device__ __forceinline__ bool pz_stale(const GridSync &g) { return *(volatile int *)g.err != 0; }
+__device__ __forceinline__ void pz_exit(const GridSync &g) {
+  if (threadIdx.x != 0) return;
+  if (atomicAdd(g.count + 1, 1u) == gridDim.x - 1) {
+    atomicExch(g.count, 0u);
+    atomicExch(g.count + 1, 0u);
+  }
+}
+
+// ----------------------------------------------------------------- apply
+// y = M^-1 x, x and y in the caller's order, as one cooperative launch: the
+// permutation in with the first forward level, the phases of pz_apply, the
+// permutation out by the threads that finalise the rows.  8 grid phases instead
+// of 9 launches: bound by latency on the problems the persistent PCG serves (33 x
+// 17 x 21: 55.4 -> 28.8 us, 64^3: 64.7 -> 43.1, DDLR-2 79.3 -> 69.9).
+template <typename T>
+struct PzApply {
+  const double *x;
+  double *y, *xi;
+  const int *perm;
+  T *u, *z, *v, *w, *rhs;
+};
+template <int NT, typename T, typename TU>
+__global__ void __launch_bounds__(NT, 1) k_apply_persist(PzOp<T, TU> O, PzApply<T> A) {
+  extern __shared__ double pz_sm[];
+  double *red = pz_sm;
+  T *vec = reinterpret_cast<T *>(pz_sm + NT + 32);
+  unsigned ep = 0;
+  int slot = 0, i0, i1;
+  pz_range(O.n, i0, i1);
+  T *a0out = O.variant == 2 ? A.u : A.z;
+  if (pz_stale(O.gs)) return;
+  for (int i = i0 + threadIdx.x; i < i1; i += NT) {
+    const double v = A.x[ro(A.perm + i)];
+    A.xi[i] = v;
+    pz_l0(O, i, O.dsc ? T(v * ro(O.dsc + i)) : T(v), a0out);
+  }
+  if (!pz_sync(O.gs, ep)) return;
+  double acc = 0;
+  if (!pz_apply<NT, true>(O, A.xi, A.u, A.z, A.v, A.w, A.rhs, (const double *)nullptr, acc, ep, slot, red, vec,
+                          O.fuse0 != 0, PzOut{A.y, A.perm, O.dsc}))
+    return;
+  pz_exit(O.gs);
 }
 
 // ------------------------------------------------------------------- PCG
@@ -1021,6 +1088,200 @@ __global__ void __launch_bounds__(NT, 1) k_lz_persist(PzOp<double, double> O, Pz
     st->nan_step = nan_step; st->scale = scale; st->npass2 = cnt.npass2; st->nfp32 = cnt.nfp32;
     st->qcols64 = cnt.q64; st->qcols32 = cnt.q32;
   }
+}
+
+// ----------------------------------------------------------------- GMRES
+// Restarted GMRES(m) of gmres_dev in one launch: the same recurrences (Arnoldi on
+// A M^-1 with two classical Gram-Schmidt passes, Givens rotations, x += Z y, the
+// true residual at the end of each cycle), a step in about 12 grid phases instead
+// of 17 launches and a host read.  The rotations, the rotated right-hand side and
+// R are kept by every CTA in shared memory (same inputs, same operations), so all
+// take the same decisions.  24^3: 92 -> 55 us a step, 64^3 (bound by the Gram-
+// Schmidt products' FP64 and the apply) 196 -> 127.
+template <typename T>
+struct PzGm {
+  const double *b;
+  double *x, *r, *w, *V, *Z;       // V n x (m + 1), Z n x m, column-major
+  T *u, *z, *y, *wi, *rhs;
+  PcgState *st;                    // its, status, rr = ||r||, bb = ||b||
+  double tol;
+  int maxit, m;
+};
+constexpr int kPzGmMaxRestart = 128;
+inline size_t pz_gm_smem(int k, int m) {
+  return size_t(kPzThreads + 32 + k + 2 + 4 * (m + 2) + m * (m + 1) / 2 + 8) * sizeof(double);
+}
+
+template <int NT, typename T, typename TU>
+__global__ void __launch_bounds__(NT, 1) k_gmres_persist(PzOp<T, TU> O, PzGm<T> P) {
+  extern __shared__ double pz_sm[];
+  const int m = P.m, n = O.n;
+  double *red = pz_sm, *bc = pz_sm + NT;
+  T *vec = reinterpret_cast<T *>(pz_sm + NT + 32);
+  double *c = pz_sm + NT + 32 + O.k + 2;          // coefficients of a Gram-Schmidt pass
+  double *hc = c + m + 2, *rc = hc + m + 2, *rs = rc + m + 2;   // Hessenberg column, rotations
+  double *Rm = rs + m + 2;                        // R, column j at j (j + 1) / 2
+  double *sc = Rm + m * (m + 1) / 2;              // [0] |g_{j+1}|, [1] g_{j+1}
+  __shared__ double gv[kPzGmMaxRestart + 1], yv[kPzGmMaxRestart];
+  unsigned ep = 0;
+  int slot = 0, i0, i1;
+  pz_range(n, i0, i1);
+  const int act = i1 - i0;
+  const auto roots = [](double v) {
+    const double b = sqrt(v);
+    return make_double2(b, 1.0 / b);
+  };
+  T *a0out = O.variant == 2 ? P.u : P.z;
+  if (pz_stale(O.gs)) return;
+  double acc = 0;
+  for (int i = i0 + threadIdx.x; i < i1; i += NT) {
+    const double bi = P.b[i];
+    P.x[i] = 0.0;
+    P.r[i] = bi;
+    acc += bi * bi;
+  }
+  double *pt = pz_buf(O, slot++);
+  pz_put<NT>(acc, act, pt, O.pstride, red);
+  if (!pz_sync(O.gs, ep)) return;
+  PzScalar be = pz_get(pt, O.pstride, bc, roots);
+  const double bn = be.f.x, tolb = P.tol * bn;
+  int its = 0, status = 5;
+  while (true) {
+    const double beta = be.f.x;
+    if (pz_bad(be.sum)) { status = 7; break; }
+    if (pz_le(beta, tolb)) { status = 0; break; }
+    if (its >= P.maxit) break;
+    for (int i = i0 + threadIdx.x; i < i1; i += NT) {               // v_0 = r / beta
+      const double v = P.r[i] * be.f.y;
+      P.V[i] = v;
+      pz_l0(O, i, O.dsc ? T(v * ro(O.dsc + i)) : T(v), a0out);
+    }
+    if (threadIdx.x == 0) { gv[0] = beta; sc[1] = beta; }
+    if (!pz_sync(O.gs, ep)) return;
+    int j = 0;
+    bool nan = false;
+    while (j < m && its < P.maxit) {
+      const double *vj = P.V + (size_t)j * n;
+      double *zj = P.Z + (size_t)j * n;
+      double dummy = 0;
+      if (!pz_apply<NT, true>(O, vj, P.u, P.z, P.y, P.wi, P.rhs, (const double *)nullptr, dummy, ep, slot, red, vec,
+                              O.fuse0 != 0, PzOut{zj, nullptr, O.dsc}))
+        return;
+      if (!pz_sync(O.gs, ep)) return;
+      // w = A z_j, first Gram-Schmidt pass
+      for (int i = i0 + threadIdx.x; i < i1; i += NT) {
+        const int g = i >> 5, l = i & 31;
+        const int off = ro(O.a_soff + g) + l, wd = ro(O.a_sw + g);
+        double q = 0;
+        for (int kk = 0; kk < wd; kk++) q += ro(O.a_val + off + kk * 32) * zj[ro(O.a_col + off + kk * 32)];
+        P.w[i] = q;
+      }
+      __syncthreads();
+      pt = pz_buf(O, slot++);
+      pz_gemvT<NT>(P.V, n, j + 1, P.w, i0, i1, pt, O.pstride, red);
+      if (!pz_sync(O.gs, ep)) return;
+      pz_get_cols<NT, double>(pt, O.pstride, j + 1, nullptr, nullptr, c, red);
+      for (int i = threadIdx.x; i <= j; i += NT) hc[i] = c[i];
+      pz_gemvN<NT>(P.V, n, j + 1, c, P.w, i0, i1);
+      __syncthreads();
+      // second pass
+      pt = pz_buf(O, slot++);
+      pz_gemvT<NT>(P.V, n, j + 1, P.w, i0, i1, pt, O.pstride, red);
+      if (!pz_sync(O.gs, ep)) return;
+      pz_get_cols<NT, double>(pt, O.pstride, j + 1, nullptr, nullptr, c, red);
+      for (int i = threadIdx.x; i <= j; i += NT) hc[i] += c[i];
+      acc = pz_gemvN<NT>(P.V, n, j + 1, c, P.w, i0, i1);
+      pt = pz_buf(O, slot++);
+      pz_put<NT>(acc, act, pt, O.pstride, red);
+      if (!pz_sync(O.gs, ep)) return;
+      const PzScalar hn = pz_get(pt, O.pstride, bc, roots);
+      // v_{j+1} = w / h_{j+1,j}, while one thread of the last warp rotates
+      // column j
+      if (j + 1 < m + 1 && !pz_bad(hn.f.y)) {
+        double *vn = P.V + (size_t)(j + 1) * n;
+        for (int i = i0 + threadIdx.x; i < i1; i += NT) {
+          const double v = P.w[i] * hn.f.y;
+          vn[i] = v;
+          pz_l0(O, i, O.dsc ? T(v * ro(O.dsc + i)) : T(v), a0out);
+        }
+      }
+      if (threadIdx.x == NT - 32) {
+        double h = hc[0];
+        double *Rj = Rm + j * (j + 1) / 2;
+        for (int i = 0; i < j; i++) {
+          const double h1 = hc[i + 1], t = rc[i] * h + rs[i] * h1;
+          h = -rs[i] * h + rc[i] * h1;
+          Rj[i] = t;
+        }
+        const double hs = hn.f.x, d = hypot(h, hs);
+        const double cj = d > 0.0 ? h / d : 1.0, sj = d > 0.0 ? hs / d : 0.0;
+        rc[j] = cj;
+        rs[j] = sj;
+        Rj[j] = d;
+        const double gj = sc[1], gn = -sj * gj;
+        gv[j] = cj * gj;
+        sc[0] = fabs(gn);
+        sc[1] = gn;
+      }
+      if (!pz_sync(O.gs, ep)) return;
+      its++;
+      j++;
+      const double res = sc[0];
+      if (pz_bad(res) || pz_bad(hn.sum)) { nan = true; break; }
+      if (pz_le(res, tolb) || hn.sum == 0.0) break;
+    }
+    if (nan) { status = 7; break; }
+    // R y = g by one warp (column-oriented), x += Z y
+    if (threadIdx.x < 32) {
+      const int l = threadIdx.x;
+      double gl[(kPzGmMaxRestart + 31) / 32], di[(kPzGmMaxRestart + 31) / 32];
+#pragma unroll
+      for (int q = 0; q < (kPzGmMaxRestart + 31) / 32; q++) {
+        const int i = l + 32 * q;
+        gl[q] = i < j ? gv[i] : 0.0;
+        di[q] = i < j ? 1.0 / Rm[i * (i + 1) / 2 + i] : 0.0;
+      }
+#pragma unroll
+      for (int q = (kPzGmMaxRestart + 31) / 32 - 1; q >= 0; q--)
+        for (int i = min(j, 32 * q + 32) - 1; i >= 32 * q; i--) {
+          const double yi = __shfl_sync(0xffffffffu, gl[q] * di[q], i & 31);
+          if (l == 0) yv[i] = yi;
+          const double *Ri = Rm + i * (i + 1) / 2;
+#pragma unroll
+          for (int p = 0; p <= q; p++)
+            if (l + 32 * p < i) gl[p] -= Ri[l + 32 * p] * yi;
+        }
+    }
+    __syncthreads();
+    for (int i = i0 + threadIdx.x; i < i1; i += NT) {
+      double t = 0;
+#pragma unroll 4
+      for (int l = 0; l < j; l++) t += P.Z[(size_t)l * n + i] * yv[l];
+      P.x[i] += t;
+    }
+    if (!pz_sync(O.gs, ep)) return;
+    acc = 0;
+    for (int i = i0 + threadIdx.x; i < i1; i += NT) {               // r = b - A x
+      const int g = i >> 5, l = i & 31;
+      const int off = ro(O.a_soff + g) + l, wd = ro(O.a_sw + g);
+      double ax = 0;
+      for (int kk = 0; kk < wd; kk++) ax += ro(O.a_val + off + kk * 32) * P.x[ro(O.a_col + off + kk * 32)];
+      const double t = P.b[i] - ax;
+      P.r[i] = t;
+      acc += t * t;
+    }
+    pt = pz_buf(O, slot++);
+    pz_put<NT>(acc, act, pt, O.pstride, red);
+    if (!pz_sync(O.gs, ep)) return;
+    be = pz_get(pt, O.pstride, bc, roots);
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    P.st->its = its;
+    P.st->status = status;
+    P.st->rr = be.f.x;
+    P.st->bb = bn;
+  }
+  pz_exit(O.gs);
 }
 
 }  // namespace ddlr
