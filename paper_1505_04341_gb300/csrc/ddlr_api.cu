@@ -548,6 +548,19 @@ void desc_sweeps(ddlr_ctx *c, cudaStream_t st, const char *fam, const T *lv0, co
       KL(c, fam, st, (k_sptrsv_desc<T, 1, TX>), grid, kThreads, 0, d, cnt, mode, lc, uc, lv, uv, di, x, z, gate,
          o64);
   };
+  if constexpr (sizeof(T) == 4)
+    if (nL == 2 && !c->chunk_rows) {
+      auto two = [&](auto mode, int L, const int *col, const T *val) {
+        const int cnt = ptr[L + 1] - ptr[L];
+        if (cnt > 0)
+          KL(c, fam, st, (k_sptrsv_two<T, decltype(mode)::value, TX>), (cnt + kThreads - 1) / kThreads, kThreads, 0,
+             c->lv_desc + ptr[L], cnt, col, val, di, x, z, gate, z64);
+      };
+      if (lx) two(std::integral_constant<int, 5>{}, 1, c->S.l_col, lx);
+      else two(std::integral_constant<int, 3>{}, 1, c->S.l_col, lv0);
+      two(std::integral_constant<int, 4>{}, 0, c->S.u_col, uv);
+      return;
+    }
   if (nL == 2) {
     launch(1, lx ? 5 : 3);
     launch(0, 4);
@@ -2864,12 +2877,12 @@ void a0_solve_mr(ddlr_ctx *c, const T *X, T *Z, int R, const int *gate) {
       constexpr int kV = Vec16<T>::n;
       if (R % kV == 0) {
         // 16-byte vectors of kV columns per thread; 256 threads
-        const int per = 256 / (R / kV), rows = per * kMrRowsPerThread;
+        const int per = 256 / (R / kV), rows = per * kMrRowsPerThread<T>;
         KL(c, "sptrsv_levels_mr", c->stream, k_sptrsv_desc_mr_v<T>, (cnt + rows - 1) / rows, per * (R / kV), 0,
            c->lv_desc + dptr[L], cnt, mode, c->S.l_col, c->S.u_col, lv, uv, di, X, Z, R, gate);
         return;
       }
-      const int bd = chunk_block(c, R), rows = (bd / R) * kMrRowsPerThread;
+      const int bd = chunk_block(c, R), rows = (bd / R) * kMrRowsPerThread<T>;
       KL(c, "sptrsv_levels_mr", c->stream, k_sptrsv_desc_mr<T>, (cnt + rows - 1) / rows, bd, 0,
          c->lv_desc + dptr[L], cnt, mode, c->S.l_col, c->S.u_col, lv, uv, di, X, Z, R, gate);
       return;

@@ -82,15 +82,19 @@ __global__ void k_sptrsv_chunks_mr(SolveLayout S, const int4 *chunks, int mode,
 // rows a pass of the CTA covers (blockDim / R).  A thread takes its
 // kMrRowsPerThread rows together: the rows of a level depend only on rows of
 // other levels, so their descriptor, operand and gathered loads are all in
-// flight at once (a thread walking its rows one by one kept one dependent
-// chain of loads in flight).  Each row's arithmetic is that of one row alone.
-constexpr int kMrRowsPerThread = 4;
+// flight at once.  Each row's arithmetic is that of one row alone.  Two rows in
+// FP32, bound by the latency of the gathers (a launch, 96^3: 32 columns 85, 73
+// and 77 us with 1, 2 and 4 rows; 16 columns 49, 42 and 43); one in FP64, where
+// the FMA slots of the rows that have fewer entries than their thread's longest
+// cost more than the loads in flight give (64^3 x 8: 24.5, 25.3 and 30.4 us;
+// 96^3 x 16: 117, 120 and 152; 128^3 x 4: 78, 79 and 98).
+template <typename T> constexpr int kMrRowsPerThread = sizeof(T) == 8 ? 1 : 2;
 template <typename T>
 __global__ void k_sptrsv_desc_mr(const int4 *desc, int count, int mode, const int *l_col, const int *u_col,
                                  const T *lval, const T *uval, const T *dinv, const T *X, T *Z, int R,
                                  const int *gate) {
   if (gate && *gate) return;
-  constexpr int RR = kMrRowsPerThread;
+  constexpr int RR = kMrRowsPerThread<T>;
   const int per = blockDim.x / R;
   const int q = threadIdx.x % R, sub = threadIdx.x / R;
   if (sub >= per) return;
@@ -185,7 +189,7 @@ __global__ void k_sptrsv_desc_mr_v(const int4 *desc, int count, int mode, const 
   if (gate && *gate) return;
   using VT = Vec16<T>;
   using V = typename VT::V;
-  constexpr int kV = VT::n, RR = kMrRowsPerThread;
+  constexpr int kV = VT::n, RR = kMrRowsPerThread<T>;
   const int tpr = R / kV;                       // threads per row
   const int per = blockDim.x / tpr;
   const int q0 = (threadIdx.x % tpr) * kV, sub = threadIdx.x / tpr;

@@ -463,6 +463,55 @@ k_sptrsv_desc(const int4 *desc, int count, int mode, const int *l_col, const int
     }
 }
 
+// The two launches of a two-level solve (mode MODE of k_sptrsv_chunks: 5 or 3,
+// then 4) in FP32, a row per thread with its entries in groups of kTwoGroup (all
+// of a 7-point row): the columns and values of a group are loaded together, then
+// its gathers, where k_sptrsv_desc waits for a column and a gather per entry.
+// Bound by the latency of descriptor, entry and gather; per row the arithmetic
+// of k_sptrsv_desc.  A0 solve, 128^3: 81.6 -> 79.0 us, 96^3 irregular boxes: 54.0
+// -> 42.5 (groups of 3 and 4: 83 and 89; 43 and 46; two and four rows a thread
+// 78 to 93; 42 to 48).  FP64 stays with k_sptrsv_desc: a group's idle slots
+// take FP64 issue (128^3: 76 -> 82 us).
+constexpr int kTwoGroup = 6;
+template <typename T, int MODE, typename TX = T>
+__global__ void __launch_bounds__(kThreads)
+k_sptrsv_two(const int4 *__restrict__ desc, int count, const int *__restrict__ col, const T *__restrict__ val,
+             const T *__restrict__ dinv, const TX *x, T *z, const int *gate, double *z64) {
+  static_assert(MODE == 3 || MODE == 4 || MODE == 5, "modes of a two-level solve");
+  if (gate && *gate) return;
+  const int idx = blockIdx.x * kThreads + threadIdx.x;
+  if (idx >= count) return;
+  const int4 d = __ldg(desc + idx);
+  const int row = d.x, off = MODE == 4 ? d.z : d.y;
+  const int w = MODE == 4 ? int(unsigned(d.w) >> 16) : int(unsigned(d.w) & 0xffffu);
+  const T dr = __ldg(dinv + row);
+  T acc = T(x[row]);
+  if (MODE == 4) acc = acc * dr;
+  for (int k0 = 0; k0 < w; k0 += kTwoGroup) {
+    int c[kTwoGroup];
+    T v[kTwoGroup], g[kTwoGroup], dc[kTwoGroup];
+#pragma unroll
+    for (int j = 0; j < kTwoGroup; j++)
+      if (k0 + j < w) {
+        c[j] = __ldg(col + off + (k0 + j) * 32);
+        v[j] = __ldg(val + off + (k0 + j) * 32);
+      }
+#pragma unroll
+    for (int j = 0; j < kTwoGroup; j++)
+      if (k0 + j < w) {
+        g[j] = MODE == 4 ? z[c[j]] : T(x[c[j]]);
+        if (MODE == 3) dc[j] = __ldg(dinv + c[j]);
+      }
+#pragma unroll
+    for (int j = 0; j < kTwoGroup; j++)
+      if (k0 + j < w) acc -= v[j] * (MODE == 3 ? g[j] * dc[j] : g[j]);
+  }
+  T a = acc * dr;
+  if (MODE != 4) a = a * dr;
+  z[row] = a;
+  if (z64) z64[row] = double(a);
+}
+
 // ======================================================= E, E^T products
 // v = E w + xadd = [a^-1 Ehat w ; -a w] + xadd   (eq. EF), rows [0, n)
 template <typename T>
