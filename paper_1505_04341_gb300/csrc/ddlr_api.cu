@@ -154,6 +154,9 @@ struct ddlr_ctx {
   int *blk_row0 = nullptr;
   int *chunks = nullptr;
   int4 *lv_desc = nullptr;    // level-order row descriptors (shallow factors)
+  int4 *e_desc = nullptr;     // two levels: those of the rows that E^T A0^-1 needs (null: all)
+  std::vector<int> e_ptr;     // their offsets by level
+  double e_entries = 0;       // and factor entries
   // deep factors (ddlr_deep.cuh): the interior blocks, a CTA each, and C_a
   // (D_a) by one cluster; ctas == 0: not served (the interior blocks then take
   // k_sptrsv_blocks, C_a a launch per level)
@@ -518,13 +521,23 @@ void c_block_solve(ddlr_ctx *c, cudaStream_t st, const char *fam, const T *lv, c
   else chunk_sweeps<T>(c, st, c->P.ch_c_ptr, fam, lv, uv, di, x, z, gate);
 }
 
-// the same sweeps over the level-order descriptor list (all blocks); x may be
+// what a solve that only E^T reads leaves out of the bytes of a full one (v: bytes of a value)
+double e_rows_saved(const ddlr_ctx *c, double v) {
+  if (!c->e_desc) return 0.0;
+  const double n = c->P.n;
+  return (2.0 * (double(c->P.nnz_factor) - n) - c->e_entries) * (v + 4.0) + 6.0 * v * (n - double(c->e_ptr[2]));
+}
+
+// the same sweeps over the level-order descriptor list (all blocks); e_only: z is
+// only read by E^T, so the rows that it does not need may be left out; x may be
 // wider than T (rounded as read), z64 (optional) also receives the result in
 // FP64 (every row's final value is written in FP64 too)
 template <typename T, typename TX = T>
 void desc_sweeps(ddlr_ctx *c, cudaStream_t st, const char *fam, const T *lv0, const T *uv, const T *di,
-                 const TX *x, T *z, const int *gate, double *z64 = nullptr) {
-  const std::vector<int> &ptr = c->P.lv_ptr;
+                 const TX *x, T *z, const int *gate, double *z64 = nullptr, bool e_only = false) {
+  const bool part = e_only && c->e_desc;
+  const std::vector<int> &ptr = part ? c->e_ptr : c->P.lv_ptr;
+  const int4 *desc = part ? c->e_desc : c->lv_desc;
   const int nL = int(ptr.size()) - 1;
   const int rows = c->chunk_rows ? c->chunk_rows : (sizeof(T) == 8 ? 2 : 4);
   const T *lx = Prec<T>::lx(c);
@@ -532,7 +545,7 @@ void desc_sweeps(ddlr_ctx *c, cudaStream_t st, const char *fam, const T *lv0, co
     const int cnt = ptr[L + 1] - ptr[L];
     if (cnt <= 0) return;
     const T *lv = mode == 5 ? lx : lv0;
-    const int4 *d = c->lv_desc + ptr[L];
+    const int4 *d = desc + ptr[L];
     const int grid = (cnt + kThreads - 1) / kThreads;
     const int *lc = c->S.l_col, *uc = c->S.u_col;
     // rows are final after the top level (modes 2, 3, 5) and the backward
@@ -554,7 +567,7 @@ void desc_sweeps(ddlr_ctx *c, cudaStream_t st, const char *fam, const T *lv0, co
         const int cnt = ptr[L + 1] - ptr[L];
         if (cnt > 0)
           KL(c, fam, st, (k_sptrsv_two<T, decltype(mode)::value, TX>), (cnt + kThreads - 1) / kThreads, kThreads, 0,
-             c->lv_desc + ptr[L], cnt, col, val, di, x, z, gate, z64);
+             desc + ptr[L], cnt, col, val, di, x, z, gate, z64);
       };
       if (lx) two(std::integral_constant<int, 5>{}, 1, c->S.l_col, lx);
       else two(std::integral_constant<int, 3>{}, 1, c->S.l_col, lv0);
@@ -623,9 +636,10 @@ void cheb_tail(ddlr_ctx *c, cudaStream_t st, const T *x, T *z, int R, const int 
 // z = A0^-1 x in device order (Sec. 4.2: the p local solves with B_{i,a} and
 // the solve with C_a).  Shallow factors (multicolour orders): every level of
 // all blocks in one launch.  Deep factors: all interior blocks in one launch
-// (CTA per block) on the main stream, the C_a levels on a forked stream.
+// (CTA per block) on the main stream, the C_a levels on a forked stream.  e_only:
+// see desc_sweeps.
 template <typename T>
-void a0_solve(ddlr_ctx *c, const T *x, T *z, const int *gate) {
+void a0_solve(ddlr_ctx *c, const T *x, T *z, const int *gate, bool e_only = false) {
   const Plan &P = c->P;
   const T *lv = Prec<T>::l(c), *uv = Prec<T>::u(c), *di = Prec<T>::dinv(c);
   if (c->opt.factor >= 2) {
@@ -646,7 +660,7 @@ void a0_solve(ddlr_ctx *c, const T *x, T *z, const int *gate) {
   }
   const bool cheb = c->opt.c_solver == 1;
   if (std::max(P.levels_interior, P.levels_c) <= kShallowLevels) {
-    if (c->lv_desc) desc_sweeps<T>(c, c->stream, "sptrsv_levels", lv, uv, di, x, z, gate);
+    if (c->lv_desc) desc_sweeps<T>(c, c->stream, "sptrsv_levels", lv, uv, di, x, z, gate, nullptr, e_only);
     else chunk_sweeps<T>(c, c->stream, P.ch_all_ptr, "sptrsv_levels", lv, uv, di, x, z, gate);
     if (cheb) cheb_tail<T>(c, c->stream, x, z, 1, gate);
     else if (c->opt.c_solver == 2) mr_apply_c<T>(c, c->stream, x, z, 1, gate);
@@ -810,7 +824,7 @@ void apply_dev(ddlr_ctx *c, const TU *U, const T *x, T *u, const int *gate) {
   if (c->opt.variant == 1) {
     T *z = Prec<T>::w(c, 0), *y = Prec<T>::w(c, 1), *w = Prec<T>::w(c, 2), *rhs = Prec<T>::w(c, 3);
     T *t = Prec<T>::w(c, 4);
-    a0_solve<T>(c, x, z, gate);                                      // A0 z = x
+    a0_solve<T>(c, x, z, gate, true);                                // A0 z = x where E^T reads it
     KL(c, "et", c->stream, k_et<T>, nblk(s), kThreads, 0,            // y = E^T z
        s, m, c->eht_rp, c->eht_ci, Prec<T>::eht(c), ia, a, z, y, gate);
     launch_utx<T, TU>(c, s, k, U, y, part, Prec<T>::coef(c), (const T *)nullptr, t, gate);   // t = D U^T y
@@ -853,7 +867,7 @@ void apply_dev_x64(ddlr_ctx *c, const TU *U, const double *x, double *u64, const
   float *part = c->part32;
   float *z = c->w32[0], *y = c->w32[1], *w = c->w32[2], *rhs = c->w32[3], *t = c->w32[4], *u = c->w32[7];
   const float *lv = c->l32, *uv = c->u32, *di = c->dinv32;
-  desc_sweeps<float, double>(c, c->stream, "sptrsv_levels", lv, uv, di, x, z, gate);     // A0 z = x
+  desc_sweeps<float, double>(c, c->stream, "sptrsv_levels", lv, uv, di, x, z, gate, nullptr, true);   // A0 z = x
   KL(c, "et", c->stream, k_et<float>, nblk(s), kThreads, 0, s, m, c->eht_rp, c->eht_ci, c->eht32, ia, a, z, y,
      gate);                                                                               // y = E^T z
   launch_utx<float, TU>(c, s, k, U, y, part, c->coef32, (const float *)nullptr, t, gate);   // t = D U^T y
@@ -942,9 +956,9 @@ void lanczos_step(ddlr_ctx *c, const LzBufs &L) {
   const size_t csm = size_t(L.mmax + 2) * sizeof(double);
   KL(c, "e_vec", c->stream, k_e_vec<double>, nblk(n), kThreads, 0,
      m, s, c->eh_rp, c->eh_ci, c->eh64, ia, a, L.qcur, (const double *)nullptr, v, stop);
-  a0_solve<double>(c, v, z, stop);
+  a0_solve<double>(c, v, z, stop, c->opt.variant == 1);
   if (c->opt.variant == 2) {
-    a0_solve<double>(c, z, v, stop);
+    a0_solve<double>(c, z, v, stop, true);
     std::swap(v, z);
   }
   KL(c, "et", c->stream, k_et<double>, nblk(s), kThreads, 0, s, m, c->eht_rp, c->eht_ci, c->eht64, ia, a, z,
@@ -1171,7 +1185,8 @@ ddlr_status run_lanczos(ddlr_ctx *c, bool resume = false) {
       double a0 = 0;
       ddlr_get_traffic(c, nullptr, &a0, nullptr, 0);
       const double ne = double(P.nnz_ehat), sd = double(s) * 8.0, nd = double(n) * 8.0;
-      const double step = ne * 12.0 + sd + nd + (c->opt.variant == 2 ? 2.0 : 1.0) * a0 + ne * 12.0 + nd + sd +
+      const double step = ne * 12.0 + sd + nd + (c->opt.variant == 2 ? 2.0 : 1.0) * a0 - e_rows_saved(c, 8.0) +
+                          ne * 12.0 + nd + sd +
                           8.0 * sd;
       const double steps = double(hs.j);
       c->pz_lz_bytes += steps * (step + 4.0 * s) + sd * hs.qcols64 + 4.0 * s * hs.qcols32;
@@ -1584,7 +1599,7 @@ const int *pcg_gate(ddlr_ctx *c) {
 
 void batch_alloc(ddlr_ctx *c, int R);
 template <typename T>
-void a0_solve_mr(ddlr_ctx *c, const T *X, T *Z, int R, const int *gate);
+void a0_solve_mr(ddlr_ctx *c, const T *X, T *Z, int R, const int *gate, bool e_only = false);
 
 // H_k = (I - U_k^T E V_k)^-1 for DDLR-2 from the partial sums of its products:
 // Cholesky (an I - K that is not positive definite sets the NOT_SPD flag,
@@ -2164,6 +2179,11 @@ PzOp<T, TU> make_pzop(ddlr_ctx *c) {
   O.a = c->opt.alpha; O.ia = 1.0 / c->opt.alpha;
   for (int i = 0; i <= O.nL; i++) O.lvl_ptr[i] = P.lv_ptr[i];
   O.desc = c->lv_desc;
+  if (c->e_desc) {
+    O.desc_e = c->e_desc + c->e_ptr[1];
+    O.cnt_e = c->e_ptr[2] - c->e_ptr[1];
+  }
+  O.u_span = c->u_span;
   O.l_col = c->S.l_col;
   O.u_col = c->S.u_col;
   O.lval = Prec<T>::l(c); O.uval = Prec<T>::u(c); O.dinv = Prec<T>::dinv(c);
@@ -2280,6 +2300,29 @@ bool gmres_persist_t(ddlr_ctx *c, const double *b, double *x, double tol, int ma
                        args);
 }
 
+// the descriptors of the rows that E^T A0^-1 needs (two-level factors); DDLR_E_ROWS=0:
+// all rows are solved for
+void e_rows_setup(ddlr_ctx *c) {
+  const Plan &P = c->P;
+  const char *env = getenv("DDLR_E_ROWS");
+  if (!c->lv_desc || P.lv_ptr.size() != 3 || c->opt.factor >= 2 || (env && env[0] == '0')) return;
+  const int n = P.n, p1 = P.lv_ptr[1], ne = int(P.eht_ci.size());
+  const int nb0 = (p1 + kThreads - 1) / kThreads, nb = nb0 + (n - p1 + kThreads - 1) / kThreads;
+  unsigned char *mark = c->alloc<unsigned char>(n);
+  int *cnt = c->alloc<int>(nb + 1);
+  unsigned long long *tot = c->alloc<unsigned long long>(3), h[3];
+  ck(cudaMemsetAsync(mark, 0, n, c->stream), "memset");
+  ck(cudaMemsetAsync(tot, 0, sizeof(h), c->stream), "memset");
+  if (ne > 0) KL(c, "setup", c->stream, k_erow_mark, (ne + kThreads - 1) / kThreads, kThreads, 0, ne, c->eht_ci, mark);
+  KL(c, "setup", c->stream, k_erow_count, nb, kThreads, 0, c->lv_desc, nb0, p1, n, P.m, c->S.l_col, mark, cnt, tot + 2);
+  KL(c, "setup", c->stream, k_erow_scan, 1, 1024, 0, nb, nb0, cnt, tot);
+  read_dev(c, h, tot, sizeof(h));
+  c->e_desc = c->alloc<int4>(size_t(h[1]) + 1);
+  c->e_ptr = {0, int(h[0]), int(h[1])};
+  c->e_entries = double(h[2]);
+  KL(c, "setup", c->stream, k_erow_list, nb, kThreads, 0, c->lv_desc, nb0, p1, n, P.m, c->S.l_col, mark, cnt, c->e_desc);
+}
+
 // grid barriers of one PCG iteration and of one Lanczos step, upper bounds
 int pz_barriers_per_iteration(const ddlr_ctx *c) {
   const int nL = int(c->P.ch_all_ptr.size()) - 1;
@@ -2381,6 +2424,7 @@ void allocate(ddlr_ctx *c) {
   int mmax = c->opt.lanczos_max > 0 ? c->opt.lanczos_max : 5 * k;
   mmax = std::max(std::min(mmax, P.s), k);
   c->part64 = c->alloc<double>(size_t(kRedGrid) * std::max(k + 2, mmax + 2) + 2 * kRedGrid);
+  e_rows_setup(c);
   pz_setup(c, mmax);
   panel_plan<double>(c, 0);
   deep_plan<double>(c, 0);
@@ -2863,12 +2907,14 @@ inline int batch_width(const ddlr_ctx *c) {
 
 // Z = A0^-1 X for a block of R vectors: every level of all blocks per launch
 template <typename T>
-void a0_solve_mr(ddlr_ctx *c, const T *X, T *Z, int R, const int *gate) {
+void a0_solve_mr(ddlr_ctx *c, const T *X, T *Z, int R, const int *gate, bool e_only) {
   const Plan &P = c->P;
   const T *lv0 = Prec<T>::l(c), *lx = Prec<T>::lx(c), *uv = Prec<T>::u(c), *di = Prec<T>::dinv(c);
   const std::vector<int> &ptr = P.ch_all_ptr;
   const int nL = int(ptr.size()) - 1;
-  const std::vector<int> &dptr = P.lv_ptr;
+  const bool only = e_only && c->e_desc;
+  const std::vector<int> &dptr = only ? c->e_ptr : P.lv_ptr;
+  const int4 *desc = only ? c->e_desc : c->lv_desc;
   auto launch = [&](int L, int mode) {
     const T *lv = mode == 5 ? lx : lv0;
     if (c->lv_desc) {
@@ -2879,12 +2925,12 @@ void a0_solve_mr(ddlr_ctx *c, const T *X, T *Z, int R, const int *gate) {
         // 16-byte vectors of kV columns per thread; 256 threads
         const int per = 256 / (R / kV), rows = per * kMrRowsPerThread<T>;
         KL(c, "sptrsv_levels_mr", c->stream, k_sptrsv_desc_mr_v<T>, (cnt + rows - 1) / rows, per * (R / kV), 0,
-           c->lv_desc + dptr[L], cnt, mode, c->S.l_col, c->S.u_col, lv, uv, di, X, Z, R, gate);
+           desc + dptr[L], cnt, mode, c->S.l_col, c->S.u_col, lv, uv, di, X, Z, R, gate);
         return;
       }
       const int bd = chunk_block(c, R), rows = (bd / R) * kMrRowsPerThread<T>;
       KL(c, "sptrsv_levels_mr", c->stream, k_sptrsv_desc_mr<T>, (cnt + rows - 1) / rows, bd, 0,
-         c->lv_desc + dptr[L], cnt, mode, c->S.l_col, c->S.u_col, lv, uv, di, X, Z, R, gate);
+         desc + dptr[L], cnt, mode, c->S.l_col, c->S.u_col, lv, uv, di, X, Z, R, gate);
       return;
     }
     const int nch = ptr[L + 1] - ptr[L];
@@ -2940,7 +2986,7 @@ void apply_mr(ddlr_ctx *c, const TU *U, const T *X, T *Out, int R, const int *ga
   T *part = BPrec<T>::part(c), *Tm = BPrec<T>::w(c, 4);
   if (c->opt.variant == 1) {
     T *Z = BPrec<T>::w(c, 0), *Y = BPrec<T>::w(c, 1), *W = BPrec<T>::w(c, 2), *RHS = BPrec<T>::w(c, 3);
-    a0_solve_mr<T>(c, X, Z, R, gate);
+    a0_solve_mr<T>(c, X, Z, R, gate, true);
     constexpr int kV = Vec16<T>::n;
     const bool vec = R % kV == 0;
     if (vec)
@@ -4158,11 +4204,15 @@ ddlr_status ddlr_reset_counters(ddlr_handle c) {
 // k_sptrsv_*_mr): the off-diagonal factor entries and the inverse diagonal once
 // per sweep, every column read and written once per sweep (gathered reads of
 // other rows as cache hits)
+// (DDLR-1: the mean of a full solve and one of the rows that E^T reads)
 static double batch_a0_bytes(const ddlr_ctx *c, double R) {
   const Plan &P = c->P;
   const double v = c->opt.precision == 1 ? 4.0 : 8.0;
   const double off = double(P.nnz_factor) - double(P.n);
-  return 2.0 * (off * (v + 4.0) + double(P.n) * v + 2.0 * double(P.n) * R * v);
+  const double full = 2.0 * (off * (v + 4.0) + double(P.n) * v + 2.0 * double(P.n) * R * v);
+  if (!c->e_desc || c->opt.variant != 1) return full;
+  const double part = c->e_entries * (v + 4.0) + 2.0 * double(c->e_ptr[2]) * (v + 2.0 * R * v);
+  return 0.5 * (full + part);
 }
 static double batch_a0_launches(const ddlr_ctx *c) {
   const int nL = int(c->P.ch_all_ptr.size()) - 1;
@@ -4204,7 +4254,7 @@ ddlr_status ddlr_get_traffic(ddlr_handle c, double *apply_bytes, double *a0_byte
   const double wr = s * k * ub + 4.0 * s * v;
   const double ei = ne * (v + 4.0) + 4.0 * m + 2.0 * m * v;
   const double uadd = n * k * ub + 2.0 * n * v;
-  const double apply = c->opt.variant == 1 ? 2.0 * a0 + et + utx + wr + ei : a0 + utx + uadd;
+  const double apply = c->opt.variant == 1 ? 2.0 * a0 - e_rows_saved(c, v) + et + utx + wr + ei : a0 + utx + uadd;
   if (apply_bytes) *apply_bytes = apply;
   if (a0_bytes) *a0_bytes = a0;
   if (family_bytes) {
@@ -4218,7 +4268,8 @@ ddlr_status ddlr_get_traffic(ddlr_handle c, double *apply_bytes, double *a0_byte
       const std::string &f = c->fam_names[i];
       double b = 0.0;
       if (f == "sptrsv_blocks") b = blocks;
-      else if (f == "sptrsv_levels") b = (blocks + cblk) / sweeps(std::max(P.levels_interior, P.levels_c));
+      else if (f == "sptrsv_levels") b = (blocks + cblk - (c->opt.variant == 1 ? 0.5 * e_rows_saved(c, v) : 0.0)) /
+            sweeps(std::max(P.levels_interior, P.levels_c));
       else if (f == "sptrsv_c" || f == "cheb_dsolve") b = cblk / clev;
       else if (f == "cheb") b = cheb_k / t;
       else if (f == "mr_apply") b = mr_k;

@@ -96,6 +96,9 @@ struct PzOp {
   double a, ia;
   int lvl_ptr[kPzMaxLevels + 1];       // level-order descriptor offsets, levels of all blocks
   const int4 *desc;                    // {row, first L slot, first L^T slot, counts} per row
+  const int4 *desc_e;                  // two levels: the top level's rows of a solve that only E^T reads
+  int cnt_e;                           // (desc_e == nullptr: such a solve is done in full)
+  const int2 *u_span;                  // {first slot, entries} of a row of L^T
   const int *l_col, *u_col;            // sliced-ELL columns of L and L^T
   const T *lval, *uval, *dinv;
   const int *eh_rp, *eh_ci;
@@ -366,14 +369,13 @@ __device__ __forceinline__ void pz_out(const PzOut &o, int r, T z) {
 // 1, 2) add racc_r (zsc_r z_r) to acc when racc is given; z2 (level 0,
 // backward) receives the first forward level of a solve whose input is z.
 template <int NT, bool OUT = false, typename T, typename TU, typename TX>
-__device__ __forceinline__ void pz_level(const PzOp<T, TU> &O, int L, int mode, const TX *x, const double *xsc,
-                                         T *z, const double *racc, const double *zsc, double &acc, T *z2,
-                                         const PzOut &po = PzOut{}) {
-  const int c0 = O.lvl_ptr[L];
+__device__ __forceinline__ void pz_rows(const PzOp<T, TU> &O, const int4 *desc, int cnt, int mode, const TX *x,
+                                        const double *xsc, T *z, const double *racc, const double *zsc, double &acc,
+                                        T *z2, const PzOut &po = PzOut{}) {
   int v0, v1;
-  pz_range(O.lvl_ptr[L + 1] - c0, v0, v1);        // a level's rows over all CTAs
+  pz_range(cnt, v0, v1);                          // a level's rows over all CTAs
   for (int v = v0 + threadIdx.x; v < v1; v += NT) {
-    const int4 d = ro(O.desc + c0 + v);
+    const int4 d = ro(desc + v);
     const int r = d.x;
     T zr;
     const T dr = ro(O.dinv + r);
@@ -396,6 +398,13 @@ __device__ __forceinline__ void pz_level(const PzOp<T, TU> &O, int L, int mode, 
   }
 }
 
+template <int NT, bool OUT = false, typename T, typename TU, typename TX>
+__device__ __forceinline__ void pz_level(const PzOp<T, TU> &O, int L, int mode, const TX *x, const double *xsc,
+                                         T *z, const double *racc, const double *zsc, double &acc, T *z2,
+                                         const PzOut &po = PzOut{}) {
+  pz_rows<NT, OUT>(O, O.desc + O.lvl_ptr[L], O.lvl_ptr[L + 1] - O.lvl_ptr[L], mode, x, xsc, z, racc, zsc, acc, z2, po);
+}
+
 // z = A0^-1 x (Sec. 4.2), x read as pz_in, phases separated by grid barriers;
 // the last phase is left open (the caller adds its own work and barrier).
 // l0_done: the producer of x has already done the first forward level
@@ -415,6 +424,42 @@ __device__ __forceinline__ bool pz_a0(const PzOp<T, TU> &O, const TX *x, const d
     pz_level<NT, OUT>(O, L, 1, x, xsc, z, racc, zsc, acc, L == 0 ? z2 : (T *)nullptr, po);
   }
   return true;
+}
+
+// y = E^T A0^-1 x at interface row j, in the two halves around a grid barrier.
+// Two levels (desc_e): the first half is the top level's rows that E^T needs; the
+// second forms the backward rows where E^T reads them (a row next to two interface
+// nodes twice), with the arithmetic of pz_level, so the backward phase and its
+// barrier are not there and the rows that nothing reads are not computed.  The
+// producer of x has done the first forward level (pz_l0).  Otherwise the whole
+// solve precedes.  Setup and solve 64^3 DDLR-2 29.7 -> 28.9 ms, 128^3 120.9 ->
+// 118.8, GMRES at 32^3 7.80 -> 7.59; 32^3 PCG 2.79 -> 2.78 (the phase that is gone
+// is paid for by the longer chain of loads in the one that is left).
+template <int NT, typename T, typename TU, typename TX>
+__device__ __forceinline__ bool pz_et_a0(const PzOp<T, TU> &O, const TX *x, const double *xsc, T *z, unsigned &ep,
+                                         bool l0_done) {
+  double dummy = 0;
+  if (O.desc_e) pz_rows<NT>(O, O.desc_e, O.cnt_e, 2, x, xsc, z, nullptr, nullptr, dummy, (T *)nullptr);
+  else if (!pz_a0<NT>(O, x, xsc, z, nullptr, nullptr, dummy, ep, l0_done)) return false;
+  return pz_sync(O.gs, ep);
+}
+template <typename T, typename TU>
+__device__ __forceinline__ T pz_zfin(const PzOp<T, TU> &O, const T *z, int r) {
+  T t = z[r];
+  if (O.desc_e && ro(O.lvl0 + r)) {
+    const int2 sp = ro(O.u_span + r);
+    const T dr = ro(O.dinv + r);
+    for (int kk = 0; kk < sp.y; kk++) t -= ro(O.uval + sp.x + kk * 32) * z[ro(O.u_col + sp.x + kk * 32)];
+    t = t * dr;
+  }
+  return t;
+}
+template <typename T, typename TU>
+__device__ __forceinline__ T pz_et_row(const PzOp<T, TU> &O, const T *z, int j, T a, T ia) {
+  T t = 0;
+  const int q1 = ro(O.eht_rp + j + 1);
+  for (int q = ro(O.eht_rp + j); q < q1; q++) t += ro(O.eht + q) * pz_zfin(O, z, ro(O.eht_ci + q));
+  return ia * t - a * pz_zfin(O, z, O.m + j);
 }
 
 // u = M^-1 (dsc .* x) in precision T without the final dsc scaling, DDLR-1
@@ -445,18 +490,11 @@ __device__ __forceinline__ bool pz_apply(const PzOp<T, TU> &O, const double *x, 
     }
     return true;
   }
-  double dummy = 0;
-  if (!pz_a0<NT>(O, x, xsc, z, nullptr, nullptr, dummy, ep, l0_done)) return false;
-  if (!pz_sync(O.gs, ep)) return false;
+  if (!pz_et_a0<NT>(O, x, xsc, z, ep, l0_done)) return false;
   const T a = T(O.a), ia = T(O.ia);
   int j0, j1;
   pz_range(s, j0, j1);
-  for (int j = j0 + threadIdx.x; j < j1; j += NT) {                // y = E^T z
-    T t = 0;
-    const int q1 = ro(O.eht_rp + j + 1);
-    for (int q = ro(O.eht_rp + j); q < q1; q++) t += ro(O.eht + q) * z[ro(O.eht_ci + q)];
-    y[j] = ia * t - a * z[m + j];
-  }
+  for (int j = j0 + threadIdx.x; j < j1; j += NT) y[j] = pz_et_row(O, z, j, a, ia);   // y = E^T z
   __syncthreads();
   double *pt = pz_buf(O, slot++);
   pz_utx<NT, T>(k, O.U, y, (const double *)nullptr, j0, j1, pt, O.pstride, red);   // D U^T y, this CTA's rows
@@ -965,24 +1003,22 @@ __global__ void __launch_bounds__(NT, 1) k_lz_persist(PzOp<double, double> O, Pz
       if (!pz_sync(O.gs, ep)) return;
     }
     have_v = false;
-    double dummy = 0;
     const bool f0 = O.fuse0 != 0;
-    // DDLR-2: the first solve's last level also does the second's first
-    if (!pz_a0<NT>(O, v, nullptr, z, nullptr, nullptr, dummy, ep, f0, O.variant == 2 && f0 ? v : nullptr)) return;
-    if (!pz_sync(O.gs, ep)) return;
     double *res = z;
     if (O.variant == 2) {
-      if (!pz_a0<NT>(O, z, nullptr, v, nullptr, nullptr, dummy, ep, f0)) return;
+      // DDLR-2: the first solve's last level also does the second's first
+      double dummy = 0;
+      if (!pz_a0<NT>(O, v, nullptr, z, nullptr, nullptr, dummy, ep, f0, f0 ? v : nullptr)) return;
       if (!pz_sync(O.gs, ep)) return;
+      if (!pz_et_a0<NT>(O, z, (const double *)nullptr, v, ep, f0)) return;
       res = v;
+    } else if (!pz_et_a0<NT>(O, v, (const double *)nullptr, z, ep, f0)) {
+      return;
     }
     // w = E^T res, alpha_j = q_j . w
     double acc = 0;
     for (int r = j0 + threadIdx.x; r < j1; r += NT) {
-      double t = 0;
-      const int q1 = ro(O.eht_rp + r + 1);
-      for (int q = ro(O.eht_rp + r); q < q1; q++) t += ro(O.eht + q) * res[ro(O.eht_ci + q)];
-      const double wr = O.ia * t - O.a * res[m + r];
+      const double wr = pz_et_row(O, res, r, O.a, O.ia);
       L.w[r] = wr;
       acc += L.qcur[r] * wr;
     }
