@@ -2862,10 +2862,10 @@ void batch_alloc(ddlr_ctx *c, int R) {
     // the tensor-core U_k^T Y writes kTcRedGrid partials plus a k x R sum
     B.part32 = (float *)al((size_t(kTcRedGrid) + 1) * std::max<size_t>(k * R, 2 * R) * 4);
   }
-  B.part64 = (double *)al(size_t(kRedGrid) * std::max<size_t>(k * R, 2 * R) * 8);
+  B.part64 = (double *)al(size_t(kRedGrid + kMrRedGroups) * std::max<size_t>(k * R, 2 * R) * 8);
   B.fpart = (double *)al(std::max(size_t((P.n + kFbRows - 1) / kFbRows), size_t(2 * kRedGrid * kDotSub)) * R * 8);
-  B.count = (unsigned *)al(16);
-  ck(cudaMemsetAsync(B.count, 0, 16, c->stream), "memset");
+  B.count = (unsigned *)al((1 + kMrRedGroups) * sizeof(unsigned));
+  ck(cudaMemsetAsync(B.count, 0, (1 + kMrRedGroups) * sizeof(unsigned), c->stream), "memset");
   if (c->opt.c_solver == 1)
     for (int i = 0; i < 5; i++) {
       B.cb64[i] = (double *)al(nR * 8);
@@ -2928,8 +2928,10 @@ void a0_solve_mr(ddlr_ctx *c, const T *X, T *Z, int R, const int *gate, bool e_o
            desc + dptr[L], cnt, mode, c->S.l_col, c->S.u_col, lv, uv, di, X, Z, R, gate);
         return;
       }
-      const int bd = chunk_block(c, R), rows = (bd / R) * kMrRowsPerThread<T>;
-      KL(c, "sptrsv_levels_mr", c->stream, k_sptrsv_desc_mr<T>, (cnt + rows - 1) / rows, bd, 0,
+      const int bd = chunk_block(c, R);
+      const int rr = (long long)cnt * R < kMrScalarWide ? 1 : kMrRowsScalar<T>, rows = (bd / R) * rr;
+      const auto fn = rr == 1 ? k_sptrsv_desc_mr<T, 1> : k_sptrsv_desc_mr<T, kMrRowsScalar<T>>;
+      KL(c, "sptrsv_levels_mr", c->stream, fn, (cnt + rows - 1) / rows, bd, 0,
          desc + dptr[L], cnt, mode, c->S.l_col, c->S.u_col, lv, uv, di, X, Z, R, gate);
       return;
     }

@@ -89,12 +89,18 @@ __global__ void k_sptrsv_chunks_mr(SolveLayout S, const int4 *chunks, int mode,
 // cost more than the loads in flight give (64^3 x 8: 24.5, 25.3 and 30.4 us;
 // 96^3 x 16: 117, 120 and 152; 128^3 x 4: 78, 79 and 98).
 template <typename T> constexpr int kMrRowsPerThread = sizeof(T) == 8 ? 1 : 2;
-template <typename T>
+// The scalar form (widths that are not whole vectors) shares less per row: FP32 takes
+// four rows where the level fills the chip that way, one below kMrScalarWide
+// elements (solves, 1, 2 and 4 rows: 24^3 x 31 6.62, 6.77 and 6.81 ms; 40^3 x 7 all
+// 9.7; 40^3 x 13 12.2, 12.1 and 11.6; 64^3 x 5 23.5, 22.8 and 22.0; 64^3 x 31 79.9,
+// 72.8 and 68.2).
+template <typename T> constexpr int kMrRowsScalar = sizeof(T) == 8 ? 1 : 4;
+constexpr long long kMrScalarWide = 300000;
+template <typename T, int RR>
 __global__ void k_sptrsv_desc_mr(const int4 *desc, int count, int mode, const int *l_col, const int *u_col,
                                  const T *lval, const T *uval, const T *dinv, const T *X, T *Z, int R,
                                  const int *gate) {
   if (gate && *gate) return;
-  constexpr int RR = kMrRowsPerThread<T>;
   const int per = blockDim.x / R;
   const int q = threadIdx.x % R, sub = threadIdx.x / R;
   if (sub >= per) return;
@@ -1094,11 +1100,17 @@ __device__ __forceinline__ void mr_step(PcgStateMR *st, const double *sm) {
 
 // Second stage of a column reduction and the scalar step: CTA g of kRedGrid adds
 // the rows of range g of bpart (row blocks; kDotSub per range after
-// k_dot_rz_mr) in order into partials[g][o], o < no; the CTA that arrives last
-// (counter, no waiting) adds the ranges as col_sums does and takes step S.  One
-// launch instead of two.  The rows are staged in shared memory by all threads,
+// k_dot_rz_mr) in order into partials[g][o], o < no.  The ranges are added as
+// col_sums does, by arrival (counters, no waiting): the last CTA of ranges j, j +
+// 32, ... adds those, what lane j of a warp of col_sums adds, and the last of these
+// 32 CTAs adds their sums in the order of its shuffle tree and takes step S.  All of
+// it in one CTA took FP64 issue slots: 304 adds per column, 64 cycles a warp and
+// sub-partition each, 8 us at 62 columns (24^3 x 31, mixed: a solve 8.12 -> 6.8 ms, 64^3 x 31 73.3 -> 68.2).
+// One launch instead of two.  The rows are staged in shared memory by all threads,
 // so that one load latency precedes the serial adds instead of one per few.
-constexpr int kMrRedNT = 512, kMrStage = 2048;
+// count: 1 + kMrRedGroups counters, 0 between launches; partials: the ranges' rows,
+// then those of the groups.
+constexpr int kMrRedNT = 256, kMrStage = 2048, kMrRedGroups = 32;
 template <MrStep S>
 __global__ void __launch_bounds__(kMrRedNT)
 k_reduce_step_mr(int nrows, int no, const double *bpart, double *partials, PcgStateMR *st, unsigned *count,
@@ -1122,11 +1134,52 @@ k_reduce_step_mr(int nrows, int no, const double *bpart, double *partials, PcgSt
   if (threadIdx.x < no) partials[(long long)blockIdx.x * 2 * R + threadIdx.x] = v;
   __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) last = atomicAdd(count, 1u) == gridDim.x - 1;
+  static_assert(kRedGrid >= kMrRedGroups, "no empty group");
+  const int G = gridDim.x, grp = blockIdx.x % kMrRedGroups;
+  if (threadIdx.x == 0) {
+    last = atomicAdd(count + 1 + grp, 1u) == unsigned((G - grp + kMrRedGroups - 1) / kMrRedGroups) - 1u;
+    if (last) count[1 + grp] = 0u;
+  }
   __syncthreads();
   if (!last) return;
   __threadfence();
-  col_sums(partials, gridDim.x, R, no, sm);
+  double *gsum = partials + (long long)G * 2 * R;
+  if (threadIdx.x < no) {
+    v = 0.0;
+#pragma unroll 10
+    for (int g = grp; g < G; g += kMrRedGroups) v += __ldcg(partials + (long long)g * 2 * R + threadIdx.x);
+    gsum[(long long)grp * 2 * R + threadIdx.x] = v;
+  }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(count, 1u) == kMrRedGroups - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  constexpr int CW = kMrStage / kMrRedGroups;         // columns of a pass
+  for (int c0 = 0; c0 < no; c0 += CW) {
+    const int w = min(CW, no - c0);
+    for (int i = threadIdx.x; i < kMrRedGroups * w; i += kMrRedNT)
+      stage[i] = __ldcg(gsum + (long long)(i / w) * 2 * R + c0 + i % w);
+    __syncthreads();
+    // four threads per column: strides 16, 8 and 4 of the tree are a thread's own
+    for (int i0 = 0; i0 < 4 * w; i0 += kMrRedNT) {
+      const int i = i0 + threadIdx.x, c = min(i >> 2, w - 1), part = i & 3;
+      if (i0 + (threadIdx.x & ~31) < 4 * w) {
+        double t[8];
+#pragma unroll
+        for (int q = 0; q < 8; q++) t[q] = stage[(part + 4 * q) * w + c];
+#pragma unroll
+        for (int h = 4; h > 0; h >>= 1)
+#pragma unroll
+          for (int q = 0; q < h; q++) t[q] += t[q + h];
+        t[0] += __shfl_down_sync(0xffffffffu, t[0], 2, 4);
+        t[0] += __shfl_down_sync(0xffffffffu, t[0], 1, 4);
+        if (part == 0 && i < 4 * w) sm[c0 + c] = t[0];
+      }
+    }
+    __syncthreads();
+  }
   mr_step<S>(st, sm);
   if (threadIdx.x == 0) *count = 0u;
 }
