@@ -386,7 +386,15 @@ k_deep_solve(DeepGeo g, const unsigned char *pk_l, const unsigned char *pk_u, co
     if (ln < sr.y) z[sr.x + ln] = zs[i * 32 + ln];
   }
   __syncwarp();
-  if (g.ctas > 1) cluster_sync_all();
+  if (g.ctas > 1) {
+    cluster_sync_all();
+    if (is_late()) {
+      // its peers' last pushes into this CTA, which it no longer counts, may be
+      // under way (they take about 1 us)
+      const unsigned long long t0 = gtimer_ns();
+      while (gtimer_ns() - t0 < 50000ull) {}
+    }
+  }
 }
 
 // ------------------------------------------------------------ narrow blocks
