@@ -262,7 +262,8 @@ struct ddlr_ctx {
   // persistent cooperative kernels (shallow factors): one CTA per SM
   double *pz_part = nullptr;  // 3 x pz_grid x pz_pstride partial sums
   unsigned *pz_bar = nullptr; // grid-barrier arrival counter
-  unsigned *pz_bar2 = nullptr;// the same and the exit counter of the kernels that reset them (pz_exit)
+  unsigned *pz_bar2 = nullptr;// the same, the exit counter and the word that ends waits of the kernels that
+                              // leave them at 0 (pz_exit)
   unsigned char *pz_lvl0 = nullptr;  // rows on the first level of their block
   int pz_grid = 0, pz_pstride = 0, pz_mmax = 0;
   bool pz_pcg = false, pz_lz = false;
@@ -2153,8 +2154,8 @@ void pz_setup(ddlr_ctx *c, int mmax) {
   if (!c->pz_pcg && !c->pz_lz) return;
   c->pz_part = c->alloc<double>(size_t(3) * c->pz_grid * c->pz_pstride);
   c->pz_bar = c->alloc<unsigned>(1);
-  c->pz_bar2 = c->alloc<unsigned>(2);
-  ck(cudaMemsetAsync(c->pz_bar2, 0, 2 * sizeof(unsigned), c->stream), "memset");
+  c->pz_bar2 = c->alloc<unsigned>(3);
+  ck(cudaMemsetAsync(c->pz_bar2, 0, 3 * sizeof(unsigned), c->stream), "memset");
   std::vector<unsigned char> f0(P.n, 0);
   for (int b = 0; b + 1 < int(P.blk_lvl0.size()); b++) {
     const int l0 = P.blk_lvl0[b];
@@ -2196,7 +2197,7 @@ PzOp<T, TU> make_pzop(ddlr_ctx *c) {
   O.fuse0 = O.nL >= 2 ? 1 : 0;
   O.part = c->pz_part;
   O.gs.count = c->pz_bar;
-  O.gs.err = c->dflag + 3;
+  O.gs.err = O.gs.abort = c->dflag + 3;
   O.gs.wait_ns = c->wait_ns;
   // tests of the timeout path: DDLR_TEST_UNMET_BARRIER=1 makes the first grid
   // barrier of this launch wait for an arrival that never comes
@@ -2242,8 +2243,14 @@ bool pz_launch(ddlr_ctx *c, const char *fam, const void *fn, size_t smem, void *
   return true;
 }
 
-// a cooperative launch of a kernel that resets its counters itself, on `grid`
-// CTAs; false as for pz_launch
+// the barrier of the kernels that end with pz_exit: words of its own
+template <typename T, typename TU>
+void pz_own_barrier(ddlr_ctx *c, PzOp<T, TU> &O) {
+  O.gs.count = c->pz_bar2;
+  O.gs.abort = reinterpret_cast<int *>(c->pz_bar2 + 2);
+}
+
+// a cooperative launch of such a kernel on `grid` CTAs; false as for pz_launch
 bool pz_launch_own(ddlr_ctx *c, const char *fam, const void *fn, int grid, size_t smem, void **args) {
   ddlr_ctx::Scope sc(c, fam, c->stream);
   const char *fake = getenv("DDLR_FAKE_COOP_REFUSAL");
@@ -2269,7 +2276,7 @@ int pz_small_grid(const ddlr_ctx *c) {
 template <typename T, typename TU>
 bool apply_persist_t(ddlr_ctx *c, const double *x, double *y, T *u, T *z, T *v, T *w, T *rhs) {
   PzOp<T, TU> O = make_pzop<T, TU>(c);
-  O.gs.count = c->pz_bar2;
+  pz_own_barrier(c, O);
   PzApply<T> A{x, y, c->pv[1], c->perm, u, z, v, w, rhs};
   void *args[] = {&O, &A};
   return pz_launch_own(c, "apply_persist", (const void *)k_apply_persist<kPzThreads, T, TU>, pz_small_grid(c),
@@ -2289,7 +2296,7 @@ template <typename T, typename TU>
 bool gmres_persist_t(ddlr_ctx *c, const double *b, double *x, double tol, int maxit, int m, T *u, T *z, T *y, T *w,
                      T *rhs) {
   PzOp<T, TU> O = make_pzop<T, TU>(c);
-  O.gs.count = c->pz_bar2;
+  pz_own_barrier(c, O);
   O.pstride = c->gm.pz_stride;
   O.part = c->gm.pz_part;
   PzGm<T> P{b, x, c->pv[1], c->pv[3], c->gm.V, c->gm.Z, u, z, y, w, rhs, c->pcg, tol, maxit, m};
@@ -3385,7 +3392,6 @@ namespace {
 // and report DDLR_ERR_TIMEOUT
 void clear_timeout(ddlr_ctx *c) {
   cudaMemsetAsync(c->dflag + 3, 0, sizeof(int), c->stream);
-  if (c->pz_bar2) cudaMemsetAsync(c->pz_bar2, 0, 2 * sizeof(unsigned), c->stream);
   cudaStreamSynchronize(c->stream);
 }
 [[noreturn]] void timeout_fail(ddlr_ctx *c) {

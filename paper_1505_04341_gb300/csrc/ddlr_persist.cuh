@@ -30,11 +30,12 @@ constexpr int kPzMaxLevels = 8;          // deepest factor served (levels per bl
 template <typename T>
 __device__ __forceinline__ T ro(const T *p) { return __ldg(p); }
 
-// arrival counter of the grid barrier (zeroed before each launch) and the
-// shared timeout flag
+// arrival counter of the grid barrier (0 when a launch starts), the handle's
+// timeout flag, which the host reads and clears, and the word that ends the other
+// CTAs' waits: the flag itself, or (pz_exit) one that every launch leaves at 0
 struct GridSync {
   unsigned *count;
-  int *err;
+  int *err, *abort;
   unsigned long long wait_ns;   // wait limit of one barrier (the handle's wait_limit_s)
   int unmet;                    // tests: the first barrier waits for one arrival that
                                 // never comes, so it runs out after wait_ns
@@ -71,12 +72,13 @@ __device__ __forceinline__ bool pz_sync(const GridSync &g, unsigned &epoch) {
     unsigned it = 0;
     while (pz_ld_acquire(g.count) < target) {
       if ((++it & 63u) == 0) {
-        if (*(volatile int *)g.err) { ok = 0; break; }
+        if (*(volatile int *)g.abort) { ok = 0; break; }
         const unsigned long long t = pz_clock_ns();
         if (t0 == 0) {
           t0 = t;
         } else if (t - t0 > g.wait_ns) {
           atomicExch(g.err, 1);
+          atomicExch(g.abort, 1);
           ok = 0;
           break;
         }
@@ -523,16 +525,16 @@ __device__ __forceinline__ bool pz_apply(const PzOp<T, TU> &O, const double *x, 
   return pz_a0<NT, OUT>(O, rhs, (const double *)nullptr, u, racc, O.dsc, acc, ep, O.fuse0 != 0, (T *)nullptr, po);
 }
 
-// The last act of a kernel with a counter of its own: the CTA that leaves last
-// puts the barrier's counter and the exit counter behind it back to 0, so that
-// the next launch needs no memset (a launch of its own, as long as two phases).
-// Every CTA has passed its last barrier when the last one leaves.  A launch that
-// timed out leaves them as they are; the host clears them with the flag, and
-// until then a launch does nothing (pz_stale).
-__device__ __forceinline__ bool pz_stale(const GridSync &g) { return *(volatile int *)g.err != 0; }
+// The last act of a kernel with a counter of its own, by every CTA and on every
+// way out, a wait that ran out among them: the CTA that leaves last puts the
+// barrier's counter, the exit counter behind it and the word that ends waits
+// back to 0, so that the next launch needs no memset (a launch of its own, as long
+// as two phases) and finds nothing of one that timed out.  No CTA waits any more
+// when the last one leaves.
 __device__ __forceinline__ void pz_exit(const GridSync &g) {
   if (threadIdx.x != 0) return;
   if (atomicAdd(g.count + 1, 1u) == gridDim.x - 1) {
+    atomicExch(g.abort, 0);
     atomicExch(g.count, 0u);
     atomicExch(g.count + 1, 0u);
   }
@@ -552,7 +554,7 @@ struct PzApply {
   T *u, *z, *v, *w, *rhs;
 };
 template <int NT, typename T, typename TU>
-__global__ void __launch_bounds__(NT, 1) k_apply_persist(PzOp<T, TU> O, PzApply<T> A) {
+__device__ __forceinline__ void pz_apply_call(const PzOp<T, TU> &O, const PzApply<T> &A) {
   extern __shared__ double pz_sm[];
   double *red = pz_sm;
   T *vec = reinterpret_cast<T *>(pz_sm + NT + 32);
@@ -560,7 +562,6 @@ __global__ void __launch_bounds__(NT, 1) k_apply_persist(PzOp<T, TU> O, PzApply<
   int slot = 0, i0, i1;
   pz_range(O.n, i0, i1);
   T *a0out = O.variant == 2 ? A.u : A.z;
-  if (pz_stale(O.gs)) return;
   for (int i = i0 + threadIdx.x; i < i1; i += NT) {
     const double v = A.x[ro(A.perm + i)];
     A.xi[i] = v;
@@ -568,9 +569,12 @@ __global__ void __launch_bounds__(NT, 1) k_apply_persist(PzOp<T, TU> O, PzApply<
   }
   if (!pz_sync(O.gs, ep)) return;
   double acc = 0;
-  if (!pz_apply<NT, true>(O, A.xi, A.u, A.z, A.v, A.w, A.rhs, (const double *)nullptr, acc, ep, slot, red, vec,
-                          O.fuse0 != 0, PzOut{A.y, A.perm, O.dsc}))
-    return;
+  pz_apply<NT, true>(O, A.xi, A.u, A.z, A.v, A.w, A.rhs, (const double *)nullptr, acc, ep, slot, red, vec,
+                     O.fuse0 != 0, PzOut{A.y, A.perm, O.dsc});
+}
+template <int NT, typename T, typename TU>
+__global__ void __launch_bounds__(NT, 1) k_apply_persist(PzOp<T, TU> O, PzApply<T> A) {
+  pz_apply_call<NT>(O, A);
   pz_exit(O.gs);
 }
 
@@ -1149,7 +1153,7 @@ inline size_t pz_gm_smem(int k, int m) {
 }
 
 template <int NT, typename T, typename TU>
-__global__ void __launch_bounds__(NT, 1) k_gmres_persist(PzOp<T, TU> O, PzGm<T> P) {
+__device__ __forceinline__ void pz_gmres_call(const PzOp<T, TU> &O, const PzGm<T> &P) {
   extern __shared__ double pz_sm[];
   const int m = P.m, n = O.n;
   double *red = pz_sm, *bc = pz_sm + NT;
@@ -1168,7 +1172,6 @@ __global__ void __launch_bounds__(NT, 1) k_gmres_persist(PzOp<T, TU> O, PzGm<T> 
     return make_double2(b, 1.0 / b);
   };
   T *a0out = O.variant == 2 ? P.u : P.z;
-  if (pz_stale(O.gs)) return;
   double acc = 0;
   for (int i = i0 + threadIdx.x; i < i1; i += NT) {
     const double bi = P.b[i];
@@ -1317,6 +1320,10 @@ __global__ void __launch_bounds__(NT, 1) k_gmres_persist(PzOp<T, TU> O, PzGm<T> 
     P.st->rr = be.f.x;
     P.st->bb = bn;
   }
+}
+template <int NT, typename T, typename TU>
+__global__ void __launch_bounds__(NT, 1) k_gmres_persist(PzOp<T, TU> O, PzGm<T> P) {
+  pz_gmres_call<NT>(O, P);
   pz_exit(O.gs);
 }
 
