@@ -343,7 +343,9 @@ ddlr_status ddlr_set_stream(ddlr_handle h, void *cuda_stream);
  * sets a device flag, every CTA of the kernel returns, and the call that
  * launched it returns DDLR_ERR_TIMEOUT (its results are invalid); the flag is
  * cleared then, so the handle stays usable.  A call that does not wait for the
- * device (an apply into device memory) leaves it to the next one that does.  Errors: INVALID. */
+ * device (an apply into device memory) leaves it to the next solve, rebuild,
+ * ddlr_set_lowrank or apply into host memory, which returns it; the launches
+ * in between are not affected.  Errors: INVALID. */
 ddlr_status ddlr_set_wait_limit(ddlr_handle h, double seconds);
 
 /* Self-test of the library's binary64 <-> binary32 conversions written on the

@@ -1005,6 +1005,12 @@ void lanczos_step(ddlr_ctx *c, const LzBufs &L) {
   KL(c, "lanczos", c->stream, k_lz_advance, 1, 32, 0, L.st);
 }
 
+// the flags of a factorisation or a low-rank build; the timeout flag [3] stays
+// until the next call that waits has reported it
+void clear_flags(ddlr_ctx *c) { ck(cudaMemsetAsync(c->dflag, 0, 3 * sizeof(int), c->stream), "memset"); }
+// what such a call does instead of a plain sync
+void sync_or_timeout(ddlr_ctx *c);
+
 void hk_build(ddlr_ctx *c, int k, const double *EV, double *kp, double *hw);
 void ddlr2_columns(ddlr_ctx *c, int k, const double *V, double *EV, double *ev, double *uc);
 ddlr_status lowrank_status(ddlr_ctx *c, const int *fl);
@@ -1797,7 +1803,7 @@ ddlr_status run_lbd(ddlr_ctx *c) {
   KL(c, "ritz", c->stream, k_lbd_bmy, nblk((long long)mm * k), kThreads, 0, mm, k, B.al, B.be, B.eY, B.G);
   KL(c, "ritz", c->stream, k_ritz_gemm<16>, nblk(n), kThreads, 0, n, mm, k, B.Uq, (long long)n, B.G, c->U64);
   // H_k = (I - U_k^T E V_k)^-1
-  ck(cudaMemsetAsync(c->dflag, 0, 4 * sizeof(int), c->stream), "memset");
+  clear_flags(c);
   KL(c, "e_vec", c->stream, k_e_block, nblk((long long)n * k), kThreads, 0, m0, s, k, c->eh_rp, c->eh_ci, c->eh64,
      1.0 / a, a, B.Vk, B.EV);
   hk_build(c, k, B.EV, B.kp, B.hw);
@@ -1876,7 +1882,7 @@ ddlr_status run_randomized(ddlr_ctx *c) {
     KL(c, "rand_orth", c->stream, k_chol_inv, 1, kRandMaxL, 0, L, R.G, R.Linv, c->dflag + 0);
     KL(c, "rand_orth", c->stream, k_apply_rinv, nblk(s), kThreads, 0, (long long)s, L, Q, R.Linv, Y);
   };
-  ck(cudaMemsetAsync(c->dflag, 0, 4 * sizeof(int), c->stream), "memset");
+  clear_flags(c);
   KL(c, "rand_op", c->stream, k_rand_omega, nblk((long long)s * L), kThreads, 0, s, L, R.rank, c->opt.seed, R.Qb);
   op(R.Qb, R.Yb);
   orth(R.Yb, R.Qb);                       // Q in Yb
@@ -1894,6 +1900,7 @@ ddlr_status run_randomized(ddlr_ctx *c) {
   KL(c, "rand_eig", c->stream, k_back_transform, 1, 64, 0, L, k, R.Hv, R.eY);
   int fl[4];
   read_dev(c, fl, c->dflag, sizeof(fl));
+  if (fl[3]) { clear_timeout(c); return DDLR_ERR_TIMEOUT; }
   if (fl[0]) { c->err = "randomized range basis is rank-deficient (Cholesky QR failed)"; return DDLR_ERR_BREAKDOWN; }
   c->msteps = L;
   c->ritz.assign(L, 0.0);
@@ -2040,7 +2047,7 @@ ddlr_status numeric_setup(ddlr_ctx *c) {
   const int n = P.n;
   const long long nnz = P.nnz, nf = P.nnz_factor;
   const double a = c->opt.alpha;
-  ck(cudaMemsetAsync(c->dflag, 0, 4 * sizeof(int), c->stream), "memset");
+  clear_flags(c);
   if (c->opt.scale_diag) {
     KL(c, "setup", c->stream, k_diag_scale, nblk(n), kThreads, 0, n, c->diag_pos, c->val, c->dsc);
     KL(c, "setup", c->stream, k_scale_vals, nblk(nnz), kThreads, 0, nnz, c->orow, c->ocol, c->val, c->dsc, c->vals);
@@ -2423,6 +2430,7 @@ void allocate(ddlr_ctx *c) {
   ck(cudaMemsetAsync(c->Hk64, 0, sizeof(double) * k * k, c->stream), "memset");
   ck(cudaMemsetAsync(c->inv1mt64, 0, sizeof(double), c->stream), "memset");
   c->dflag = c->alloc<int>(4);
+  ck(cudaMemsetAsync(c->dflag, 0, 4 * sizeof(int), c->stream), "memset");
   c->udone = c->alloc<unsigned>(1);
   ck(cudaMemsetAsync(c->udone, 0, sizeof(unsigned), c->stream), "memset");
   c->pdone = c->alloc<unsigned>(1);
@@ -3379,7 +3387,7 @@ void batch_store(ddlr_ctx *c, const double *srcb, double *y, int ld, int R, bool
   if (host) {
     ck(cudaMemcpy2DAsync(y, sizeof(double) * size_t(ld), c->bt.S, sizeof(double) * n, sizeof(double) * n, R,
                          cudaMemcpyDeviceToHost, c->stream), "D2H");
-    sync(c);
+    sync_or_timeout(c);
   }
 }
 
@@ -3397,6 +3405,11 @@ void clear_timeout(ddlr_ctx *c) {
 [[noreturn]] void timeout_fail(ddlr_ctx *c) {
   clear_timeout(c);
   throw Fail{DDLR_ERR_TIMEOUT, "a bounded device wait timed out"};
+}
+void sync_or_timeout(ddlr_ctx *c) {
+  int timed_out;
+  read_dev(c, &timed_out, c->dflag + 3, sizeof(int));
+  if (timed_out) timeout_fail(c);
 }
 
 ddlr_status run_guarded(ddlr_ctx *c, const std::function<ddlr_status()> &f) {
@@ -3846,10 +3859,8 @@ static ddlr_status vec_call(ddlr_ctx *c, const double *x, double *y, int nrhs, i
       if (hy) yd = c->stg_out;
       body(xd, yd);
       if (hy) {
-        int timed_out;   // a device wait of this call or of one before it that did not wait
         ck(cudaMemcpyAsync(yj, yd, sizeof(double) * n, cudaMemcpyDeviceToHost, c->stream), "D2H");
-        read_dev(c, &timed_out, c->dflag + 3, sizeof(int));
-        if (timed_out) timeout_fail(c);
+        sync_or_timeout(c);   // a device wait of this call or of one before it that did not wait
       }
     }
     return DDLR_OK;
@@ -4152,7 +4163,7 @@ ddlr_status ddlr_set_lowrank(ddlr_handle c, const double *U, const double *lam, 
       v.push_back(theta);
       double *dv = c->w64[7];
       ck(cudaMemcpyAsync(dv, v.data(), sizeof(double) * v.size(), cudaMemcpyHostToDevice, c->stream), "H2D");
-      ck(cudaMemsetAsync(c->dflag, 0, 4 * sizeof(int), c->stream), "memset");
+      clear_flags(c);
       KL(c, "setup", c->stream, k_ddlr1_coef, 1, 32, 0, k + 1, k, 1, dv, c->theta_d, c->inv1mt64,
          c->coef64, c->dflag + 1);
       c->theta = theta;
@@ -4161,7 +4172,7 @@ ddlr_status ddlr_set_lowrank(ddlr_handle c, const double *U, const double *lam, 
       ck(cudaMemcpyAsync(c->Hk64, Hk, sizeof(double) * k * k, cudaMemcpyHostToDevice, c->stream), "H2D");
     }
     lowrank_to_low_precision(c);
-    sync(c);
+    sync_or_timeout(c);
     return DDLR_OK;
   });
 }

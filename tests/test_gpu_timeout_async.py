@@ -59,3 +59,28 @@ def test_later_launches_are_not_affected(kw, monkeypatch):
         assert (h.apply(x.cpu().numpy()) == y0.cpu().numpy()).all()
         assert torch.equal(h.gmres(x, tol=1e-6)[0], z0)
     h.close()
+
+
+@pytest.mark.parametrize("call", ["refactor", "set_lowrank", "batch"])
+def test_pending_timeout_is_reported(call, monkeypatch):
+    """No call that waits clears the flag without reporting it, and the call
+    repeated then leaves the handle as it was."""
+    h, x = _handle(max_nrhs=3)
+    U, lam, theta, _ = h.lowrank()
+    X = torch.stack([x, 2 * x, -x]).T
+
+    def run():
+        if call == "refactor":
+            h.refactor()
+        elif call == "set_lowrank":
+            h.set_lowrank(U, lam, theta)
+        else:
+            return h.apply(X.cpu().numpy())
+
+    run()
+    y0 = h.apply(x).clone()
+    _unmet_apply(h, x, torch.empty_like(x), monkeypatch)
+    _times_out(run)
+    run()
+    assert torch.equal(h.apply(x), y0)
+    h.close()
