@@ -499,8 +499,12 @@ void deep_solve(ddlr_ctx *c, cudaStream_t st, const char *fam, const ddlr_ctx::D
                 const int *gate) {
   ddlr_ctx::Scope sc(c, fam, st);
   DeepLaunch L(D.g, deep_smem_bytes<T>(D.g), st);
+  // tests of the timeout path: DDLR_TEST_DEEP_GIVE_UP=j lets the last part give
+  // up at its stage j
+  const char *gu = getenv("DDLR_TEST_DEEP_GIVE_UP");
   ck(cudaLaunchKernelEx(&L.cfg, k_deep_solve<T>, D.g, (const unsigned char *)D.pl, (const unsigned char *)D.pu, x, z,
-                        gate, c->dflag + 3, std::max(c->wait_ns, kDeepMinWaitNs)), "cudaLaunchKernelEx");
+                        gate, c->dflag + 3, std::max(c->wait_ns, kDeepMinWaitNs), gu ? atoi(gu) : -1),
+     "cudaLaunchKernelEx");
 }
 
 template <typename T>

@@ -192,13 +192,17 @@ __device__ __forceinline__ T deep_chain(T acc, const T *zs, const int *ad, const
 // with L, then backward with L^T.  CTA b takes part b; with g.ctas > 1 the grid
 // is one cluster.  Waits are bounded (limit_ns): a thread whose wait runs out
 // sets *err and the CTA's late flag; the CTA then runs through its stages
-// without waiting or computing (its warps keep to the named barriers), waits,
-// bounded again, for its copies, and meets its peers at the last barrier, so
-// that no CTA leaves while another may still push into its shared memory.
+// without waiting or computing (its warps keep to the named barriers) and starts
+// no more copies, but its pushes are made all the same, whatever they carry:
+// every CTA issues all of its pushes before the last barrier, so that after it a
+// CTA that stopped counting them waits until its mbarriers have the bytes of all.
+// These last waits, and those for the copies in flight, are for transfers that
+// have started; they have a limit of their own (kDeepExitWaitNs).  give_up_at
+// (tests; else -1): the last part's copy warp gives up after this stage.
 template <typename T>
 __global__ void __launch_bounds__(kDeepThreads)
 k_deep_solve(DeepGeo g, const unsigned char *pk_l, const unsigned char *pk_u, const T *x, T *z, const int *gate,
-             int *err, unsigned long long limit_ns) {
+             int *err, unsigned long long limit_ns, int give_up_at) {
   if (gate && *gate) return;               // the same word for every CTA, not written meanwhile
   extern __shared__ __align__(128) unsigned char smraw[];
   constexpr int NT = kDeepThreads, SW = kDeepSetWarps;
@@ -263,27 +267,29 @@ k_deep_solve(DeepGeo g, const unsigned char *pk_l, const unsigned char *pk_u, co
     const uint32_t zb = smem_u32(zs), hb = smem_u32(halo);
     int4 pe = make_int4(0, 0, 0, 0);                       // this lane's first push of the next stage
     if (nst > 0 && st[0].push + ln < st[1].push) pe = g.push[st[0].push + ln];
+    bool late = false;
     for (int j = 0; j < nst; j++) {
       const int p0 = st[j].push + ln, p1 = st[j + 1].push;
       // the sets run ahead of this warp by fewer than kDeepBars levels: it
       // brings in level j + kDeepBars only after level j
       uint64_t *dj = done + (j % kDeepBars);
       const unsigned par = unsigned(j / kDeepBars) & 1u;
-      if (!mbar_try_wait(dj, par)) {
+      if (!late && !mbar_try_wait(dj, par)) {
         const unsigned long long t0 = gtimer_ns();
         while (!mbar_try_wait(dj, par)) {
           if (is_late()) break;
           if (gtimer_ns() - t0 > limit_ns) { give_up(); break; }
         }
       }
-      if (__any_sync(0xffffffffu, is_late())) break;
+      if (j == give_up_at && blockIdx.x == gridDim.x - 1) give_up();
+      late = __any_sync(0xffffffffu, is_late());
       for (int p = p0; p < p1; p += 32) {
         if (p != p0) pe = g.push[p];
         st_async(cluster_map(zb + unsigned(pe.z) * unsigned(sizeof(T)), pe.y), zs[pe.x],
                  cluster_map(hb + unsigned(pe.w) * 8u, pe.y));
       }
       if (j + 1 < nst && p1 + ln < st[j + 2].push) pe = g.push[p1 + ln];
-      if (ln == 0) {
+      if (ln == 0 && !late) {
         // the level is done with its place in the ring: order its reads before
         // the copies into it
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -297,7 +303,7 @@ k_deep_solve(DeepGeo g, const unsigned char *pk_l, const unsigned char *pk_u, co
       const unsigned long long t0 = gtimer_ns();
       for (int q = max(0, jn - kDeepBars); q < jn; q++)
         while (!mbar_try_wait(bar + (q % kDeepBars), unsigned(q / kDeepBars) & 1u))
-          if (gtimer_ns() - t0 > limit_ns) break;
+          if (gtimer_ns() - t0 > kDeepExitWaitNs) break;
     }
     __syncwarp();
   } else {
@@ -331,10 +337,15 @@ k_deep_solve(DeepGeo g, const unsigned char *pk_l, const unsigned char *pk_u, co
       for (int u = 0; u < U; u++)
         if (u < w) ad[u] = entry(u, av[u]);
     };
-    // all of a level that does not depend on other rows' results
+    // all of a level that does not depend on other rows' results.  Once the CTA is
+    // late no warp reads the ring again, also one that had no slice at the stage
+    // that never came: 32 stages on, the parity it would wait for is that of a phase
+    // long over.  (A stage has a warp that waits for it, so every warp sees it late
+    // before then.)
     bool ok = true;
     auto prefetch = [&](int j) {
       const DeepStage s = st[j];
+      ok = ok && !is_late();
       a = s.a + ws;
       b = s.b;
       hl = s.halo;
@@ -344,6 +355,7 @@ k_deep_solve(DeepGeo g, const unsigned char *pk_l, const unsigned char *pk_u, co
       }
     };
     if (set < nst) prefetch(set);
+    __syncwarp();
     for (int j = set; j < nst; j += 2) {
       if (j > 0) set_sync(set ^ 1);                        // level j - 1 is done
       if (hl > 0 && a < b) ok = ok && wait_for(halo + j, 0u, true);
@@ -389,10 +401,11 @@ k_deep_solve(DeepGeo g, const unsigned char *pk_l, const unsigned char *pk_u, co
   if (g.ctas > 1) {
     cluster_sync_all();
     if (is_late()) {
-      // its peers' last pushes into this CTA, which it no longer counts, may be
-      // under way (they take about 1 us)
+      // its peers' last pushes into this CTA
       const unsigned long long t0 = gtimer_ns();
-      while (gtimer_ns() - t0 < 50000ull) {}
+      for (int i = tid; i < nst; i += NT)
+        while (!mbar_try_wait_cluster(halo + i, 0u))
+          if (gtimer_ns() - t0 > kDeepExitWaitNs) break;
     }
   }
 }

@@ -203,9 +203,10 @@ __device__ __forceinline__ unsigned long long gtimer_ns() {
   return t;
 }
 
-// the deep solve waits at least this long for its copies (a CTA must not exit
-// with copies still in flight into its shared memory)
+// the deep solve waits at least this long for a level
 constexpr unsigned long long kDeepMinWaitNs = 1000000000ull;
+// and before it leaves, for transfers in flight into its shared memory
+constexpr unsigned long long kDeepExitWaitNs = 1000000000ull;
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
   return (uint32_t)__cvta_generic_to_shared(p);

@@ -6,6 +6,8 @@ reports the timeout, once.
 The wait is made to run out as in test_gpu_timeout.py: DDLR_TEST_UNMET_BARRIER=1
 lets the first grid barrier of a launch wait for an arrival that nothing provides,
 for 1 ms."""
+import time
+
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -83,4 +85,34 @@ def test_pending_timeout_is_reported(call, monkeypatch):
     _times_out(run)
     run()
     assert torch.equal(h.apply(x), y0)
+    h.close()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("ctas", [1, 2, 8])
+def test_deep_solve_gives_up(ctas, precision, monkeypatch):
+    """A part of a deep solve that gives up after some stage (DDLR_TEST_DEEP_GIVE_UP)
+    leaves when the transfers into its shared memory have arrived, well before
+    the limit of that wait, and so do its peers."""
+    monkeypatch.setenv("DDLR_DEEP_CTAS", str(ctas))
+    shape = (30, 29, 31)
+    A = W.laplacian(shape)
+    part, p = W.box_partition(shape, (2, 2, 3))
+    h = pkg.DDLR(A, part, p, rank_k=4, precision=precision)
+    x = W.rhs(A[0], 1)
+    y0 = h.a0_solve(x)
+    levels = h.info()["levels_c"]
+    for at in (0, 1, 7, levels // 2, levels - 1, levels, levels + 9, 2 * levels - 1):
+        monkeypatch.setenv("DDLR_TEST_DEEP_GIVE_UP", str(at))
+        t = time.perf_counter()
+        if at <= 7:                        # a stage that every part has
+            _times_out(lambda: h.a0_solve(x))
+        else:
+            try:
+                h.a0_solve(x)
+            except pkg.DdlrError as e:
+                assert e.status == "TIMEOUT"
+        assert time.perf_counter() - t < 0.5
+        monkeypatch.delenv("DDLR_TEST_DEEP_GIVE_UP")
+        assert (h.a0_solve(x) == y0).all()
     h.close()
