@@ -4,17 +4,20 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <cstdint>
 #include <cstdlib>
 #include <cstring>
 #include <functional>
+#include <future>
 #include <type_traits>
 #include <map>
 #include <mutex>
 #include <stdexcept>
 #include <string>
+#include <thread>
 #include <vector>
 
 #include "ddlr.h"
@@ -479,12 +482,16 @@ void chunk_sweeps(ddlr_ctx *c, cudaStream_t st, const std::vector<int> &ptr, con
 
 // launch configuration of the deep solve: one cluster of g.ctas CTAs, or (1)
 // one CTA per block
+template <typename T>
+auto deep_fn(const DeepGeo &g) {
+  return g.sw == kDeepSetWarps ? k_deep_solve<T, kDeepSetWarps> : k_deep_solve<T, kDeepWideWarps>;
+}
 struct DeepLaunch {
   cudaLaunchConfig_t cfg{};
   cudaLaunchAttribute at{};
   DeepLaunch(const DeepGeo &g, size_t smem, cudaStream_t st) {
     cfg.gridDim = dim3(g.nparts);
-    cfg.blockDim = dim3(kDeepThreads);
+    cfg.blockDim = dim3(deep_threads(g.sw));
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     at.id = cudaLaunchAttributeClusterDimension;
@@ -502,7 +509,7 @@ void deep_solve(ddlr_ctx *c, cudaStream_t st, const char *fam, const ddlr_ctx::D
   // tests of the timeout path: DDLR_TEST_DEEP_GIVE_UP=j lets the last part give
   // up at its stage j
   const char *gu = getenv("DDLR_TEST_DEEP_GIVE_UP");
-  ck(cudaLaunchKernelEx(&L.cfg, k_deep_solve<T>, D.g, (const unsigned char *)D.pl, (const unsigned char *)D.pu, x, z,
+  ck(cudaLaunchKernelEx(&L.cfg, deep_fn<T>(D.g), D.g, (const unsigned char *)D.pl, (const unsigned char *)D.pu, x, z,
                         gate, c->dflag + 3, std::max(c->wait_ns, kDeepMinWaitNs), gu ? atoi(gu) : -1),
      "cudaLaunchKernelEx");
 }
@@ -1362,10 +1369,12 @@ void panel_plan(ddlr_ctx *c, int which) {
 // interior blocks (a part each), 1 C_a cut into the parts of one cluster.
 // C_a takes the smallest cluster that holds its solution and gives a level of
 // average width at most one pass of a set of warps per CTA (64^3, natural order,
-// 420 rows a level: see k_deep_solve).  Served where every part's solution,
-// tables and a ring of eight of its largest stages (or of all its stages) fit
-// the shared memory of a CTA.
-// DDLR_DEEP=0 switches it off, DDLR_DEEP_CTAS sets the smallest cluster (tests).
+// 420 rows a level: see k_deep_solve), with a ring of eight of its largest stages
+// (or of all its stages); the largest cluster, and an interior block, take what
+// ring the shared memory of a CTA leaves beside the part's solution and tables,
+// down to one stage.
+// DDLR_DEEP=0 switches it off, DDLR_DEEP_CTAS sets the smallest cluster and
+// DDLR_DEEP_STAGES the largest ring in stages (tests).
 template <typename T>
 void deep_plan(ddlr_ctx *c, int which) {
   const Plan &P = c->P;
@@ -1380,115 +1389,100 @@ void deep_plan(ddlr_ctx *c, int which) {
   cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (sms <= 0) return;
-  // blocks beyond one per SM share an SM's memory, up to four of them
+  // blocks beyond one per SM share an SM's memory, up to four of them, also where
+  // that leaves each a ring of one or two stages (a solve, FP64, 512 boxes of 14^3
+  // rows, one to four to an SM: 143, 144, 139 and 103 us; of 16^3: 270, 184, 181,
+  // 173).  Two stages are nearly as good as any number, one costs more: blocks of
+  // 23^3 with one, two, three and eight stages 157, 126, 121 and 121 us (a launch of
+  // k_sptrsv_blocks 185), of 27^3 212, 176, 174 and 174 (252), C_a of 64^3 332, 203,
+  // 227 and 206 (level by level 1,865); all with the narrow sets.
   const int cps = which == 1 ? 1 : std::max(1, std::min(4, (P.p + sms - 1) / sms));
   const long long budget0 = std::min<long long>(optin, per_sm / cps - 1024) - 128;
   const int cmin = which == 0 ? 1 : std::max(force ? atoi(force) : 1, int((long long)P.s / (128LL * NLc)));
-  for (int C = 1; C <= (which == 0 ? 1 : kDeepMaxCtas); C *= 2) {
+  const char *most = getenv("DDLR_DEEP_STAGES");
+  // multicolour orders (deep ones come from fill) scatter a level over the
+  // original order: nearly every row would be exchanged (64^3, IC(2): more
+  // received values than fit), so they are cut no further than one part
+  const int cmax = which == 0 || c->opt.c_order != 0 ? 1 : kDeepMaxCtas;
+  // rows of a level in the order of their parts (the rule for every order): a
+  // part's rows of a level are then found where those of the part before end
+  bool sorted = true;
+  if (which == 1)
+    for (int l = P.blk_lvl0[P.p]; l < P.blk_lvl0[P.p + 1]; l++)
+      for (int r = P.lvl_row0[l] + 1; r < P.lvl_row0[l] + P.lvl_nrows[l]; r++)
+        sorted &= P.iface_rank[r - P.m] > P.iface_rank[r - 1 - P.m];
+  for (int C = 1; C <= cmax; C *= 2) {
     if (which == 1 && C < cmin && C < kDeepMaxCtas) continue;
-    // multicolour orders (deep ones come from fill) scatter a level over the
-    // original order: nearly every row would be exchanged (64^3, IC(2): more
-    // received values than fit), so they are cut no further than one part
-    if (which == 1 && C > 1 && c->opt.c_order != 0) return;
     if (which == 1 && ((long long)P.s / C) * (long long)sizeof(T) > budget0) continue;
     const int np = which == 0 ? P.p : C;
     std::vector<DeepPart> part;
+    std::vector<int> rows_of;                  // rows of a part
     std::vector<DeepStage> stage;
     std::vector<int4> sl, push, fix;
     std::vector<int2> srow;
     std::vector<int> rpos(P.n, 0);
-    std::vector<int> lvl_of_stage, owner;      // owner: part of an interface row
+    std::vector<int> owner;                    // part of an interface row
     std::vector<std::vector<int>> stage_of(np);// stage of (part, level) forward, counted in the part, or -1
     if (which == 1) {
       owner.resize(P.s);
       for (int j = 0; j < P.s; j++) owner[j] = int((long long)P.iface_rank[j] * C / P.s);
     }
+    std::vector<int> next_row;                 // per level of C_a: where the next part's rows start
+    if (which == 1) next_row.assign(P.lvl_row0.begin() + P.blk_lvl0[P.p], P.lvl_row0.begin() + P.blk_lvl0[P.p + 1]);
     long long ol = 0, ou = 0, total_max = 0, stage_max = 0;
-    int zcap = 0, scap = 0, tcap = 0;
+    int scap = 0, tcap = 0;
     bool bad = false;
     for (int q = 0; q < np; q++) {
       DeepPart pt{int(sl.size()), 0, int(stage.size()), 0, 0, 0};
+      int nrow = 0;
       const int b = which == 0 ? q : P.p, l0 = P.blk_lvl0[b], NL = P.blk_lvl0[b + 1] - l0;
       stage_of[q].assign(NL, -1);
       for (int l = 0; l < NL; l++) {
         const int r0 = P.lvl_row0[l0 + l], r1 = r0 + P.lvl_nrows[l0 + l], s0 = int(sl.size());
-        for (int r = r0; r < r1;) {
-          if (which == 1 && owner[r - P.m] != q) { r++; continue; }
+        int r = which == 1 && sorted ? next_row[l] : r0;
+        while (r < r1) {
+          if (which == 1 && owner[r - P.m] != q) {
+            if (sorted) break;
+            r++;
+            continue;
+          }
           int e = r;
           while (e < r1 && e - r < kSlice && (which == 0 || owner[e - P.m] == q)) e++;
           int wl = 0, wu = 0;
           for (int t = r; t < e; t++) {
             wl = std::max(wl, P.l_span[2 * t + 1]);
             wu = std::max(wu, P.u_span[2 * t + 1]);
-            rpos[t] = (int(sl.size()) - pt.slice0) * 32 + (t - r);
+            rpos[t] = nrow + (t - r);
           }
           wl = deep_width(wl);
           wu = deep_width(wu);
-          sl.push_back(make_int4(int(ol / 128), wl, int(ou / 128), wu));
+          if (std::max(wl, wu) > kDeepMaxWidth) return;
+          sl.push_back(make_int4(int(ol / 128), nrow << 6 | (e - r), int(ou / 128), int(unsigned(wl) | unsigned(wu) << 16)));
+          nrow += e - r;
           srow.push_back(make_int2(r, e - r));
           ol += (long long)deep_slice_bytes<T>(wl);
           ou += (long long)deep_slice_bytes<T>(wu);
           r = e;
         }
+        if (which == 1) next_row[l] = r;
         if (int(sl.size()) == s0) continue;
         stage_of[q][l] = int(stage.size()) - pt.stage0;
         DeepStage st{};
         st.a = s0 - pt.slice0;
         st.b = int(sl.size()) - pt.slice0;
         stage.push_back(st);
-        lvl_of_stage.push_back(l);
       }
       pt.nslice = int(sl.size()) - pt.slice0;
       pt.nfwd = int(stage.size()) - pt.stage0;
-      for (int j = pt.nfwd - 1; j >= 0; j--) {
-        stage.push_back(stage[pt.stage0 + j]);
-        lvl_of_stage.push_back(lvl_of_stage[pt.stage0 + j]);
-      }
+      for (int j = pt.nfwd - 1; j >= 0; j--) stage.push_back(stage[pt.stage0 + j]);
       pt.nstage = 2 * pt.nfwd;
       part.push_back(pt);
+      rows_of.push_back(nrow);
       scap = std::max(scap, pt.nslice);
       tcap = std::max(tcap, pt.nstage);
       if (ol / 128 > 0x7fffffffLL || ou / 128 > 0x7fffffffLL) { bad = true; break; }
     }
     if (bad) return;
-    // received values: every row of another part that a part's rows read, once
-    // per sweep, counted for the stage that reads it first
-    std::vector<std::vector<std::vector<int4>>> out(np);
-    if (np > 1 && which == 1) {
-      for (int q = 0; q < np; q++) out[q].resize(part[q].nstage);
-      std::vector<int> seen(P.s), at(P.s);
-      for (int dir = 0; dir < 2; dir++) {
-        std::fill(seen.begin(), seen.end(), -1);
-        for (int q = 0; q < np; q++) {
-          DeepPart &pt = part[q];
-          for (int j = 0; j < pt.nfwd; j++) {
-            const int js = dir ? pt.nfwd + j : j;
-            DeepStage &sg = stage[pt.stage0 + js];
-            for (int i = sg.a; i < sg.b; i++)
-              for (int t = 0; t < srow[pt.slice0 + i].y; t++) {
-                const int r = srow[pt.slice0 + i].x + t;
-                const int *sp = (dir ? P.u_span.data() : P.l_span.data()) + 2 * size_t(r);
-                for (int kk = 0; kk < sp[1]; kk++) {
-                  const int cc = (dir ? P.u_col : P.l_col)[sp[0] + 32 * kk], h = cc - P.m, o = owner[h];
-                  if (o == q) continue;
-                  if (seen[h] != q) {
-                    seen[h] = q;
-                    at[h] = pt.nslice * 32 + pt.nhalo++;
-                    sg.halo++;
-                    // the level of row cc is that of its stage in its part
-                    const int lv = int(std::upper_bound(P.lvl_row0.begin() + P.blk_lvl0[P.p], P.lvl_row0.end(), cc) -
-                                       P.lvl_row0.begin()) - 1 - P.blk_lvl0[P.p];
-                    const int so = stage_of[o][lv];
-                    out[o][dir ? part[o].nstage - 1 - so : so].push_back(make_int4(rpos[cc], q, at[h], js));
-                  }
-                  fix.push_back(make_int4(pt.slice0 + i, dir, kk * 32 + t, at[h]));
-                }
-              }
-          }
-        }
-      }
-    }
-    for (int q = 0; q < np; q++) zcap = std::max(zcap, part[q].nslice * 32 + part[q].nhalo);
     for (int q = 0; q < np; q++) {
       const DeepPart &pt = part[q];
       long long lin = 0;
@@ -1497,24 +1491,103 @@ void deep_plan(ddlr_ctx *c, int which) {
         const int4 ea = sl[pt.slice0 + sg.a], eb = sl[pt.slice0 + sg.b - 1];
         const bool f = j < pt.nfwd;
         sg.src = f ? ea.x : ea.z;
-        sg.bytes = (f ? eb.x : eb.z) - sg.src + int(deep_slice_bytes<T>(f ? eb.y : eb.w) / 128);
-        sg.push = int(push.size());
-        if (!out[q].empty()) push.insert(push.end(), out[q][j].begin(), out[q][j].end());
+        sg.bytes = (f ? eb.x : eb.z) - sg.src + int(deep_slice_bytes<T>(deep_w(eb, f ? 0 : 1)) / 128);
         stage_max = std::max(stage_max, (long long)sg.bytes * 128);
         lin += sg.bytes;
       }
       total_max = std::max(total_max, lin * 128);
     }
+    DeepGeo g{};
+    // wide levels of blocks that have an SM each: twice the warps (kDeepWideRows)
+    const bool wide = which == 0 && P.p <= sms && P.m >= (long long)kDeepWideRows * P.blk_lvl0[P.p];
+    g.sw = wide ? kDeepWideWarps : kDeepSetWarps;
+    g.ctas = C; g.nparts = np; g.scap = scap; g.tcap = tcap;
+    const long long all = total_max + stage_max;
+    const long long least = C == cmax ? stage_max : std::min(all, std::max(8 * stage_max, 16LL << 10));
+    // received values: every row of another part that a part's rows read, once
+    // per sweep, counted for the stage that reads it first; a thread takes parts by
+    // their number until one leaves too little for the ring
+    struct Recv {
+      std::vector<int4> fix, push;             // push: its entry of the push list, by stage of this part
+      std::vector<int2> from;                  // {part, its stage} that pushes it
+    };
+    std::vector<Recv> recv(np);
+    long long ring = budget0;
+    std::mutex mu;
+    std::atomic<int> next(0);
+    auto receive = [&]() {
+      std::vector<int> seen, at;
+      if (C > 1) {
+        seen.assign(P.s, -1);
+        at.resize(P.s);
+      }
+      for (int q; (q = next++) < np;) {
+        DeepPart &pt = part[q];
+        for (int js = 0; C > 1 && js < pt.nstage; js++) {
+          const int dir = js < pt.nfwd ? 0 : 1, sw = 2 * q + dir;
+          const auto &span = dir ? P.u_span : P.l_span;
+          const auto &col = dir ? P.u_col : P.l_col;
+          DeepStage &sg = stage[pt.stage0 + js];
+          for (int i = sg.a; i < sg.b; i++)
+            for (int t = 0; t < srow[pt.slice0 + i].y; t++) {
+              const int r = srow[pt.slice0 + i].x + t;
+              for (int kk = 0; kk < span[2 * size_t(r) + 1]; kk++) {
+                const int cc = col[span[2 * size_t(r)] + 32 * kk], h = cc - P.m, o = owner[h];
+                if (o == q) continue;
+                if (seen[h] != sw) {
+                  seen[h] = sw;
+                  at[h] = rows_of[q] + pt.nhalo++;
+                  sg.halo++;
+                  // the level of row cc is that of its stage in its part
+                  const int lv = int(std::upper_bound(P.lvl_row0.begin() + P.blk_lvl0[P.p], P.lvl_row0.end(), cc) -
+                                     P.lvl_row0.begin()) - 1 - P.blk_lvl0[P.p];
+                  const int so = stage_of[o][lv];
+                  recv[q].push.push_back(make_int4(rpos[cc], q, at[h], js));
+                  recv[q].from.push_back(make_int2(o, dir ? part[o].nstage - 1 - so : so));
+                }
+                recv[q].fix.push_back(make_int4(pt.slice0 + i, dir, kk * 32 + t, at[h]));
+              }
+            }
+        }
+        std::lock_guard<std::mutex> lk(mu);
+        g.zcap = std::max(g.zcap, rows_of[q] + pt.nhalo);
+        ring = (budget0 - (long long)deep_smem_bytes<T>(g)) & ~127LL;
+        if (ring < least) next = np;
+      }
+    };
+    const int threads = C > 1 && P.s >= 20000 ? std::min(C, std::max(1, int(std::thread::hardware_concurrency()))) : 1;
+    if (threads == 1) {
+      receive();
+    } else {
+      std::vector<std::future<void>> run;
+      for (int t = 0; t < threads; t++) run.push_back(std::async(std::launch::async, receive));
+      for (auto &f : run) f.get();
+    }
+    if (ring < least) continue;
+    ring = std::min(ring, std::min(all, std::max(8 * stage_max, 64LL << 10)) & ~127LL);
+    if (most) ring = std::min(ring, std::max(1, atoi(most)) * stage_max);
+    if (ring < least) continue;
+    g.ring_bytes = int(ring);
+    // the push lists, in the order of the pushing stages
+    for (DeepStage &sg : stage) sg.push = 0;
+    for (const Recv &R : recv) {
+      fix.insert(fix.end(), R.fix.begin(), R.fix.end());
+      for (const int2 &f : R.from) stage[part[f.x].stage0 + f.y].push++;
+    }
+    int npush = 0;
+    for (DeepStage &sg : stage) {
+      const int cnt = sg.push;
+      sg.push = npush;
+      npush += cnt;
+    }
+    push.resize(npush);
+    std::vector<int> put(stage.size());
+    for (size_t i = 0; i < stage.size(); i++) put[i] = stage[i].push;
+    for (const Recv &R : recv)
+      for (size_t i = 0; i < R.from.size(); i++) push[put[part[R.from[i].x].stage0 + R.from[i].y]++] = R.push[i];
     DeepStage end{};
     end.push = int(push.size());
     stage.push_back(end);
-    DeepGeo g{};
-    g.ctas = C; g.nparts = np; g.zcap = zcap; g.scap = scap; g.tcap = tcap;
-    const long long budget = budget0 - (long long)deep_smem_bytes<T>(g);
-    const long long want = std::min(total_max + stage_max, std::max(8 * stage_max, 16LL << 10));
-    const long long ring = std::min(std::min(budget, total_max + stage_max), 64LL << 10) & ~127LL;
-    if (std::min(budget, std::max(want, ring)) < want) continue;
-    g.ring_bytes = int(std::max(ring, (want + 127) & ~127LL));
     // places in the ring: one stage after the other, from the start again
     // where one does not fit before the end
     for (const DeepPart &pt : part) {
@@ -1531,12 +1604,12 @@ void deep_plan(ddlr_ctx *c, int which) {
     }
     const size_t smem = deep_smem_bytes<T>(g);
     if ((long long)smem > budget0) continue;
-    raise_smem_limit((const void *)k_deep_solve<T>, smem);
-    if (C > 8) ck(cudaFuncSetAttribute(k_deep_solve<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1), "attr");
+    raise_smem_limit((const void *)deep_fn<T>(g), smem);
+    if (C > 8) ck(cudaFuncSetAttribute(deep_fn<T>(g), cudaFuncAttributeNonPortableClusterSizeAllowed, 1), "attr");
     if (C > 1) {
       int fit = 0;
       DeepLaunch L(g, smem, nullptr);
-      if (cudaOccupancyMaxActiveClusters(&fit, k_deep_solve<T>, &L.cfg) != cudaSuccess || fit < 1) {
+      if (cudaOccupancyMaxActiveClusters(&fit, deep_fn<T>(g), &L.cfg) != cudaSuccess || fit < 1) {
         cudaGetLastError();
         continue;
       }

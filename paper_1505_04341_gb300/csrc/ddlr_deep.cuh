@@ -26,8 +26,14 @@
 
 namespace ddlr {
 
-constexpr int kDeepSetWarps = 4;                              // warps of one set
-constexpr int kDeepThreads = (2 * kDeepSetWarps + 1) * 32;    // two sets and the copy / push warp
+// Warps of one set, and of one for wide levels: blocks that have an SM each and
+// kDeepWideRows rows a level on average.  Below that line the two are alike (a solve,
+// FP64, edges of 11 and 13: 41.6 and 42.2 us, 47.6 and 46.2), above it a level takes a
+// warp several slices (15: 60.4 and 52.5, 23: 121 and 96, 28: 219 and 177; FP32, 35:
+// 285 and 219).  Two blocks to an SM fill it with the narrow sets (FP32, 112 x 112 x
+// 96 in 294 boxes: 82 and 100).
+constexpr int kDeepSetWarps = 4, kDeepWideWarps = 8, kDeepWideRows = 80;
+__host__ __device__ constexpr int deep_threads(int sw) { return (2 * sw + 1) * 32; }   // two sets and the copy / push warp
 constexpr int kDeepMaxCtas = 16;
 constexpr int kDeepBars = 32;            // ring mbarriers: stages in flight at most
 
@@ -50,26 +56,31 @@ static_assert(sizeof(DeepStage) == 32 && sizeof(DeepPart) == 24, "tables are cop
 
 // Geometry of one launch: ctas = CTAs of a cluster (1: independent blocks)
 struct DeepGeo {
-  int ctas, nparts;
+  int ctas, nparts, sw;    // sw: warps of a set
   int ring_bytes;          // staging ring (multiple of 128)
-  int zcap, scap, tcap;    // most slices * 32 + received values, slices, stages of a part
+  int zcap, scap, tcap;    // most rows + received values, slices, stages of a part
   const DeepPart *part;
   const DeepStage *stage;
   const int4 *push;        // {position here, part's rank, position there, stage there}
-  const int4 *sl;          // per slice: {L offset / 128, L width, U offset / 128, U width}
+  const int4 *sl;          // per slice: {L offset / 128, position << 6 | rows, U offset / 128, L width | U width << 16}
   const int2 *srow;        // per slice: {first row, rows}
 };
 
 // stored width of a slice: beyond four entries a multiple of four, so that the
 // row's chain is straight code (a test per entry costs as much as its FMA)
+constexpr int kDeepMaxWidth = 0xffff;
 inline int deep_width(int w) { return w <= 4 ? w : (w + 3) & ~3; }
+// width of slice entry e for direction dir (1: L^T)
+__host__ __device__ inline int deep_w(const int4 &e, int dir) {
+  return dir ? int(unsigned(e.w) >> 16) : int(unsigned(e.w) & 0xffffu);
+}
 template <typename T>
 __host__ __device__ inline size_t deep_slice_bytes(int w) {
   return size_t(w) * 32 * (sizeof(T) + 4) + 32 * sizeof(T);
 }
 template <typename T>
 __host__ __device__ inline size_t deep_smem_bytes(const DeepGeo &g) {
-  return 16 * kDeepBars + size_t(g.ring_bytes) + al128(size_t(g.zcap) * sizeof(T)) +
+  return 16 * kDeepBars + size_t(g.ring_bytes) + al128(size_t(g.zcap + 1) * sizeof(T)) +
          al128(size_t(g.tcap + 1) * sizeof(DeepStage)) + al128(size_t(g.scap) * 16) +
          (g.ctas > 1 ? size_t(g.tcap) * 8 : 0);
 }
@@ -83,7 +94,7 @@ __global__ void k_deep_cols(DeepGeo g, const int2 *l_span, const int2 *u_span, c
   const int4 e = g.sl[blockIdx.x];
   const int2 sr = g.srow[blockIdx.x];
   for (int dir = 0; dir < 2; dir++) {
-    const int w = dir ? e.w : e.y;
+    const int w = deep_w(e, dir);
     unsigned char *p = dir ? pk_u + size_t(e.z) * 128 : pk_l + size_t(e.x) * 128;
     int *pc = reinterpret_cast<int *>(p + size_t(w) * 32 * sizeof(T));
     for (int i = threadIdx.x; i < w * 32; i += blockDim.x) {
@@ -100,7 +111,7 @@ __global__ void k_deep_fix(int cnt, DeepGeo g, const int4 *fix, unsigned char *p
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= cnt) return;
   const int4 f = fix[i], e = g.sl[f.x];
-  const int w = f.y ? e.w : e.y;
+  const int w = deep_w(e, f.y);
   unsigned char *p = f.y ? pk_u + size_t(e.z) * 128 : pk_l + size_t(e.x) * 128;
   reinterpret_cast<int *>(p + size_t(w) * 32 * sizeof(T))[f.z] = f.w;
 }
@@ -112,7 +123,7 @@ __global__ void k_deep_pack(DeepGeo g, const int2 *l_span, const int2 *u_span, c
   const int4 e = g.sl[blockIdx.x];
   const int2 sr = g.srow[blockIdx.x];
   for (int dir = 0; dir < 2; dir++) {
-    const int w = dir ? e.w : e.y;
+    const int w = deep_w(e, dir);
     unsigned char *p = dir ? pk_u + size_t(e.z) * 128 : pk_l + size_t(e.x) * 128;
     T *pv = reinterpret_cast<T *>(p);
     T *pd = reinterpret_cast<T *>(p + size_t(w) * 32 * (sizeof(T) + 4));
@@ -169,12 +180,14 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t *bar, unsigned pa
       : "memory");
   return ok != 0;
 }
-// named barriers 1 and 2: end of a level of set 0 and of set 1
+// named barriers 1 and 2: end of a level of set 0 and of set 1 (of SW warps each)
+template <int SW>
 __device__ __forceinline__ void set_arrive(int set) {
-  asm volatile("bar.arrive %0, %1;" ::"r"(1 + set), "n"(2 * kDeepSetWarps * 32) : "memory");
+  asm volatile("bar.arrive %0, %1;" ::"r"(1 + set), "n"(2 * SW * 32) : "memory");
 }
+template <int SW>
 __device__ __forceinline__ void set_sync(int set) {
-  asm volatile("bar.sync %0, %1;" ::"r"(1 + set), "n"(2 * kDeepSetWarps * 32) : "memory");
+  asm volatile("bar.sync %0, %1;" ::"r"(1 + set), "n"(2 * SW * 32) : "memory");
 }
 
 // acc - sum of the first W prefetched entries, the loads before the FMAs
@@ -199,13 +212,14 @@ __device__ __forceinline__ T deep_chain(T acc, const T *zs, const int *ad, const
 // These last waits, and those for the copies in flight, are for transfers that
 // have started; they have a limit of their own (kDeepExitWaitNs).  give_up_at
 // (tests; else -1): the last part's copy warp gives up after this stage.
-template <typename T>
-__global__ void __launch_bounds__(kDeepThreads)
+// Four narrow CTAs share an SM: that many fit its registers.
+template <typename T, int SW>
+__global__ void __launch_bounds__(deep_threads(SW), SW == kDeepSetWarps ? 4 : 2)
 k_deep_solve(DeepGeo g, const unsigned char *pk_l, const unsigned char *pk_u, const T *x, T *z, const int *gate,
              int *err, unsigned long long limit_ns, int give_up_at) {
   if (gate && *gate) return;               // the same word for every CTA, not written meanwhile
   extern __shared__ __align__(128) unsigned char smraw[];
-  constexpr int NT = kDeepThreads, SW = kDeepSetWarps;
+  constexpr int NT = deep_threads(SW);
   const int tid = threadIdx.x, wi = tid >> 5, ln = tid & 31;
   const DeepPart P = g.part[blockIdx.x];
   const int nst = P.nstage;
@@ -213,7 +227,7 @@ k_deep_solve(DeepGeo g, const unsigned char *pk_l, const unsigned char *pk_u, co
   uint64_t *done = bar + kDeepBars;                        // levels finished by their set
   unsigned char *ring = smraw + 16 * kDeepBars;
   T *zs = reinterpret_cast<T *>(ring + g.ring_bytes);
-  DeepStage *st = reinterpret_cast<DeepStage *>(reinterpret_cast<unsigned char *>(zs) + al128(size_t(g.zcap) * sizeof(T)));
+  DeepStage *st = reinterpret_cast<DeepStage *>(reinterpret_cast<unsigned char *>(zs) + al128(size_t(g.zcap + 1) * sizeof(T)));
   int4 *sl = reinterpret_cast<int4 *>(reinterpret_cast<unsigned char *>(st) + al128(size_t(g.tcap + 1) * sizeof(DeepStage)));
   uint64_t *halo = reinterpret_cast<uint64_t *>(reinterpret_cast<unsigned char *>(sl) + al128(size_t(g.scap) * 16));
   __shared__ int s_late;
@@ -238,7 +252,8 @@ k_deep_solve(DeepGeo g, const unsigned char *pk_l, const unsigned char *pk_u, co
 #pragma unroll 4
   for (int i = wi; i < P.nslice; i += NT / 32) {           // the right-hand side
     const int2 sr = srow[i];
-    zs[i * 32 + ln] = ln < sr.y ? x[sr.x + ln] : T(0);
+    const int p = g.sl[P.slice0 + i].y >> 6;
+    if (ln < sr.y) zs[p + ln] = x[sr.x + ln];
   }
   __syncthreads();
   if (g.ctas > 1) {
@@ -310,7 +325,7 @@ k_deep_solve(DeepGeo g, const unsigned char *pk_l, const unsigned char *pk_u, co
     // ---- set wi / SW: levels of its parity; this warp's slices a + ws, a + ws + SW, ...
     const int set = wi / SW, ws = wi % SW;
     constexpr int U = 4;
-    int a = 0, b = 0, w = 0, hl = 0;
+    int a = 0, b = 0, w = 0, hl = 0, zi = 0;               // zi: this lane's row (a spare place past the slice's last)
     T acc = T(0), dr = T(0), av[U];
     int ad[U];
     const unsigned char *pe = nullptr;
@@ -329,10 +344,11 @@ k_deep_solve(DeepGeo g, const unsigned char *pk_l, const unsigned char *pk_u, co
     };
     auto open_slice = [&](const DeepStage &s, bool fwd, int i) {
       const int4 e = sl[i];
-      w = fwd ? e.y : e.w;
+      w = deep_w(e, fwd ? 0 : 1);
+      zi = ln < (e.y & 63) ? (e.y >> 6) + ln : g.zcap;
       pe = ring + size_t(s.pos + (fwd ? e.x : e.z) - s.src) * 128;
       dr = reinterpret_cast<const T *>(pe + size_t(w) * 32 * (sizeof(T) + 4))[ln];
-      acc = zs[i * 32 + ln];
+      acc = zs[zi];
 #pragma unroll
       for (int u = 0; u < U; u++)
         if (u < w) ad[u] = entry(u, av[u]);
@@ -357,11 +373,11 @@ k_deep_solve(DeepGeo g, const unsigned char *pk_l, const unsigned char *pk_u, co
     if (set < nst) prefetch(set);
     __syncwarp();
     for (int j = set; j < nst; j += 2) {
-      if (j > 0) set_sync(set ^ 1);                        // level j - 1 is done
+      if (j > 0) set_sync<SW>(set ^ 1);                        // level j - 1 is done
       if (hl > 0 && a < b) ok = ok && wait_for(halo + j, 0u, true);
       // the turn: the top level's forward results were not there to prefetch
       // (every other backward level is at least three levels after its forward)
-      if (j == P.nfwd && a < b) acc = zs[a * 32 + ln];
+      if (j == P.nfwd && a < b) acc = zs[zi];
       for (int i = a; ok && i < b; i += SW) {
         if (i != a) open_slice(st[j], j < P.nfwd, i);
         switch (min(w, U + 1)) {
@@ -382,10 +398,10 @@ k_deep_solve(DeepGeo g, const unsigned char *pk_l, const unsigned char *pk_u, co
               for (int u = 0; u < U; u++) acc -= av[u] * zv[u];
             }
         }
-        zs[i * 32 + ln] = acc * dr;
+        zs[zi] = acc * dr;
       }
       __syncwarp();
-      if (j + 1 < nst) set_arrive(set);
+      if (j + 1 < nst) set_arrive<SW>(set);
       if (ln == 0) mbar_arrive(done + (j % kDeepBars));
       if (j + 2 < nst) prefetch(j + 2);
       __syncwarp();
@@ -395,7 +411,7 @@ k_deep_solve(DeepGeo g, const unsigned char *pk_l, const unsigned char *pk_u, co
 #pragma unroll 4
   for (int i = wi; i < P.nslice; i += NT / 32) {           // the result
     const int2 sr = srow[i];
-    if (ln < sr.y) z[sr.x + ln] = zs[i * 32 + ln];
+    if (ln < sr.y) z[sr.x + ln] = zs[(sl[i].y >> 6) + ln];
   }
   __syncwarp();
   if (g.ctas > 1) {
