@@ -1394,8 +1394,8 @@ void deep_plan(ddlr_ctx *c, int which) {
   // rows, one to four to an SM: 143, 144, 139 and 103 us; of 16^3: 270, 184, 181,
   // 173).  Two stages are nearly as good as any number, one costs more: blocks of
   // 23^3 with one, two, three and eight stages 157, 126, 121 and 121 us (a launch of
-  // k_sptrsv_blocks 185), of 27^3 212, 176, 174 and 174 (252), C_a of 64^3 332, 203,
-  // 227 and 206 (level by level 1,865); all with the narrow sets.
+  // k_sptrsv_blocks 185), of 27^3 212, 176, 174 and 174 (252), C_a of 64^3 414, 216,
+  // 205 and 205 (level by level 1,865); all with the narrow sets.
   const int cps = which == 1 ? 1 : std::max(1, std::min(4, (P.p + sms - 1) / sms));
   const long long budget0 = std::min<long long>(optin, per_sm / cps - 1024) - 128;
   const int cmin = which == 0 ? 1 : std::max(force ? atoi(force) : 1, int((long long)P.s / (128LL * NLc)));
@@ -1503,7 +1503,10 @@ void deep_plan(ddlr_ctx *c, int which) {
     g.sw = wide ? kDeepWideWarps : kDeepSetWarps;
     g.ctas = C; g.nparts = np; g.scap = scap; g.tcap = tcap;
     const long long all = total_max + stage_max;
-    const long long least = C == cmax ? stage_max : std::min(all, std::max(8 * stage_max, 16LL << 10));
+    long long want = std::min(all, std::max(8 * stage_max, 64LL << 10)) & ~127LL;
+    if (most) want = std::min(want, std::max(1, atoi(most)) * stage_max);
+    const long long least =
+        C == cmax ? stage_max : std::min(want, std::min(all, std::max(8 * stage_max, 16LL << 10)));
     // received values: every row of another part that a part's rows read, once
     // per sweep, counted for the stage that reads it first; a thread takes parts by
     // their number until one leaves too little for the ring
@@ -1564,10 +1567,7 @@ void deep_plan(ddlr_ctx *c, int which) {
       for (auto &f : run) f.get();
     }
     if (ring < least) continue;
-    ring = std::min(ring, std::min(all, std::max(8 * stage_max, 64LL << 10)) & ~127LL);
-    if (most) ring = std::min(ring, std::max(1, atoi(most)) * stage_max);
-    if (ring < least) continue;
-    g.ring_bytes = int(ring);
+    g.ring_bytes = int(std::min(ring, want));
     // the push lists, in the order of the pushing stages
     for (DeepStage &sg : stage) sg.push = 0;
     for (const Recv &R : recv) {
