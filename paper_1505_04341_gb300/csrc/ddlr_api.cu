@@ -2366,9 +2366,28 @@ bool apply_persist_t(ddlr_ctx *c, const double *x, double *y, T *u, T *z, T *v, 
   return pz_launch_own(c, "apply_persist", (const void *)k_apply_persist<kPzThreads, T, TU>, pz_small_grid(c),
                        pz_pcg_smem(c->opt.rank_k), args);
 }
-// y = M^-1 x in the caller's order as one launch; false: not served
+// DDLR-2 streams U_k (n x k) twice per apply.  The per-phase kernels do so with
+// 16-byte loads from four times the resident threads where k fits those (uvec_lanes),
+// the persistent kernels an element at a time (U_k^T x) and a row per thread, so
+// beyond a number of elements they lose more than the launches cost.
+bool ddlr2_streams_u(ddlr_ctx *c, double elements) {
+  const int k = c->opt.rank_k;
+  const int lanes = c->opt.precision == 0 ? uvec_lanes<double>(c, k)
+                    : c->opt.uk_bf16      ? uvec_lanes<__nv_bfloat16>(c, k)
+                                          : uvec_lanes<float>(c, k);
+  return c->opt.variant == 2 && lanes > 0 && double(c->P.n) * k >= elements;
+}
+
+// y = M^-1 x in the caller's order as one launch; false: not served.  DDLR-2, per
+// phase and in one launch: BF16 U_k, 64^3 with k = 16, 32 and 128 38 and 35, 46 and
+// 52, 87 and 161 us, 76^3 with k = 16 42 and 50; FP32 U_k, 52^3 with k = 32 and 64 43
+// and 38, 54 and 60, 40^3 with k = 128 71 and 62; FP64, 64^3 with k = 32 80 and 70,
+// 76^3 with k = 32 110 and 117, with k = 64 (no direct kernels) 277 and 196.
 bool apply_persist(ddlr_ctx *c, const double *x, double *y) {
   if (!c->pz_pcg) return false;
+  if (c->opt.precision == 0 ? c->opt.rank_k <= 32 && ddlr2_streams_u(c, 12e6)
+                            : c->P.n >= 100000 && ddlr2_streams_u(c, 6e6))
+    return false;
   double *const *D = c->w64;
   float *const *F = c->w32;
   if (c->opt.precision == 0) return apply_persist_t<double, double>(c, x, y, c->pv[7], D[0], D[1], D[2], D[3]);
@@ -2751,8 +2770,12 @@ void gmres_dev(ddlr_ctx *c, const double *b, double *x, double tol, int maxit, i
     G.st = c->alloc<double>(4);
     G.m = m;
   }
-  // shallow factors on small problems: the whole solve in one launch
-  if (c->pz_pcg && m <= kPzGmMaxRestart &&
+  // shallow factors on small problems: the whole solve in one launch.  DDLR-2 in
+  // mixed precision: what a launch per step loses outside the applies grows with m
+  // (per step and in one launch, BF16 U_k, 64^3 with k = 64, m = 10, 40 and 128: 1.27
+  // and 1.33, 6.5 and 6.4, 40.9 and 32.4 ms; 76^3 with k = 64: 1.63 and 2.07, 9.2 and
+  // 10.0, 58 and 51).
+  if (c->pz_pcg && m <= kPzGmMaxRestart && !(c->opt.precision == 1 && ddlr2_streams_u(c, 14e6 + 0.24e6 * m)) &&
       (long long)(maxit + 2) * (2 * pz_barriers_per_iteration(c)) * c->pz_grid < (1LL << 31)) {
     const int stride = std::max(c->opt.rank_k, m + 2);
     if (G.pz_stride < stride) {
