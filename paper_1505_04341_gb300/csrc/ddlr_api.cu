@@ -3287,8 +3287,8 @@ struct FbShape {
 };
 template <MrStep S>
 void mr_reduce(ddlr_ctx *c, int rows, int no, const int *gate) {
-  KL(c, "pcg_mr_red", c->stream, k_reduce_step_mr<S>, kRedGrid, kMrRedNT, 0, rows, no, c->bt.fpart, c->bt.part64,
-     c->bt.st, c->bt.count, gate);
+  KL(c, "pcg_mr_red", c->stream, k_reduce_step_mr<S>, mr_narrow(rows, no) ? kMrRedGroups : kRedGrid, kMrRedNT, 0,
+     rows, no, c->bt.fpart, c->bt.part64, c->bt.st, c->bt.count, gate);
 }
 inline void mr_apply_prec(ddlr_ctx *c, const double *in, double *z, int R, const int *gate) {
   apply_mr<double, double>(c, c->U64, in, z, R, gate);

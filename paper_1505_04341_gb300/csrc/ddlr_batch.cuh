@@ -1110,7 +1110,15 @@ __device__ __forceinline__ void mr_step(PcgStateMR *st, const double *sm) {
 // so that one load latency precedes the serial adds instead of one per few.
 // count: 1 + kMrRedGroups counters, 0 between launches; partials: the ranges' rows,
 // then those of the groups.
-constexpr int kMrRedNT = 256, kMrStage = 2048, kMrRedGroups = 32;
+// Narrow blocks with few rows (mr_narrow) take one CTA per group instead, a thread
+// per range and column: a step less on the way, and 32 CTAs to launch (a solve, FP32,
+// with 304 and 32: 16^3 x 5 3.92 and 3.48 ms, 24^3 x 13 6.06 and 5.60, 64^3 x 7 24.8
+// and 23.9).  A thread takes its rows one after the other there, eight loads at a time:
+// the line lies at 16 rows, two such trips (a range has 108 at 128^3).
+constexpr int kMrRedNT = 256, kMrStage = 2048, kMrRedGroups = 32, kMrNarrowRows = 16 * kRedGrid;
+inline bool mr_narrow(int nrows, int no) {
+  return ((kRedGrid + kMrRedGroups - 1) / kMrRedGroups) * no <= kMrRedNT && nrows <= kMrNarrowRows;
+}
 template <MrStep S>
 __global__ void __launch_bounds__(kMrRedNT)
 k_reduce_step_mr(int nrows, int no, const double *bpart, double *partials, PcgStateMR *st, unsigned *count,
@@ -1119,36 +1127,61 @@ k_reduce_step_mr(int nrows, int no, const double *bpart, double *partials, PcgSt
   if (S == kMrDec && !st->any_check) return;
   __shared__ double stage[kMrStage], sm[2 * kMaxR];
   __shared__ bool last;
-  long long b0, b1;
-  red_range(nrows, blockIdx.x, gridDim.x, b0, b1);
-  const int R = st->R, per = kMrStage / no;           // rows staged at once
-  double v = 0.0;
-  for (long long b = b0; b < b1; b += per) {
-    const int cnt = (int)min((long long)per, b1 - b);
-    for (int i = threadIdx.x; i < cnt * no; i += kMrRedNT) stage[i] = bpart[b * no + i];
-    __syncthreads();
-    if (threadIdx.x < no)
-      for (int i = 0; i < cnt; i++) v += stage[i * no + threadIdx.x];
-    __syncthreads();
-  }
-  if (threadIdx.x < no) partials[(long long)blockIdx.x * 2 * R + threadIdx.x] = v;
-  __threadfence();
-  __syncthreads();
   static_assert(kRedGrid >= kMrRedGroups, "no empty group");
-  const int G = gridDim.x, grp = blockIdx.x % kMrRedGroups;
-  if (threadIdx.x == 0) {
-    last = atomicAdd(count + 1 + grp, 1u) == unsigned((G - grp + kMrRedGroups - 1) / kMrRedGroups) - 1u;
-    if (last) count[1 + grp] = 0u;
-  }
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
+  constexpr int G = kRedGrid;
+  const int R = st->R, grp = blockIdx.x % kMrRedGroups, ng = (G - grp + kMrRedGroups - 1) / kMrRedGroups;
   double *gsum = partials + (long long)G * 2 * R;
-  if (threadIdx.x < no) {
-    v = 0.0;
+  long long b0, b1;
+  double v = 0.0;
+  if (gridDim.x == kMrRedGroups) {                    // mr_narrow: this CTA's ranges at once
+    const int g = threadIdx.x / no, o = threadIdx.x % no;
+    if (g < ng) {
+      red_range(nrows, grp + g * kMrRedGroups, G, b0, b1);
+      constexpr int U = 8;
+      for (long long b = b0; b < b1; b += U) {
+        double t[U];
+#pragma unroll
+        for (int u = 0; u < U; u++)
+          if (b + u < b1) t[u] = bpart[(b + u) * no + o];
+#pragma unroll
+        for (int u = 0; u < U; u++)
+          if (b + u < b1) v += t[u];
+      }
+      stage[threadIdx.x] = v;
+    }
+    __syncthreads();
+    if (threadIdx.x < no) {
+      v = 0.0;
+      for (int q = 0; q < ng; q++) v += stage[q * no + threadIdx.x];
+      gsum[(long long)grp * 2 * R + threadIdx.x] = v;
+    }
+  } else {
+    red_range(nrows, blockIdx.x, G, b0, b1);
+    const int per = kMrStage / no;                    // rows staged at once
+    for (long long b = b0; b < b1; b += per) {
+      const int cnt = (int)min((long long)per, b1 - b);
+      for (int i = threadIdx.x; i < cnt * no; i += kMrRedNT) stage[i] = bpart[b * no + i];
+      __syncthreads();
+      if (threadIdx.x < no)
+        for (int i = 0; i < cnt; i++) v += stage[i * no + threadIdx.x];
+      __syncthreads();
+    }
+    if (threadIdx.x < no) partials[(long long)blockIdx.x * 2 * R + threadIdx.x] = v;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      last = atomicAdd(count + 1 + grp, 1u) == unsigned(ng) - 1u;
+      if (last) count[1 + grp] = 0u;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    if (threadIdx.x < no) {
+      v = 0.0;
 #pragma unroll 10
-    for (int g = grp; g < G; g += kMrRedGroups) v += __ldcg(partials + (long long)g * 2 * R + threadIdx.x);
-    gsum[(long long)grp * 2 * R + threadIdx.x] = v;
+      for (int g = grp; g < G; g += kMrRedGroups) v += __ldcg(partials + (long long)g * 2 * R + threadIdx.x);
+      gsum[(long long)grp * 2 * R + threadIdx.x] = v;
+    }
   }
   __threadfence();
   __syncthreads();
