@@ -4380,7 +4380,10 @@ ddlr_status ddlr_get_traffic(ddlr_handle c, double *apply_bytes, double *a0_byte
     // launches per A0 sweep pair: two for two-level factors (modes 3 and 4),
     // else forward, top and backward levels
     auto sweeps = [](int L) { return L == 2 ? 2 : std::max(1, 2 * L - 1); };
-    const double clev = sweeps(P.levels_c);
+    // (one where k_panel_solve or k_deep_solve takes the block)
+    const bool one = c->opt.precision == 1 ? c->pan32[1].g.nblk > 0 || c->deep32[1].g.ctas > 0
+                                           : c->pan64[1].g.nblk > 0 || c->deep64[1].g.ctas > 0;
+    const double clev = one ? 1 : sweeps(P.levels_c);
     const double nnz_a = double(P.nnz);
     const double R = std::max(1, c->bt.last_R);
     for (int i = 0; i < cap_f && i < int(c->fam_names.size()); i++) {
