@@ -408,7 +408,7 @@ void raise_smem_limit(const void *fn, size_t bytes) {
 
 template <typename T>
 size_t sf_smem_bytes(const Plan &P) {
-  return ((size_t(P.tma_zs) * sizeof(T) + 15) & ~size_t(15)) + size_t(P.tma_zs) * 4;
+  return ((size_t(P.blk_rows_max) * sizeof(T) + 15) & ~size_t(15)) + size_t(P.blk_rows_max) * 4;
 }
 
 template <typename T> struct Prec;
@@ -2487,10 +2487,10 @@ void allocate(ddlr_ctx *c) {
   if (!P.lv_desc.empty()) c->lv_desc = reinterpret_cast<int4 *>(c->upload(P.lv_desc));
   {
     // interior-solve kernel for deep factors: the level pipeline of
-    // ddlr_deep.cuh (default), synchronisation-free, or plain level schedule
-    // (DDLR_SOLVE=tma|sf|plain)
+    // ddlr_deep.cuh (default), synchronisation-free (DDLR_SOLVE=sf), or plain level
+    // schedule (DDLR_SOLVE=plain)
     const char *env = getenv("DDLR_SOLVE");
-    const std::string kind = env ? env : "tma";
+    const std::string kind = env ? env : "";
     const char *uv = getenv("DDLR_UVEC");
     c->uvec = !(uv && uv[0] == '0');
     const char *cr = getenv("DDLR_CHUNK_ROWS");
@@ -2498,7 +2498,7 @@ void allocate(ddlr_ctx *c) {
     int dev = 0, optin = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    const bool sf_ok = P.tma_zs > 0 && kind == "sf";
+    const bool sf_ok = P.blk_rows_max > 0 && kind == "sf";
     c->use_sf64 = sf_ok && sf_smem_bytes<double>(P) <= size_t(optin);
     c->use_sf32 = sf_ok && sf_smem_bytes<float>(P) <= size_t(optin);
     c->deep_int = kind != "plain" && !c->use_sf64 && !c->use_sf32;
@@ -2543,9 +2543,9 @@ void allocate(ddlr_ctx *c) {
   deep_plan<double>(c, 1);
   if (c->opt.precision == 1) {
     panel_plan<float>(c, 0);
-  deep_plan<float>(c, 0);
+    deep_plan<float>(c, 0);
     panel_plan<float>(c, 1);
-  deep_plan<float>(c, 1);
+    deep_plan<float>(c, 1);
     c->l32 = c->alloc<float>(P.l_col.size());
     c->u32 = c->alloc<float>(P.u_col.size());
     c->dinv32 = c->alloc<float>(n);
@@ -3339,8 +3339,8 @@ void pcg_mr_iteration_t(ddlr_ctx *c, int R, int flexible) {
   mr_reduce<kMrRr>(c, int(F.nb), R, gate);
   // the check kernels run on a small grid: most iterations they return at once
   // (1,216 CTAs took 17 us to do so, 304 take 3)
-  const unsigned gchk = (unsigned)std::min<long long>(eblk(nR, 256), 2 * 152);
-  KL(c, "pcg_mr_check", c->stream, k_pcgmr_true_res, std::min(F.grid, 2 * 152u), F.threads, 0, n, B.st, c->a_soff,
+  const unsigned gchk = (unsigned)std::min<long long>(eblk(nR, 256), kRedGrid);
+  KL(c, "pcg_mr_check", c->stream, k_pcgmr_true_res, std::min(F.grid, unsigned(kRedGrid)), F.threads, 0, n, B.st, c->a_soff,
      c->a_sw, c->a_col, c->a_val, B.B, B.X, B.T, B.fpart);
   mr_reduce<kMrDec>(c, int(F.nb), R, gate);
   KL(c, "pcg_mr_check", c->stream, k_pcgmr_copy_r<T>, gchk, 256, 0, (long long)n, B.st, B.T, B.Rr, c->dsc_dev,

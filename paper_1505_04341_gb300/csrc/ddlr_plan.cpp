@@ -819,23 +819,7 @@ ddlr_status build_plan(int n, const int *rp, const int *ci, const double *val,
       });
     }
   }
-  for (int b = 0; b < p; b++) {
-    const int l0 = P.blk_lvl0[b], l1 = P.blk_lvl0[b + 1];
-    if (l1 == l0) continue;
-    P.tma_zs = std::max(P.tma_zs, P.blk_row0[b + 1] - P.blk_row0[b]);
-    P.tma_nl = std::max(P.tma_nl, l1 - l0);
-    P.tma_ns = std::max(P.tma_ns, P.lvl_slice0[l1] - P.lvl_slice0[l0] + 1);
-    long long be = 0, bs = 0;
-    for (int l = l0; l < l1; l++) {
-      const int s0 = P.lvl_slice0[l], s1 = P.lvl_slice0[l + 1];
-      P.tma_e = std::max(P.tma_e, std::max(P.l_soff[s1] - P.l_soff[s0], P.u_soff[s1] - P.u_soff[s0]));
-      P.tma_s = std::max(P.tma_s, s1 - s0);
-      be += (P.l_soff[s1] - P.l_soff[s0]) + (P.u_soff[s1] - P.u_soff[s0]);
-      bs += 2 * (s1 - s0);
-    }
-    P.tma_blk_e = std::max(P.tma_blk_e, be);
-    P.tma_blk_s = std::max(P.tma_blk_s, bs);
-  }
+  for (int b = 0; b < p; b++) P.blk_rows_max = std::max(P.blk_rows_max, P.blk_row0[b + 1] - P.blk_row0[b]);
   return DDLR_OK;
 }
 

@@ -82,9 +82,7 @@ struct Plan {
   pvec<int> map_l, map_u;                 // factor entry -> slot (-1 for diagonal)
   pvec<int> row_slot;                     // row -> slice*32 + lane (inverse diagonal in slice layout)
   pvec<int> l_span, u_span;               // per row: {first slot, entries} of its L and L^T rows
-  // shared-memory capacities of the TMA-pipelined interior solve
-  int tma_zs = 0, tma_nl = 0, tma_ns = 0, tma_e = 0, tma_s = 0;
-  long long tma_blk_e = 0, tma_blk_s = 0;   // largest per-block totals over all stages
+  int blk_rows_max = 0;                   // rows of the largest interior block
   // level chunks (record, first row, rows) of at most kChunk rows: level L of
   // every block = chunks [ch_all_ptr[L], ch_all_ptr[L+1]); level L of C_a alone
   // = [ch_c_ptr[L], ch_c_ptr[L+1])
