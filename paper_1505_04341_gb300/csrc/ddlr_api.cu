@@ -1438,7 +1438,7 @@ void deep_plan(ddlr_ctx *c, int which) {
       const int b = which == 0 ? q : P.p, l0 = P.blk_lvl0[b], NL = P.blk_lvl0[b + 1] - l0;
       stage_of[q].assign(NL, -1);
       for (int l = 0; l < NL; l++) {
-        const int r0 = P.lvl_row0[l0 + l], r1 = r0 + P.lvl_nrows[l0 + l], s0 = int(sl.size());
+        const int r0 = P.lvl_row0[l0 + l], r1 = r0 + P.lvl_nrows[l0 + l], s0 = int(sl.size()), z0 = nrow;
         int r = which == 1 && sorted ? next_row[l] : r0;
         while (r < r1) {
           if (which == 1 && owner[r - P.m] != q) {
@@ -1469,7 +1469,9 @@ void deep_plan(ddlr_ctx *c, int which) {
         stage_of[q][l] = int(stage.size()) - pt.stage0;
         DeepStage st{};
         st.a = s0 - pt.slice0;
-        st.b = int(sl.size()) - pt.slice0;
+        st.rows = nrow - z0;
+        st.z0 = z0;
+        bad |= int(sl.size()) - s0 != (st.rows + kSlice - 1) / kSlice;   // a run that is not one piece
         stage.push_back(st);
       }
       pt.nslice = int(sl.size()) - pt.slice0;
@@ -1480,7 +1482,8 @@ void deep_plan(ddlr_ctx *c, int which) {
       rows_of.push_back(nrow);
       scap = std::max(scap, pt.nslice);
       tcap = std::max(tcap, pt.nstage);
-      if (ol / 128 > 0x7fffffffLL || ou / 128 > 0x7fffffffLL) { bad = true; break; }
+      bad |= ol / 128 > 0x7fffffffLL || ou / 128 > 0x7fffffffLL;
+      if (bad) break;
     }
     if (bad) return;
     for (int q = 0; q < np; q++) {
@@ -1488,18 +1491,20 @@ void deep_plan(ddlr_ctx *c, int which) {
       long long lin = 0;
       for (int j = 0; j < pt.nstage; j++) {
         DeepStage &sg = stage[pt.stage0 + j];
-        const int4 ea = sl[pt.slice0 + sg.a], eb = sl[pt.slice0 + sg.b - 1];
+        const int4 ea = sl[pt.slice0 + sg.a], eb = sl[pt.slice0 + sg.a + (sg.rows - 1) / kSlice];
         const bool f = j < pt.nfwd;
         sg.src = f ? ea.x : ea.z;
-        sg.bytes = (f ? eb.x : eb.z) - sg.src + int(deep_slice_bytes<T>(deep_w(eb, f ? 0 : 1)) / 128);
+        const int bytes = (f ? eb.x : eb.z) - sg.src + int(deep_slice_bytes<T>(deep_w(eb, f ? 0 : 1)) / 128);
+        if (bytes > 0xffff) return;
+        sg.bytes = (unsigned short)bytes;
         stage_max = std::max(stage_max, (long long)sg.bytes * 128);
         lin += sg.bytes;
       }
       total_max = std::max(total_max, lin * 128);
     }
     DeepGeo g{};
-    // wide levels of blocks that have an SM each: twice the warps (kDeepWideRows)
-    const bool wide = which == 0 && P.p <= sms && P.m >= (long long)kDeepWideRows * P.blk_lvl0[P.p];
+    // wide levels and an SM for each part: twice the warps (kDeepWideRows)
+    const bool wide = which == 1 || (P.p <= sms && P.m >= (long long)kDeepWideRows * P.blk_lvl0[P.p]);
     g.sw = wide ? kDeepWideWarps : kDeepSetWarps;
     g.ctas = C; g.nparts = np; g.scap = scap; g.tcap = tcap;
     const long long all = total_max + stage_max;
@@ -1531,7 +1536,7 @@ void deep_plan(ddlr_ctx *c, int which) {
           const auto &span = dir ? P.u_span : P.l_span;
           const auto &col = dir ? P.u_col : P.l_col;
           DeepStage &sg = stage[pt.stage0 + js];
-          for (int i = sg.a; i < sg.b; i++)
+          for (int i = sg.a; i < sg.a + (sg.rows + kSlice - 1) / kSlice; i++)
             for (int t = 0; t < srow[pt.slice0 + i].y; t++) {
               const int r = srow[pt.slice0 + i].x + t;
               for (int kk = 0; kk < span[2 * size_t(r) + 1]; kk++) {
@@ -1596,7 +1601,7 @@ void deep_plan(ddlr_ctx *c, int which) {
       for (int j = 0; j < pt.nstage; j++) {
         DeepStage &sg = stage[pt.stage0 + j];
         if (pos + sg.bytes > R) { lin += R - pos; pos = 0; }
-        sg.pos = pos;
+        sg.pos = (unsigned short)pos;
         sg.lin = lin;
         pos += sg.bytes;
         lin += sg.bytes;

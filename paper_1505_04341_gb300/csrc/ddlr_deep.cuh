@@ -26,12 +26,13 @@
 
 namespace ddlr {
 
-// Warps of one set, and of one for wide levels: blocks that have an SM each and
-// kDeepWideRows rows a level on average.  Below that line the two are alike (a solve,
-// FP64, edges of 11 and 13: 41.6 and 42.2 us, 47.6 and 46.2), above it a level takes a
-// warp several slices (15: 60.4 and 52.5, 23: 121 and 96, 28: 219 and 177; FP32, 35:
-// 285 and 219).  Two blocks to an SM fill it with the narrow sets (FP32, 112 x 112 x
-// 96 in 294 boxes: 82 and 100).
+// Warps of one set, and of one for wide levels: C_a, and blocks that have an SM each
+// and kDeepWideRows rows a level on average.  Below that line the two are alike (a
+// solve, FP64, edges of 11 and 13: 41.6 and 42.2 us, 47.6 and 46.2), above it a level
+// takes a warp several slices (15: 60.4 and 52.5, 23: 121 and 96, 28: 219 and 177;
+// FP32, 35: 285 and 219; C_a, FP64, 64^3 on 8 CTAs 201 and 199, 48^3 in 27 boxes on 2
+// 171 and 131).  Two blocks to an SM fill it with the narrow sets (FP32, 112 x 112 x 96
+// in 294 boxes: 82 and 100).
 constexpr int kDeepSetWarps = 4, kDeepWideWarps = 8, kDeepWideRows = 80;
 __host__ __device__ constexpr int deep_threads(int sw) { return (2 * sw + 1) * 32; }   // two sets and the copy / push warp
 constexpr int kDeepMaxCtas = 16;
@@ -46,9 +47,11 @@ struct DeepPart {
   int nhalo;               // values received from other parts
 };
 struct DeepStage {
-  int src, bytes, pos, lin;// packed data (from the L or L^T pack): start, size, place in the ring,
-                           // running total before it with the gaps at the ring's end; all / 128
-  int a, b;                // its slices, counted from the part's first
+  int src;                 // packed data (from the L or L^T pack): start,
+  unsigned short bytes, pos;// size, place in the ring,
+  int lin;                 // running total before it with the gaps at the ring's end; all / 128
+  int a;                   // its first slice, counted from the part's first
+  int rows, z0;            // its rows, the first one's position in the part's shared memory
   int halo;                // values received whose first use is here
   int push;                // its first entry in the push list; the next stage's starts where it ends
 };
@@ -283,34 +286,39 @@ k_deep_solve(DeepGeo g, const unsigned char *pk_l, const unsigned char *pk_u, co
     int4 pe = make_int4(0, 0, 0, 0);                       // this lane's first push of the next stage
     if (nst > 0 && st[0].push + ln < st[1].push) pe = g.push[st[0].push + ln];
     bool late = false;
-    for (int j = 0; j < nst; j++) {
-      const int p0 = st[j].push + ln, p1 = st[j + 1].push;
-      // the sets run ahead of this warp by fewer than kDeepBars levels: it
-      // brings in level j + kDeepBars only after level j
-      uint64_t *dj = done + (j % kDeepBars);
-      const unsigned par = unsigned(j / kDeepBars) & 1u;
-      if (!late && !mbar_try_wait(dj, par)) {
-        const unsigned long long t0 = gtimer_ns();
-        while (!mbar_try_wait(dj, par)) {
-          if (is_late()) break;
-          if (gtimer_ns() - t0 > limit_ns) { give_up(); break; }
+    // two loops, the second only for give_up_at: a test for it in the loop took 7 % of
+    // a solve with narrow levels
+    const int jt = give_up_at >= 0 && blockIdx.x == gridDim.x - 1 ? min(nst, give_up_at + 1) : nst;
+    for (int j = 0, seg = 0; seg < 2; seg++) {
+      if (seg == 1 && j < nst) give_up();
+      for (const int je = seg == 0 ? jt : nst; j < je; j++) {
+        const int p0 = st[j].push + ln, p1 = st[j + 1].push;
+        // the sets run ahead of this warp by fewer than kDeepBars levels: it
+        // brings in level j + kDeepBars only after level j
+        uint64_t *dj = done + (j % kDeepBars);
+        const unsigned par = unsigned(j / kDeepBars) & 1u;
+        if (!late && !mbar_try_wait(dj, par)) {
+          const unsigned long long t0 = gtimer_ns();
+          while (!mbar_try_wait(dj, par)) {
+            if (is_late()) break;
+            if (gtimer_ns() - t0 > limit_ns) { give_up(); break; }
+          }
         }
+        late = __any_sync(0xffffffffu, is_late());
+        for (int p = p0; p < p1; p += 32) {
+          if (p != p0) pe = g.push[p];
+          st_async(cluster_map(zb + unsigned(pe.z) * unsigned(sizeof(T)), pe.y), zs[pe.x],
+                   cluster_map(hb + unsigned(pe.w) * 8u, pe.y));
+        }
+        if (j + 1 < nst && p1 + ln < st[j + 2].push) pe = g.push[p1 + ln];
+        if (ln == 0 && !late) {
+          // the level is done with its place in the ring: order its reads before
+          // the copies into it
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          produce(j + 1);
+        }
+        __syncwarp();
       }
-      if (j == give_up_at && blockIdx.x == gridDim.x - 1) give_up();
-      late = __any_sync(0xffffffffu, is_late());
-      for (int p = p0; p < p1; p += 32) {
-        if (p != p0) pe = g.push[p];
-        st_async(cluster_map(zb + unsigned(pe.z) * unsigned(sizeof(T)), pe.y), zs[pe.x],
-                 cluster_map(hb + unsigned(pe.w) * 8u, pe.y));
-      }
-      if (j + 1 < nst && p1 + ln < st[j + 2].push) pe = g.push[p1 + ln];
-      if (ln == 0 && !late) {
-        // the level is done with its place in the ring: order its reads before
-        // the copies into it
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        produce(j + 1);
-      }
-      __syncwarp();
     }
     if (ln == 0) {
       // every issued copy has arrived before the CTA may leave (on the normal
@@ -325,7 +333,9 @@ k_deep_solve(DeepGeo g, const unsigned char *pk_l, const unsigned char *pk_u, co
     // ---- set wi / SW: levels of its parity; this warp's slices a + ws, a + ws + SW, ...
     const int set = wi / SW, ws = wi % SW;
     constexpr int U = 4;
-    int a = 0, b = 0, w = 0, hl = 0, zi = 0;               // zi: this lane's row (a spare place past the slice's last)
+    // nr: rows from this warp's slice on; zp: this lane's place, zi: the same, a spare
+    // place past the slice's last row
+    int a = 0, nr = 0, w = 0, hl = 0, zp = 0, zi = 0;
     T acc = T(0), dr = T(0), av[U];
     int ad[U];
     const unsigned char *pe = nullptr;
@@ -345,7 +355,7 @@ k_deep_solve(DeepGeo g, const unsigned char *pk_l, const unsigned char *pk_u, co
     auto open_slice = [&](const DeepStage &s, bool fwd, int i) {
       const int4 e = sl[i];
       w = deep_w(e, fwd ? 0 : 1);
-      zi = ln < (e.y & 63) ? (e.y >> 6) + ln : g.zcap;
+      zi = ln < nr ? zp : g.zcap;
       pe = ring + size_t(s.pos + (fwd ? e.x : e.z) - s.src) * 128;
       dr = reinterpret_cast<const T *>(pe + size_t(w) * 32 * (sizeof(T) + 4))[ln];
       acc = zs[zi];
@@ -361,12 +371,13 @@ k_deep_solve(DeepGeo g, const unsigned char *pk_l, const unsigned char *pk_u, co
     bool ok = true;
     auto prefetch = [&](int j) {
       const DeepStage s = st[j];
-      ok = ok && !is_late();
+      const bool late = is_late();             // (read while the wait is under way)
       a = s.a + ws;
-      b = s.b;
+      nr = s.rows - ws * 32;
+      zp = s.z0 + ws * 32 + ln;
       hl = s.halo;
-      if (a < b) {
-        ok = ok && wait_for(bar + (j % kDeepBars), unsigned(j / kDeepBars) & 1u, false);
+      if (nr > 0) {
+        ok = ok && wait_for(bar + (j % kDeepBars), unsigned(j / kDeepBars) & 1u, false) && !late;
         if (ok) open_slice(s, j < P.nfwd, a);
       }
     };
@@ -374,11 +385,11 @@ k_deep_solve(DeepGeo g, const unsigned char *pk_l, const unsigned char *pk_u, co
     __syncwarp();
     for (int j = set; j < nst; j += 2) {
       if (j > 0) set_sync<SW>(set ^ 1);                        // level j - 1 is done
-      if (hl > 0 && a < b) ok = ok && wait_for(halo + j, 0u, true);
+      if (hl > 0 && nr > 0) ok = ok && wait_for(halo + j, 0u, true);
       // the turn: the top level's forward results were not there to prefetch
       // (every other backward level is at least three levels after its forward)
-      if (j == P.nfwd && a < b) acc = zs[zi];
-      for (int i = a; ok && i < b; i += SW) {
+      if (j == P.nfwd && nr > 0) acc = zs[zi];
+      for (int i = a; ok && nr > 0; i += SW, nr -= SW * 32, zp += SW * 32) {
         if (i != a) open_slice(st[j], j < P.nfwd, i);
         switch (min(w, U + 1)) {
           case 0: break;
